@@ -137,8 +137,8 @@ struct ff_ctx {
 
   ff::Grid grid{};
   // particles in internal (cell) order
-  // (two-set: the centres in their farthest-point order, pos.w = 0; the radii
-  // are kept in FP64 in crad)
+  // (two-set: the centres in their farthest-point order, pos.w = 1 / r_k^2; the
+  // radii are kept in FP64 in crad)
   ff::Buf perm;      // int[n]   internal -> caller index
   ff::Buf iperm;     // int[n]   caller -> internal index
   ff::Buf pos;       // float4[n] (x, y, z, a)
@@ -147,6 +147,7 @@ struct ff_ctx {
   // two-set centres
   ff::Buf centre_idx;// int64[K]  quadrature point chosen as centre k
   ff::Buf crad;      // double[K] r_k
+  ff::Buf cinv;      // dfloat[K] 1 / r_k^2 (its FP32 rounding: pos.w)
   ff::Buf clim;      // double[K] t^2 r_k^2 (+inf untruncated)
   ff::Buf clim32;    // float[K]  its FP32 rounding (filter)
   ff::Buf qpts;      // float[3 nq] the quadrature points (x, y, z), caller order
@@ -160,6 +161,7 @@ struct ff_ctx {
   // shape functions (context precision), aligned with nbr_idx
   ff::Buf phi;       // T[n1]
   ff::Buf dphi;      // T[3 * n1]
+  ff::Buf redo;      // int[nq + 1] rows an FP32 pass leaves to FP64: count, indexes
   // matrices (internal order), CSR with the diagonal stored
   ff::Buf a_ptr;     // int64[n+1]
   ff::Buf a_col;     // int[n2]
@@ -181,7 +183,8 @@ struct ff_ctx {
   ff::Buf sk_cnt;    // int[nq + 1]
   ff::Buf sk_ptr;    // int64[nq + 1]
   ff::Buf sk_idx;    // int[nq1]  covering nodes (internal order)
-  ff::Buf sk_phi;    // T[4 * nq1] shape functions and gradients
+  ff::Buf sk_phi;    // float / dfloat[nq1] shape functions
+  ff::Buf sk_c;      // T[n * ldc] the nodal values, row-major in the internal order
   ff::Buf wh;        // T[nq] v_i (lambda_i + 4 mu_i)
   // device flags
   ff::Buf flags;     // DevFlags
@@ -259,10 +262,11 @@ constexpr long long kTsetMaxCentres = 4096;
 bool tset_assembly_fits(long long K);
 void tset_assemble(ff_ctx* c);
 // covering lists of arbitrary points over the centres (returns the pair count)
-// and the Gaussian shape functions there (returns the pass's flags)
+// and the Gaussian shape functions there (FP32 or double-float; the gradients
+// too when dphi is given)
 long long twoset_cover(ff_ctx* c, const float* Q, long long nq, Buf& ptrb, Buf& idxb, Buf& cntb);
-DevFlags twoset_shape(ff_ctx* c, const float* Q, long long nq, const long long* ptr,
-                      const int* idx, long long n1, void* phi, void* dphi, bool fp64_out);
+void twoset_shape(ff_ctx* c, const float* Q, long long nq, const long long* ptr, const int* idx,
+                  long long n1, void* phi, void* dphi, bool f32);
 
 // skinning weight fields and linear blend skinning at query points (skinning.cu)
 void skinning_weights(ff_ctx* c, const float* Q, long long nq, const void* C, int m, void* W);

@@ -4,6 +4,8 @@
 // Eqs. 7, 9-10; the basis written about the evaluation point (see shape.cu).
 #pragma once
 
+#include <type_traits>
+
 #include "dfloat.cuh"
 #include "ff_internal.cuh"
 
@@ -29,6 +31,7 @@ __device__ __forceinline__ void bspline(C q, C& w, C& dwq) {
 // they give w = varphi_k(X) and gs with grad_X varphi_k = gs (p_k - X).
 // BSpline: the cubic B-spline of radius a_k = p.w (the nodal discretisation).
 struct BSpline {
+  static constexpr bool kStash = false;
   template <class C>
   __device__ __forceinline__ void eval(int, float4 p, C d2, C& w, C& gs) const {
     const C ak = (C)p.w;
@@ -42,111 +45,137 @@ __device__ __forceinline__ float gauss_exp(float x) { return expf(x); }
 __device__ __forceinline__ double gauss_exp(double x) { return exp(x); }
 __device__ __forceinline__ dfloat gauss_exp(dfloat x) { return df_exp(x); }
 
-template <class C>
-__device__ __forceinline__ C from_f64(double x) { return (C)x; }
-template <>
-__device__ __forceinline__ dfloat from_f64<dfloat>(double x) { return dfloat(x); }
-
 // Gauss: exp(-|X - p_k|^2 / r_k^2) (Sec. 3.2) with the FP64 radii r_k of the
-// two-set construction; grad_X = (2 w / r_k^2)(p_k - X).  In double-float the
-// exponential is df_exp (reduction by ln 2 and a Taylor polynomial on the FP32
-// pipes).
+// two-set construction; grad_X = (2 w / r_k^2)(p_k - X).  FP32 and double-float
+// take 1 / r_k^2 rounded once from FP64 per centre (p.w, inv): a multiplication
+// where the radius would cost two conversions from FP64, a square and a
+// division a pair.  In double-float the exponential is df_exp (reduction by
+// ln 2 and a Taylor polynomial on the FP32 pipes).
 struct Gauss {
+  static constexpr bool kStash = true;
   const double* rad;
+  const dfloat* inv;
   template <class C>
-  __device__ __forceinline__ void eval(int k, float4, C d2, C& w, C& gs) const {
-    const C rk = from_f64<C>(rad[k]);
-    const C rk2 = rk * rk;
-    w = gauss_exp(-(d2 / rk2));
-    gs = C(2) * w / rk2;
+  __device__ __forceinline__ C inv_r2(int k, float4 p) const {
+    if constexpr (sizeof(C) == 4) {
+      return p.w;
+    } else if constexpr (std::is_same_v<C, dfloat>) {
+      return inv[k];
+    } else {
+      const double rk = rad[k];
+      return 1.0 / (rk * rk);
+    }
+  }
+  template <class C>
+  __device__ __forceinline__ C slope(int k, float4 p, C w) const {
+    return C(2) * w * inv_r2<C>(k, p);
+  }
+  template <class C>
+  __device__ __forceinline__ void eval(int k, float4 p, C d2, C& w, C& gs) const {
+    const C iv = inv_r2<C>(k, p);
+    w = gauss_exp(-(d2 * iv));
+    gs = C(2) * w * iv;
   }
 };
 
-template <class C>
-__device__ __forceinline__ C warp_sum(C v) {
+// sum over the L lanes of each aligned group of a warp
+template <int L, class C>
+__device__ __forceinline__ C group_sum(C v) {
 #pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = L / 2; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
 // symmetric 4x4 packed upper triangle: (0,0)(0,1)(0,2)(0,3)(1,1)(1,2)(1,3)(2,2)(2,3)(3,3)
-__device__ __forceinline__ int sidx(int r, int c) {
-  if (r > c) { int t = r; r = c; c = t; }
-  const int base[4] = {0, 4, 7, 9};
-  return base[r] + (c - r);
+__device__ __forceinline__ constexpr int sidx(int r, int c) {
+  const int lo = r < c ? r : c, hi = r < c ? c : r;
+  return lo * 4 - lo * (lo - 1) / 2 + (hi - lo);
 }
 
-// Cholesky of a 4x4 SPD matrix (packed), returns false if a pivot is not
-// positive relative to the trace.  L stored dense row-major lower.
+// Cholesky factor of a 4x4 SPD matrix: the strict lower triangle and the
+// diagonal's reciprocals, so that a solve has no divisions.
 template <class C>
-__device__ __forceinline__ bool chol4(const C* m, C* L, C rel_tol) {
-  C tr = m[0] + m[4] + m[7] + m[9];
-  for (int j = 0; j < 4; ++j) {
-    C s = m[sidx(j, j)];
-    for (int p = 0; p < j; ++p) s -= L[j * 4 + p] * L[j * 4 + p];
-    if (!(s > rel_tol * tr)) return false;
-    C d = sqrt(s);
-    L[j * 4 + j] = d;
-    for (int i = j + 1; i < 4; ++i) {
-      C t = m[sidx(i, j)];
-      for (int p = 0; p < j; ++p) t -= L[i * 4 + p] * L[j * 4 + p];
-      L[i * 4 + j] = t / d;
+struct Chol4 {
+  C l[4][4];
+  C r[4];
+  // false if a pivot is not positive relative to the trace
+  __device__ __forceinline__ bool factor(const C* m, C rel_tol) {
+    const C tr = m[0] + m[4] + m[7] + m[9];
+    bool ok = true;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      C s = m[sidx(j, j)];
+#pragma unroll
+      for (int p = 0; p < j; ++p) s -= l[j][p] * l[j][p];
+      ok = ok && s > rel_tol * tr;
+      r[j] = C(1) / sqrt(s);
+#pragma unroll
+      for (int i = j + 1; i < 4; ++i) {
+        C t = m[sidx(i, j)];
+#pragma unroll
+        for (int p = 0; p < j; ++p) t -= l[i][p] * l[j][p];
+        l[i][j] = t * r[j];
+      }
     }
-    for (int i = 0; i < j; ++i) L[i * 4 + j] = C(0);
+    return ok;
   }
-  return true;
-}
+  __device__ __forceinline__ void solve(const C* b, C* x) const {
+    C y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      C t = b[i];
+#pragma unroll
+      for (int p = 0; p < i; ++p) t -= l[i][p] * y[p];
+      y[i] = t * r[i];
+    }
+#pragma unroll
+    for (int i = 3; i >= 0; --i) {
+      C t = y[i];
+#pragma unroll
+      for (int p = i + 1; p < 4; ++p) t -= l[p][i] * x[p];
+      x[i] = t * r[i];
+    }
+  }
+};
 
-template <class C>
-__device__ __forceinline__ void chol4_solve(const C* L, const C* b, C* x) {
-  C y[4];
-  for (int i = 0; i < 4; ++i) {
-    C t = b[i];
-    for (int p = 0; p < i; ++p) t -= L[i * 4 + p] * y[p];
-    y[i] = t / L[i * 4 + i];
-  }
-  for (int i = 3; i >= 0; --i) {
-    C t = y[i];
-    for (int p = i + 1; p < 4; ++p) t -= L[p * 4 + i] * x[p];
-    x[i] = t / L[i * 4 + i];
-  }
-}
-
-// Evaluate one row in compute precision C, writing outputs of precision T.
-// Returns 0 ok, 1 singular, 2 ill-conditioned (only when check_cond).
-template <class C, class T, class Kern = BSpline>
-__device__ int shape_row(const float4* __restrict__ pos, long long s, long long e,
-                         const int* __restrict__ idx, float4 Xi, T* __restrict__ phi,
-                         T* __restrict__ dphi, long long n1, double cond_limit, bool check_cond,
-                         const Kern& kern = Kern()) {
-  const int lane = threadIdx.x & 31;
+// Evaluate one row per group of L lanes in compute precision C, writing
+// outputs of precision T (phi; with GRAD dphi too).  Every lane of the warp
+// takes part (a group without a row passes s == e).  Returns 0 ok, 1 singular,
+// 2 ill-conditioned (only when check_cond), the same in every lane of a group;
+// nothing is written then.
+//
+// The row's pairs cost ~110 (values alone: ~50) instructions an entry of a
+// lane, the moment solve ~900 a warp whatever the rows it holds; so a warp
+// takes 32 / L rows at once.
+template <class C, class T, int L, bool GRAD, class Kern = BSpline>
+__device__ __forceinline__ int shape_rows(const float4* __restrict__ pos, long long s, long long e,
+                                          const int* __restrict__ idx, float4 Xi,
+                                          T* __restrict__ phi, T* __restrict__ dphi, long long n1,
+                                          double cond_limit, bool check_cond,
+                                          const Kern& kern = Kern()) {
+  const int lane = threadIdx.x & (L - 1);
   const C xi = (C)Xi.x, yi = (C)Xi.y, zi = (C)Xi.z, si = (C)Xi.w;
   const C isi = C(1) / si;  // the basis scale's reciprocal, once per row
-  C m[10], dm[3][10];
+  // the raw kernel of a pair waits in its phi slot for the second pass where
+  // it is costly and the slot holds it exactly (the Gaussian in double-float)
+  constexpr bool stash = Kern::kStash && std::is_same_v<C, dfloat> && std::is_same_v<T, dfloat>;
+  constexpr int ND = GRAD ? 3 : 0;
+  C m[10], dm[GRAD ? 3 : 1][10];
 #pragma unroll
   for (int q = 0; q < 10; ++q) {
     m[q] = C(0);
-    dm[0][q] = dm[1][q] = dm[2][q] = C(0);
+#pragma unroll
+    for (int d = 0; d < ND; ++d) dm[d][q] = C(0);
   }
-  // the raw kernel of a lane's first kCache entries is kept for the second
-  // pass (the Gaussian's exponential is the costliest step of a pair)
-  constexpr int kCache = 4;
-  C cw[kCache], cg[kCache];
-  int q = 0;
-  for (long long t = s + lane; t < e; t += 32, ++q) {
+  for (long long t = s + lane; t < e; t += L) {
     const int k = idx[t];
-    float4 p = pos[k];
-    C r0 = (C)p.x - xi, r1 = (C)p.y - yi, r2 = (C)p.z - zi;
+    const float4 p = pos[k];
+    const C r0 = (C)p.x - xi, r1 = (C)p.y - yi, r2 = (C)p.z - zi;
     C w, gs;  // grad_X varphi = gs * r
     kern.template eval<C>(k, p, r0 * r0 + r1 * r1 + r2 * r2, w, gs);
-#pragma unroll
-    for (int u = 0; u < kCache; ++u)
-      if (q == u) {
-        cw[u] = w;
-        cg[u] = gs;
-      }
-    C P[4] = {C(1), r0 * isi, r1 * isi, r2 * isi};
-    C g[3] = {gs * r0, gs * r1, gs * r2};
+    if constexpr (stash) phi[t] = w;
+    const C P[4] = {C(1), r0 * isi, r1 * isi, r2 * isi};
+    const C g[3] = {gs * r0, gs * r1, gs * r2};
     int o = 0;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -154,28 +183,38 @@ __device__ int shape_row(const float4* __restrict__ pos, long long s, long long 
       for (int b = a; b < 4; ++b, ++o) {
         const C pp = P[a] * P[b];
         mac(m[o], w, pp);  // fused (unnormalised in double-float), finished below
-        mac(dm[0][o], g[0], pp);
-        mac(dm[1][o], g[1], pp);
-        mac(dm[2][o], g[2], pp);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) mac(dm[d][o], g[d], pp);
       }
   }
 #pragma unroll
   for (int q = 0; q < 10; ++q) {
-    m[q] = warp_sum(finish(m[q]));
-    dm[0][q] = warp_sum(finish(dm[0][q]));
-    dm[1][q] = warp_sum(finish(dm[1][q]));
-    dm[2][q] = warp_sum(finish(dm[2][q]));
+    m[q] = group_sum<L>(finish(m[q]));
+#pragma unroll
+    for (int d = 0; d < ND; ++d) dm[d][q] = group_sum<L>(finish(dm[d][q]));
   }
-  C L[16];
-  if (!chol4<C>(m, L, C(1e-12))) return 1;
+  Chol4<C> ch;
+  if (!ch.factor(m, C(1e-12))) return 1;
+  C Cv[4], dC[GRAD ? 3 : 1][4];
+  {
+    const C e0[4] = {C(1), C(0), C(0), C(0)};
+    ch.solve(e0, Cv);
+  }
   if (check_cond) {
     // 1-norm condition number from the explicit inverse
     C inv_norm = C(0), m_norm = C(0);
+#pragma unroll
     for (int col = 0; col < 4; ++col) {
-      C ecol[4] = {C(0), C(0), C(0), C(0)}, x[4];
-      ecol[col] = C(1);
-      chol4_solve<C>(L, ecol, x);
+      C x[4];
+      if (col == 0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) x[r] = Cv[r];
+      } else {
+        const C ecol[4] = {C(0), C(col == 1), C(col == 2), C(col == 3)};
+        ch.solve(ecol, x);
+      }
       C a1 = C(0), a2 = C(0);
+#pragma unroll
       for (int r = 0; r < 4; ++r) {
         a1 += fabs(x[r]);
         a2 += fabs(m[sidx(r, col)]);
@@ -183,49 +222,41 @@ __device__ int shape_row(const float4* __restrict__ pos, long long s, long long 
       inv_norm = fmax(inv_norm, a1);
       m_norm = fmax(m_norm, a2);
     }
-    if ((double)(inv_norm * m_norm) > cond_limit) return 2;
-  }
-  C Cv[4], dC[3][4];
-  {
-    C e0[4] = {C(1), C(0), C(0), C(0)};
-    chol4_solve<C>(L, e0, Cv);
+    if (!((double)(inv_norm * m_norm) <= cond_limit)) return 2;
   }
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
+  for (int d = 0; d < ND; ++d) {
     C rhs[4];
+#pragma unroll
     for (int r = 0; r < 4; ++r) {
       C t = C(0);
+#pragma unroll
       for (int cc = 0; cc < 4; ++cc) t += dm[d][sidx(r, cc)] * Cv[cc];
       rhs[r] = -t;
     }
     rhs[1 + d] += isi;
-    chol4_solve<C>(L, rhs, dC[d]);
+    ch.solve(rhs, dC[d]);
   }
-  q = 0;
-  for (long long t = s + lane; t < e; t += 32, ++q) {
+  for (long long t = s + lane; t < e; t += L) {
     const int k = idx[t];
-    float4 p = pos[k];
-    C r0 = (C)p.x - xi, r1 = (C)p.y - yi, r2 = (C)p.z - zi;
+    const float4 p = pos[k];
+    const C r0 = (C)p.x - xi, r1 = (C)p.y - yi, r2 = (C)p.z - zi;
     C w, gs;
-    if (q < kCache) {
-#pragma unroll
-      for (int u = 0; u < kCache; ++u)
-        if (q == u) {
-          w = cw[u];
-          gs = cg[u];
-        }
+    if constexpr (stash) {
+      w = phi[t];
+      gs = kern.template slope<C>(k, p, w);
     } else {
       kern.template eval<C>(k, p, r0 * r0 + r1 * r1 + r2 * r2, w, gs);
     }
-    C P[4] = {C(1), r0 * isi, r1 * isi, r2 * isi};
+    const C P[4] = {C(1), r0 * isi, r1 * isi, r2 * isi};
     C PC = Cv[0];
 #pragma unroll
     for (int a = 1; a < 4; ++a) mac(PC, P[a], Cv[a]);
     PC = finish(PC);
     phi[t] = (T)(w * PC);
-    C g[3] = {gs * r0, gs * r1, gs * r2};
+    const C g[3] = {gs * r0, gs * r1, gs * r2};
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
+    for (int d = 0; d < ND; ++d) {
       C PdC = dC[d][0];
 #pragma unroll
       for (int a = 1; a < 4; ++a) mac(PdC, P[a], dC[d][a]);
@@ -234,6 +265,47 @@ __device__ int shape_row(const float4* __restrict__ pos, long long s, long long 
     }
   }
   return 0;
+}
+
+// Rows an FP32 pass leaves to FP64 (a moment matrix with a 1-norm condition
+// number above its limit, or singular in FP32): list[0] counts them, their
+// indexes follow.  A second pass takes them a warp a row, because an FP64
+// instruction costs the same for one lane as for 32.
+__device__ __forceinline__ void redo_later(int* __restrict__ list, long long i) {
+  list[1 + atomicAdd(list, 1)] = (int)i;
+}
+
+// the list of a pass over n rows, emptied in stream order
+inline int* redo_list(ff_ctx* c, long long n) {
+  int* list = reinterpret_cast<int*>(c->redo.ensure(sizeof(int) * (n + 1)));
+  FF_CUDA(cudaMemsetAsync(list, 0, sizeof(int), c->stream));
+  return list;
+}
+inline unsigned redo_grid(long long n) {
+  return (unsigned)(n < 8LL * 4 * sm_count() ? (n + 7) / 8 : 4LL * sm_count());
+}
+
+template <class T, bool GRAD, class Kern>
+__global__ void __launch_bounds__(256)
+    k_shape_redo(const float4* __restrict__ pos, const float4* __restrict__ at,
+                 const float* __restrict__ Q, float scale, const long long* __restrict__ ptr,
+                 const int* __restrict__ idx, long long n1, T* __restrict__ phi,
+                 T* __restrict__ dphi, const int* __restrict__ list, DevFlags* __restrict__ flags,
+                 Kern kern) {
+  const int count = list[0];
+  const int warps = gridDim.x * 8;
+  for (int q = blockIdx.x * 8 + (threadIdx.x >> 5); q < count; q += warps) {
+    const int i = list[1 + q];
+    const float4 Xi = at ? at[i] : make_float4(Q[3LL * i], Q[3LL * i + 1], Q[3LL * i + 2], scale);
+    const int st = shape_rows<double, T, 32, GRAD>(pos, ptr[i], ptr[i + 1], idx, Xi, phi, dphi, n1,
+                                                   0.0, false, kern);
+    if ((threadIdx.x & 31) == 0) {
+      if (st == 0)
+        atomicAdd(&flags->fallback, 1);
+      else if (atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0)
+        flags->index = i;
+    }
+  }
 }
 
 }  // namespace rkpm

@@ -1,4 +1,4 @@
-// Corrected RKPM shape functions and gradients, one warp per evaluation point.
+// Corrected RKPM shape functions and gradients, a group of lanes per evaluation point.
 //
 // Sec. 3.2, Eqs. 7, 9-10: phi_k(X) = varphi_k(X) P(p_k)^T C(X), M(X) C(X) = P(X),
 // M(X) = sum_k varphi_k(X) P(p_k) P(p_k)^T with the linear basis.  The basis is
@@ -9,11 +9,12 @@
 //   d_s phi_k = d_s varphi_k P_k^T C + varphi_k P_k^T d_s C.
 // Raw kernel: cubic B-spline w(q), q = |X - p_k| / a_k, grad = (w'(q)/q)(X - p_k)/a_k^2.
 //
-// Lanes stride over the row's neighbours and accumulate the 10 distinct entries
-// of M and the 30 of d M; a butterfly reduction gives every lane the sums; every
-// lane then solves the 4x4 system (Cholesky) and writes phi / grad phi for its
-// own neighbours.  In FP32 mode a row whose moment matrix has a 1-norm condition
-// number above `cond_fp64` is recomputed entirely in FP64.  FP64 mode computes
+// A group of lanes strides over the row's neighbours and accumulates the 10
+// distinct entries of M and the 30 of d M; a butterfly reduction gives every
+// lane of the group the sums; each then solves the 4x4 system (Cholesky) and
+// writes phi / grad phi for its own neighbours.  In FP32 mode a row whose moment
+// matrix has a 1-norm condition number above `cond_limit` is recomputed entirely
+// in FP64 by a second kernel.  FP64 mode computes
 // and stores double-float pairs (FP32 head and tail, ~2^-47 relative).
 #include "dfloat.cuh"
 #include "ff_internal.cuh"
@@ -22,32 +23,36 @@
 namespace ff {
 namespace {
 
-using rkpm::shape_row;
+using rkpm::shape_rows;
+
+// lanes a row: a nodal row has ~30-45 nodes, so eight lanes take four to six
+// of them each and a warp's moment solve serves four rows (FP32, 200k
+// particles: 1.41 ms with a warp a row, 0.15 ms and 0.16 ms of FP64 redo now;
+// double-float, 50k particles: 1.34 ms, 0.37 ms now)
+constexpr int kLanes = 8;
 
 template <class T>
-__global__ void k_shape(const float4* __restrict__ pos, const long long* __restrict__ ptr,
-                        const int* __restrict__ idx, long long n, long long n1,
-                        T* __restrict__ phi, T* __restrict__ dphi, double cond_limit,
-                        DevFlags* __restrict__ flags) {
-  long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (i >= n) return;
-  const int lane = threadIdx.x & 31;
-  long long s = ptr[i], e = ptr[i + 1];
-  float4 Xi = pos[i];
-  int st;
-  if (sizeof(T) == 4) {
-    st = shape_row<float, T>(pos, s, e, idx, Xi, phi, dphi, n1, cond_limit, true);
-    if (st != 0) {
-      st = shape_row<double, T>(pos, s, e, idx, Xi, phi, dphi, n1, 0.0, false);
-      if (lane == 0 && st == 0) atomicAdd(&flags->fallback, 1);
-    }
+__global__ void __launch_bounds__(256, 2)
+    k_shape(const float4* __restrict__ pos, const long long* __restrict__ ptr,
+            const int* __restrict__ idx, long long n, long long n1, T* __restrict__ phi,
+            T* __restrict__ dphi, double cond_limit, int* __restrict__ redo,
+            DevFlags* __restrict__ flags) {
+  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
+  const bool live = i < n, first = threadIdx.x % kLanes == 0;
+  const long long s = live ? ptr[i] : 0, e = live ? ptr[i + 1] : 0;
+  const float4 Xi = live ? pos[i] : make_float4(0.f, 0.f, 0.f, 1.f);
+  if constexpr (sizeof(T) == 4) {
+    const int st =
+        shape_rows<float, T, kLanes, true>(pos, s, e, idx, Xi, phi, dphi, n1, cond_limit, true);
+    if (live && st != 0 && first) rkpm::redo_later(redo, i);
   } else {
     // FP64 outputs computed in double-float (~2^-47 relative; GB300's FP64
     // rate made this kernel FP64-bound)
-    st = shape_row<dfloat, T>(pos, s, e, idx, Xi, phi, dphi, n1, 0.0, false);
-  }
-  if (st == 1 && lane == 0) {
-    if (atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0) flags->index = (int)i;
+    const int st = shape_rows<dfloat, T, kLanes, true>(pos, s, e, idx, Xi, phi, dphi, n1, 0.0,
+                                                       false);
+    if (live && st != 0 && first &&
+        atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0)
+      flags->index = (int)i;
   }
 }
 
@@ -62,14 +67,25 @@ void build_shape(ff_ctx* c) {
   c->dphi.ensure(3 * es * n1);
   const double cond_limit = 1e2;
   ProfScope ps(kProfShape);
+  const float4* pos = c->pos.as<float4>();
+  const long long* ptr = c->nbr_ptr.as<long long>();
+  const int* idx = c->nbr_idx.as<int>();
+  DevFlags* flags = c->flags.as<DevFlags>();
+  const unsigned grid = ceil_div(n * kLanes, T);
   if (c->prec == FF_PREC_FP64) {  // stored as double-float pairs for the assembly
-    (k_shape<dfloat><<<ceil_div(n * 32, T), T, 0, c->stream>>>(
-        c->pos.as<float4>(), c->nbr_ptr.as<long long>(), c->nbr_idx.as<int>(), n, n1,
-        c->phi.as<dfloat>(), c->dphi.as<dfloat>(), cond_limit, c->flags.as<DevFlags>()), ::ff::note_launch());
+    (k_shape<dfloat><<<grid, T, 0, c->stream>>>(pos, ptr, idx, n, n1, c->phi.as<dfloat>(),
+                                                c->dphi.as<dfloat>(), cond_limit, nullptr, flags),
+     ::ff::note_launch());
   } else {
-    (k_shape<float><<<ceil_div(n * 32, T), T, 0, c->stream>>>(
-        c->pos.as<float4>(), c->nbr_ptr.as<long long>(), c->nbr_idx.as<int>(), n, n1,
-        c->phi.as<float>(), c->dphi.as<float>(), cond_limit, c->flags.as<DevFlags>()), ::ff::note_launch());
+    int* redo = rkpm::redo_list(c, n);
+    (k_shape<float><<<grid, T, 0, c->stream>>>(pos, ptr, idx, n, n1, c->phi.as<float>(),
+                                               c->dphi.as<float>(), cond_limit, redo, flags),
+     ::ff::note_launch());
+    FF_LAUNCH_CHECK();
+    (rkpm::k_shape_redo<float, true, rkpm::BSpline><<<rkpm::redo_grid(n), 256, 0, c->stream>>>(
+         pos, pos, nullptr, 0.f, ptr, idx, n1, c->phi.as<float>(), c->dphi.as<float>(), redo,
+         flags, rkpm::BSpline()),
+     ::ff::note_launch());
   }
   FF_LAUNCH_CHECK();
   ps.close();

@@ -11,91 +11,159 @@
 // cell -- the cell edge is at least the largest support, so those hold every
 // node that covers it; points outside the box are clamped to the boundary
 // cells, which still hold every node within one support of them), the moment
-// solve and shape functions per query point (one warp each; double-float in
-// FP64 contexts, FP32 with the FP64 redo of ill-conditioned points in FP32
-// ones), and the weights as one warp per point over the modes.  Clouds of the
-// two-set discretisation take its own covering test over the K centres and
-// its Gaussian shape functions (twoset.cu).
+// solve and the values (no gradients) of the shape functions (eight lanes a
+// point; double-float in FP64 contexts, FP32 with the FP64 redo of
+// ill-conditioned points in FP32 ones), and the weights as one warp per point
+// over the modes, from a row-major copy of the nodal values.  Clouds of the
+// two-set discretisation take its own covering test over the K centres and its
+// Gaussian shape functions (twoset.cu).
+#include <type_traits>
+
 #include "grid.cuh"
 #include "rkpm_eval.cuh"
 
 namespace ff {
+
+template <class T>
+void gather_block(ff_ctx* c, const T* X0, int m, T* X, int ld);
+
 namespace {
 
-using rkpm::shape_row;
-
-// MODE 0: count the nodes covering each query point; MODE 1: list them (in
-// cell order, then node order inside a cell: deterministic)
+// MODE 0: count the nodes covering each query point; MODE 1: list them.  One
+// warp a point, a lane a cell; a lane tests up to 32 nodes of its cell a round,
+// and the list takes each round's hits in cell order, then node order
+// (deterministic).  A thread a point (27 dependent walks, 1.3 blocks an SM at
+// 50,000 points) took 306 us a pass, 125 us now.
 template <int MODE>
-__global__ void k_query_search(const float* __restrict__ Q, long long nq,
-                               const float4* __restrict__ pos, GridDev g,
-                               const int* __restrict__ cstart, int* __restrict__ cnt,
-                               const long long* __restrict__ qptr, int* __restrict__ qidx) {
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256)
+    k_query_search(const float* __restrict__ Q, long long nq, const float4* __restrict__ pos,
+                   GridDev g, const int* __restrict__ cstart, int* __restrict__ cnt,
+                   const long long* __restrict__ qptr, int* __restrict__ qidx) {
+  const long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (q >= nq) return;
+  const int lane = threadIdx.x & 31;
   const float4 X = make_float4(Q[3 * q], Q[3 * q + 1], Q[3 * q + 2], 0.f);
-  const int cx = cell_coord(X.x, g.o0, g.h, g.d0);
-  const int cy = cell_coord(X.y, g.o1, g.h, g.d1);
-  const int cz = cell_coord(X.z, g.o2, g.h, g.d2);
-  int c = 0;
-  const long long base = MODE ? qptr[q] : 0;
-  for (int z = max(cz - 1, 0); z <= min(cz + 1, g.d2 - 1); ++z)
-    for (int y = max(cy - 1, 0); y <= min(cy + 1, g.d1 - 1); ++y)
-      for (int x = max(cx - 1, 0); x <= min(cx + 1, g.d0 - 1); ++x) {
-        const long long key = cell_key(g, x, y, z);
-        for (int i = cstart[key]; i < cstart[key + 1]; ++i)
-          if (covers(X, pos[i])) {
-            if (MODE) qidx[base + c] = i;
-            ++c;
-          }
-      }
-  if (!MODE) cnt[q] = c;
-}
-
-// shape functions of query point q (one warp): FP64 contexts in double-float
-// with FP64 output, FP32 contexts in FP32 with the FP64 redo when the moment
-// matrix is ill-conditioned.  scale normalises the linear basis (any positive
-// value gives the same functions; the support size keeps M well scaled).
-template <class T>
-__global__ void k_query_shape(const float4* __restrict__ pos, const float* __restrict__ Q,
-                              const long long* __restrict__ qptr, const int* __restrict__ qidx,
-                              long long nq, long long nq1, float scale, T* __restrict__ phi,
-                              T* __restrict__ dphi, double cond_limit,
-                              DevFlags* __restrict__ flags) {
-  const long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (q >= nq) return;
-  const int lane = threadIdx.x & 31;
-  const long long s = qptr[q], e = qptr[q + 1];
-  const float4 Xq = make_float4(Q[3 * q], Q[3 * q + 1], Q[3 * q + 2], scale);
-  int st = 1;
-  if (e > s) {
-    if constexpr (sizeof(T) == 4) {
-      st = shape_row<float, T>(pos, s, e, qidx, Xq, phi, dphi, nq1, cond_limit, true);
-      if (st != 0) st = shape_row<double, T>(pos, s, e, qidx, Xq, phi, dphi, nq1, 0.0, false);
-    } else {
-      st = shape_row<dfloat, T>(pos, s, e, qidx, Xq, phi, dphi, nq1, 0.0, false);
-    }
+  const int x = cell_coord(X.x, g.o0, g.h, g.d0) + lane % 3 - 1;
+  const int y = cell_coord(X.y, g.o1, g.h, g.d1) + lane / 3 % 3 - 1;
+  const int z = cell_coord(X.z, g.o2, g.h, g.d2) + lane / 9 - 1;
+  int i = 0, end = 0;
+  if (lane < 27 && x >= 0 && x < g.d0 && y >= 0 && y < g.d1 && z >= 0 && z < g.d2) {
+    const long long key = cell_key(g, x, y, z);
+    i = cstart[key];
+    end = cstart[key + 1];
   }
-  if (st != 0 && lane == 0)
-    if (atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0) flags->index = (int)q;
+  int c = 0;
+  long long base = MODE ? qptr[q] : 0;
+  while (__any_sync(0xffffffffu, i < end)) {
+    const int n = min(end - i, 32);
+    unsigned hit = 0;
+    for (int u = 0; u < n; ++u) hit |= (unsigned)covers(X, pos[i + u]) << u;
+    const int h = __popc(hit);
+    if (MODE) {
+      int off = h;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, off, o);
+        if (lane >= o) off += t;
+      }
+      long long at = base + off - h;
+      base += __shfl_sync(0xffffffffu, off, 31);
+      for (unsigned b = hit; b; b &= b - 1) qidx[at++] = i + __ffs(b) - 1;
+    } else {
+      c += h;
+    }
+    i += max(n, 0);
+  }
+  if (!MODE) {
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) cnt[q] = c;
+  }
 }
 
-// W[q][j] = sum over the nodes k covering q of phi_k(X_q) C[j][perm k]
-// (C column-major n x m in the caller's order); one warp per point, lanes
-// over the modes
-template <class T>
-__global__ void k_query_weights(const long long* __restrict__ qptr, const int* __restrict__ qidx,
-                                const T* __restrict__ phi, long long nq,
-                                const int* __restrict__ perm, const T* __restrict__ C,
-                                long long n, int m, T* __restrict__ W) {
+// values of the shape functions at the query points, eight lanes each: FP64
+// contexts in double-float, FP32 ones in FP32 (ill-conditioned points listed
+// for the FP64 redo).  scale normalises the linear basis (any positive value
+// gives the same functions; the support size keeps M well scaled).  The
+// weights need no gradients: 30 of the 40 moment sums fall away.
+constexpr int kQueryLanes = 8;
+
+template <class S>
+__global__ void __launch_bounds__(256)
+    k_query_shape(const float4* __restrict__ pos, const float* __restrict__ Q,
+                  const long long* __restrict__ qptr, const int* __restrict__ qidx, long long nq,
+                  float scale, S* __restrict__ phi, double cond_limit, int* __restrict__ redo,
+                  DevFlags* __restrict__ flags) {
+  const long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kQueryLanes;
+  const bool live = q < nq, first = threadIdx.x % kQueryLanes == 0;
+  const long long s = live ? qptr[q] : 0, e = live ? qptr[q + 1] : 0;
+  const float4 Xq = live ? make_float4(Q[3 * q], Q[3 * q + 1], Q[3 * q + 2], scale)
+                         : make_float4(0.f, 0.f, 0.f, 1.f);
+  S* const none = nullptr;
+  if constexpr (sizeof(S) == 4) {
+    const int st = rkpm::shape_rows<float, S, kQueryLanes, false>(pos, s, e, qidx, Xq, phi, none,
+                                                                  0, cond_limit, true);
+    if (live && st != 0 && first) rkpm::redo_later(redo, q);
+  } else {
+    const int st = rkpm::shape_rows<dfloat, S, kQueryLanes, false>(pos, s, e, qidx, Xq, phi, none,
+                                                                   0, 0.0, false);
+    if (live && st != 0 && first &&
+        atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0)
+      flags->index = (int)q;
+  }
+}
+
+// W[q][j] = sum over the nodes k covering q of phi_k(X_q) C[k][j], C row-major
+// with ldc (a multiple of 16 bytes) columns.  One warp a point: W lanes of 16
+// bytes span a row of C, 32 / W rows at a time; the point's pairs are loaded 32
+// at a time, one a lane, and handed round by shuffles.  Bound by the L1 reads of
+// C's rows.  Read column by column from the caller's block (a sector a lane) it
+// took 11.6 ms for 1M points x 98 pairs x 64 FP32 modes, 1.42 ms so.  Nothing is
+// written when the shape functions failed.
+template <class T, class S, int W>
+__global__ void __launch_bounds__(256)
+    k_query_weights(const long long* __restrict__ qptr, const int* __restrict__ qidx,
+                    const S* __restrict__ phi, long long nq, const T* __restrict__ C, int ldc,
+                    int m, T* __restrict__ out, const DevFlags* __restrict__ flags) {
+  constexpr int VEC = 16 / (int)sizeof(T), SUB = 32 / W;
+  using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
   const long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (q >= nq) return;
-  const int lane = threadIdx.x & 31;
+  if (q >= nq || flags->code != 0) return;
+  const int lane = threadIdx.x & 31, sub = lane / W;
   const long long s = qptr[q], e = qptr[q + 1];
-  for (int j = lane; j < m; j += 32) {
-    T acc = T(0);
-    for (long long t = s; t < e; ++t) acc += phi[t] * C[(long long)j * n + perm[qidx[t]]];
-    W[q * m + j] = acc;
+  for (int c0 = 0; c0 < m; c0 += W * VEC) {
+    const int col = c0 + lane % W * VEC;
+    const bool in = col < m;
+    T acc[VEC];
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) acc[v] = T(0);
+    for (long long t = s; t < e; t += 32) {
+      const int cnt = (int)min(32LL, e - t);
+      int k = 0;
+      T ph = T(0);
+      if (lane < cnt) {
+        k = qidx[t + lane];
+        ph = (T)phi[t + lane];
+      }
+#pragma unroll 4
+      for (int u = 0; u < cnt; u += SUB) {
+        const int ku = __shfl_sync(0xffffffffu, k, u + sub);
+        const T pu = __shfl_sync(0xffffffffu, ph, u + sub);
+        if (in && u + sub < cnt) {
+          const V x = *reinterpret_cast<const V*>(C + (long long)ku * ldc + col);
+          const T* xv = reinterpret_cast<const T*>(&x);
+#pragma unroll
+          for (int v = 0; v < VEC; ++v) mac(acc[v], pu, xv[v]);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o >= W; o >>= 1)
+#pragma unroll
+      for (int v = 0; v < VEC; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
+    if (sub == 0)
+#pragma unroll
+      for (int v = 0; v < VEC; ++v)
+        if (col + v < m) out[q * m + col + v] = acc[v];
   }
 }
 
@@ -119,65 +187,95 @@ __global__ void k_lbs(const float* __restrict__ Q, long long nq, const T* __rest
   x[3 * q + 2] = o2;
 }
 
+template <class T, class S>
+void launch_weights(ff_ctx* c, const long long* qptr, const int* qidx, const S* phi, long long nq,
+                    const T* C, int ldc, int m, T* W) {
+  const unsigned grid = ceil_div(nq * 32, 256);
+  const DevFlags* flags = c->flags.as<DevFlags>();
+  auto go = [&](auto lanes) {
+    (k_query_weights<T, S, decltype(lanes)::value><<<grid, 256, 0, c->stream>>>(
+         qptr, qidx, phi, nq, C, ldc, m, W, flags),
+     ::ff::note_launch());
+  };
+  const int need = (m * (int)sizeof(T) + 15) / 16;  // lanes of 16 bytes a row of C
+  if (need <= 4)
+    go(std::integral_constant<int, 4>{});
+  else if (need <= 8)
+    go(std::integral_constant<int, 8>{});
+  else if (need <= 16)
+    go(std::integral_constant<int, 16>{});
+  else
+    go(std::integral_constant<int, 32>{});
+  FF_LAUNCH_CHECK();
+}
+
 template <class T>
 void weights_t(ff_ctx* c, const float* Q, long long nq, const T* C, int m, T* W) {
+  using S = std::conditional_t<sizeof(T) == 4, float, dfloat>;  // the shape values
+  constexpr bool f32 = sizeof(T) == 4;
   cudaStream_t st = c->stream;
   const int TB = 256;
+  long long nq1 = 0;
+  const long long* qptr = nullptr;
+  const int* qidx = nullptr;
+  S* phi = nullptr;
+  const char* what = "nodes";
+  // the nodal values row-major in the internal order, rows of whole 16 bytes
+  const int ldc = (m * (int)sizeof(T) + 15) / 16 * 16 / (int)sizeof(T);
+  T* Ct = reinterpret_cast<T*>(c->sk_c.ensure(sizeof(T) * (size_t)c->n * ldc));
+  gather_block<T>(c, C, m, Ct, ldc);
   if (c->twoset) {
-    const long long nq1 = twoset_cover(c, Q, nq, c->sk_ptr, c->sk_idx, c->sk_cnt);
-    const long long* qptr = c->sk_ptr.as<long long>();
-    const int* qidx = c->sk_idx.as<int>();
-    T* phi = reinterpret_cast<T*>(c->sk_phi.ensure(sizeof(T) * 4 * std::max(nq1, 1LL)));
-    const DevFlags f = twoset_shape(c, Q, nq, qptr, qidx, nq1, phi, phi + nq1, true);
-    if (f.code == FF_ERR_SINGULAR_MOMENT)
-      throw Error(FF_ERR_SINGULAR_MOMENT,
-                  "query point " + std::to_string(f.index) +
-                      " is covered by fewer than four non-coplanar centres");
-    (k_query_weights<T><<<ceil_div(nq * 32, TB), TB, 0, st>>>(qptr, qidx, phi, nq,
-                                                              c->perm.as<int>(), C, c->n, m, W),
+    nq1 = twoset_cover(c, Q, nq, c->sk_ptr, c->sk_idx, c->sk_cnt);
+    qptr = c->sk_ptr.as<long long>();
+    qidx = c->sk_idx.as<int>();
+    phi = reinterpret_cast<S*>(c->sk_phi.ensure(sizeof(S) * std::max(nq1, 1LL)));
+    reset_flags(c);
+    twoset_shape(c, Q, nq, qptr, qidx, nq1, phi, nullptr, f32);
+    what = "centres";
+  } else {
+    const Grid& g = c->grid;
+    const GridDev gd{g.origin[0], g.origin[1], g.origin[2], g.h, g.dims[0], g.dims[1], g.dims[2],
+                     g.bdims[0], g.bdims[1], g.bdims[2]};
+    int* cnt = reinterpret_cast<int*>(c->sk_cnt.ensure(sizeof(int) * (nq + 1)));
+    long long* ptr = reinterpret_cast<long long*>(c->sk_ptr.ensure(sizeof(long long) * (nq + 1)));
+    (k_query_search<0><<<ceil_div(nq * 32, TB), TB, 0, st>>>(Q, nq, c->pos.as<float4>(), gd,
+                                                             c->cell_start.as<int>(), cnt,
+                                                             nullptr, nullptr),
      ::ff::note_launch());
     FF_LAUNCH_CHECK();
+    scan_counts(cnt, ptr, nq, c, c->scratch[3]);
+    FF_CUDA(cudaMemcpyAsync(&nq1, ptr + nq, sizeof(long long), cudaMemcpyDeviceToHost, st));
     FF_CUDA(cudaStreamSynchronize(st));
-    return;
+    int* idx = reinterpret_cast<int*>(c->sk_idx.ensure(sizeof(int) * std::max(nq1, 1LL)));
+    (k_query_search<1><<<ceil_div(nq * 32, TB), TB, 0, st>>>(Q, nq, c->pos.as<float4>(), gd,
+                                                             c->cell_start.as<int>(), nullptr,
+                                                             ptr, idx),
+     ::ff::note_launch());
+    FF_LAUNCH_CHECK();
+    qptr = ptr;
+    qidx = idx;
+    phi = reinterpret_cast<S*>(c->sk_phi.ensure(sizeof(S) * std::max(nq1, 1LL)));
+    reset_flags(c);
+    const float scale = (float)(g.h / 1.001);
+    int* redo = f32 ? rkpm::redo_list(c, nq) : nullptr;
+    (k_query_shape<S><<<ceil_div(nq * kQueryLanes, TB), TB, 0, st>>>(
+         c->pos.as<float4>(), Q, qptr, qidx, nq, scale, phi, 1e2, redo, c->flags.as<DevFlags>()),
+     ::ff::note_launch());
+    FF_LAUNCH_CHECK();
+    if constexpr (f32) {
+      (rkpm::k_shape_redo<S, false, rkpm::BSpline><<<rkpm::redo_grid(nq), 256, 0, st>>>(
+           c->pos.as<float4>(), nullptr, Q, scale, qptr, qidx, 0, phi, nullptr, redo,
+           c->flags.as<DevFlags>(), rkpm::BSpline()),
+       ::ff::note_launch());
+      FF_LAUNCH_CHECK();
+    }
   }
-  const Grid& g = c->grid;
-  const GridDev gd{g.origin[0], g.origin[1], g.origin[2], g.h, g.dims[0], g.dims[1], g.dims[2],
-                   g.bdims[0], g.bdims[1], g.bdims[2]};
-  int* cnt = reinterpret_cast<int*>(c->sk_cnt.ensure(sizeof(int) * (nq + 1)));
-  long long* qptr = reinterpret_cast<long long*>(c->sk_ptr.ensure(sizeof(long long) * (nq + 1)));
-  (k_query_search<0><<<ceil_div(nq, TB), TB, 0, st>>>(Q, nq, c->pos.as<float4>(), gd,
-                                                      c->cell_start.as<int>(), cnt, nullptr,
-                                                      nullptr),
-   ::ff::note_launch());
-  FF_LAUNCH_CHECK();
-  scan_counts(cnt, qptr, nq, c, c->scratch[3]);
-  long long nq1 = 0;
-  FF_CUDA(cudaMemcpyAsync(&nq1, qptr + nq, sizeof(long long), cudaMemcpyDeviceToHost, st));
-  FF_CUDA(cudaStreamSynchronize(st));
-  int* qidx = reinterpret_cast<int*>(c->sk_idx.ensure(sizeof(int) * std::max(nq1, 1LL)));
-  (k_query_search<1><<<ceil_div(nq, TB), TB, 0, st>>>(Q, nq, c->pos.as<float4>(), gd,
-                                                      c->cell_start.as<int>(), nullptr, qptr,
-                                                      qidx),
-   ::ff::note_launch());
-  FF_LAUNCH_CHECK();
-  T* phi = reinterpret_cast<T*>(c->sk_phi.ensure(sizeof(T) * 4 * std::max(nq1, 1LL)));
-  T* dphi = phi + nq1;
-  reset_flags(c);
-  (k_query_shape<T><<<ceil_div(nq * 32, TB), TB, 0, st>>>(
-       c->pos.as<float4>(), Q, qptr, qidx, nq, nq1, (float)(g.h / 1.001), phi, dphi, 1e2,
-       c->flags.as<DevFlags>()),
-   ::ff::note_launch());
-  FF_LAUNCH_CHECK();
+  launch_weights<T, S>(c, qptr, qidx, phi, nq, Ct, ldc, m, W);
   const DevFlags f = read_flags(c);
   if (f.code == FF_ERR_SINGULAR_MOMENT)
     throw Error(FF_ERR_SINGULAR_MOMENT,
                 "query point " + std::to_string(f.index) +
-                    " is covered by fewer than four non-coplanar nodes");
-  (k_query_weights<T><<<ceil_div(nq * 32, TB), TB, 0, st>>>(qptr, qidx, phi, nq,
-                                                            c->perm.as<int>(), C, c->n, m, W),
-   ::ff::note_launch());
-  FF_LAUNCH_CHECK();
-  FF_CUDA(cudaStreamSynchronize(st));
+                    " is covered by fewer than four non-coplanar " + what);
 }
 
 }  // namespace

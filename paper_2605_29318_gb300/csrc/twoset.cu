@@ -31,12 +31,13 @@
 //   k_cover_rows   one thread per point: its covering centres, ascending
 //   k_cover_cols   one warp per centre: the points it covers, ascending, and
 //                  the centre's position in each point's row
-//   k_shape_twoset one warp per quadrature point, Eqs. 7, 9-10 with the Gaussian
+//   k_shape_twoset eight lanes per quadrature point, Eqs. 7, 9-10 with the Gaussian
 #include <cooperative_groups.h>
 
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "dfloat.cuh"
@@ -510,33 +511,46 @@ __global__ void k_cover_cols(const float* __restrict__ Xq, long long nq,
 }
 
 // ------------------------------------------------------------------ shape functions
-template <class T>
-__global__ void __launch_bounds__(256, 2) k_shape_twoset(const float4* __restrict__ cpos, const double* __restrict__ rad,
-                               const float* __restrict__ Xq, float scale,
-                               const long long* __restrict__ ptr, const int* __restrict__ idx,
-                               long long nq, long long n1, T* __restrict__ phi,
-                               T* __restrict__ dphi, double cond_limit,
-                               DevFlags* __restrict__ flags) {
-  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (i >= nq) return;
-  const int lane = threadIdx.x & 31;
-  const long long s = ptr[i], e = ptr[i + 1];
-  const float4 Xi = make_float4(Xq[3 * i], Xq[3 * i + 1], Xq[3 * i + 2], scale);
-  const rkpm::Gauss kern{rad};
-  int st = 1;
-  if (e > s) {
-    if constexpr (sizeof(T) == 4) {
-      st = rkpm::shape_row<float, T>(cpos, s, e, idx, Xi, phi, dphi, n1, cond_limit, true, kern);
-      if (st != 0) {
-        st = rkpm::shape_row<double, T>(cpos, s, e, idx, Xi, phi, dphi, n1, 0.0, false, kern);
-        if (lane == 0 && st == 0) atomicAdd(&flags->fallback, 1);
-      }
-    } else {
-      st = rkpm::shape_row<dfloat, T>(cpos, s, e, idx, Xi, phi, dphi, n1, 0.0, false, kern);
-    }
+// 1 / r_k^2 for the Gaussian's FP32 and double-float forms, rounded from FP64
+// (kept finite: a pair at distance 0 has weight 1 whatever the radius)
+__global__ void k_centre_inv(const double* __restrict__ rad, int K, float4* __restrict__ cpos,
+                             dfloat* __restrict__ inv) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= K) return;
+  const double v = fmin(1.0 / (rad[k] * rad[k]), 3e38);
+  cpos[k].w = (float)v;
+  inv[k] = dfloat(v);
+}
+
+// lanes a row: a point has ~100 covering centres, so eight lanes take a dozen
+// each and a warp's moment solve serves four points.  FP32, 1M points of 98
+// centres: 3.17 ms with a warp a point, 0.95 ms now (values alone 0.41 ms);
+// double-float, 228k points: 5.73 ms, 2.09 ms now.
+constexpr int kShapeLanes = 8;
+
+template <class T, bool GRAD>
+__global__ void __launch_bounds__(256, 2)
+    k_shape_twoset(const float4* __restrict__ cpos, const rkpm::Gauss kern,
+                   const float* __restrict__ Xq, float scale, const long long* __restrict__ ptr,
+                   const int* __restrict__ idx, long long nq, long long n1, T* __restrict__ phi,
+                   T* __restrict__ dphi, double cond_limit, int* __restrict__ redo,
+                   DevFlags* __restrict__ flags) {
+  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kShapeLanes;
+  const bool live = i < nq, first = threadIdx.x % kShapeLanes == 0;
+  const long long s = live ? ptr[i] : 0, e = live ? ptr[i + 1] : 0;
+  const float4 Xi = live ? make_float4(Xq[3 * i], Xq[3 * i + 1], Xq[3 * i + 2], scale)
+                         : make_float4(0.f, 0.f, 0.f, 1.f);
+  if constexpr (sizeof(T) == 4) {
+    const int st = rkpm::shape_rows<float, T, kShapeLanes, GRAD>(
+        cpos, s, e, idx, Xi, phi, dphi, n1, cond_limit, true, kern);
+    if (live && st != 0 && first) rkpm::redo_later(redo, i);
+  } else {
+    const int st = rkpm::shape_rows<dfloat, T, kShapeLanes, GRAD>(
+        cpos, s, e, idx, Xi, phi, dphi, n1, 0.0, false, kern);
+    if (live && st != 0 && first &&
+        atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0)
+      flags->index = (int)i;
   }
-  if (st != 0 && lane == 0)
-    if (atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0) flags->index = (int)i;
 }
 
 __global__ void k_iota(int* __restrict__ a, int* __restrict__ b, int n) {
@@ -580,34 +594,42 @@ long long twoset_cover(ff_ctx* c, const float* Q, long long nq, Buf& ptrb, Buf& 
   return n1;
 }
 
-// Gaussian shape functions of the two-set centres at nq points (one warp each);
-// outputs of the context precision: in FP64 contexts double-float pairs (for
-// the assembly) or FP64 values (fp64_out).  Returns the flags of the pass
-// (code FF_ERR_SINGULAR_MOMENT with the point).
-DevFlags twoset_shape(ff_ctx* c, const float* Q, long long nq, const long long* ptr,
-                      const int* idx, long long n1, void* phi, void* dphi, bool fp64_out) {
+// Gaussian shape functions of the two-set centres at nq points, launched on the
+// context's stream: float (with the FP64 redo) when f32, else double-float
+// pairs; with the gradients when dphi is given.  The caller resets the flags
+// before and reads them after (FF_ERR_SINGULAR_MOMENT with the point).
+void twoset_shape(ff_ctx* c, const float* Q, long long nq, const long long* ptr, const int* idx,
+                  long long n1, void* phi, void* dphi, bool f32) {
   cudaStream_t st = c->stream;
-  const int T = 256;
-  reset_flags(c);
-  ProfScope ps(kProfShape);
-  if (c->prec == FF_PREC_FP64 && fp64_out)
-    (k_shape_twoset<double><<<ceil_div(nq * 32, T), T, 0, st>>>(
-         c->pos.as<float4>(), c->crad.as<double>(), Q, c->qscale, ptr, idx, nq, n1,
-         static_cast<double*>(phi), static_cast<double*>(dphi), 1e2, c->flags.as<DevFlags>()),
+  const float4* cpos = c->pos.as<float4>();
+  const rkpm::Gauss kern{c->crad.as<double>(), c->cinv.as<dfloat>()};
+  DevFlags* flags = c->flags.as<DevFlags>();
+  const unsigned grid = ceil_div(nq * kShapeLanes, 256);
+  auto run = [&](auto tag, auto grad) {
+    using T = decltype(tag);
+    constexpr bool GRAD = decltype(grad)::value;
+    int* redo = sizeof(T) == 4 ? rkpm::redo_list(c, nq) : nullptr;
+    (k_shape_twoset<T, GRAD><<<grid, 256, 0, st>>>(cpos, kern, Q, c->qscale, ptr, idx, nq, n1,
+                                                   static_cast<T*>(phi), static_cast<T*>(dphi),
+                                                   1e2, redo, flags),
      ::ff::note_launch());
-  else if (!tables_f32(c))
-    (k_shape_twoset<dfloat><<<ceil_div(nq * 32, T), T, 0, st>>>(
-         c->pos.as<float4>(), c->crad.as<double>(), Q, c->qscale, ptr, idx, nq, n1,
-         static_cast<dfloat*>(phi), static_cast<dfloat*>(dphi), 1e2, c->flags.as<DevFlags>()),
-     ::ff::note_launch());
+    FF_LAUNCH_CHECK();
+    if constexpr (sizeof(T) == 4) {
+      (rkpm::k_shape_redo<T, GRAD, rkpm::Gauss><<<rkpm::redo_grid(nq), 256, 0, st>>>(
+           cpos, nullptr, Q, c->qscale, ptr, idx, n1, static_cast<T*>(phi),
+           static_cast<T*>(dphi), redo, flags, kern),
+       ::ff::note_launch());
+      FF_LAUNCH_CHECK();
+    }
+  };
+  if (f32 && dphi)
+    run(float{}, std::true_type{});
+  else if (f32)
+    run(float{}, std::false_type{});
+  else if (dphi)
+    run(dfloat{}, std::true_type{});
   else
-    (k_shape_twoset<float><<<ceil_div(nq * 32, T), T, 0, st>>>(
-         c->pos.as<float4>(), c->crad.as<double>(), Q, c->qscale, ptr, idx, nq, n1,
-         static_cast<float*>(phi), static_cast<float*>(dphi), 1e2, c->flags.as<DevFlags>()),
-     ::ff::note_launch());
-  FF_LAUNCH_CHECK();
-  ps.close();
-  return read_flags(c);
+    run(dfloat{}, std::false_type{});
 }
 
 // The transposed covering lists of a two-set cloud: for every centre the
@@ -788,6 +810,10 @@ void build_twoset(ff_ctx* c, const float* Xq, const float* vq, long long nq, int
   f = read_flags(c);
   FF_REQUIRE(f.code == 0, FF_ERR_INVALID_ARG,
              "centre " + std::to_string(f.index) + " has a zero radius");
+  (k_centre_inv<<<ceil_div(K, T), T, 0, st>>>(
+       rad, K, cpos, reinterpret_cast<dfloat*>(c->cinv.ensure(sizeof(dfloat) * K))),
+   ::ff::note_launch());
+  FF_LAUNCH_CHECK();
   std::vector<double> hr(K);
   FF_CUDA(cudaMemcpy(hr.data(), rad, sizeof(double) * K, cudaMemcpyDeviceToHost));
   // basis scale of the shape functions (any positive value gives the same
@@ -819,8 +845,13 @@ void build_twoset(ff_ctx* c, const float* Xq, const float* vq, long long nq, int
   const size_t es = tables_f32(c) ? 4 : 8;
   c->phi.ensure(es * std::max(n1, 1LL));
   c->dphi.ensure(3 * es * std::max(n1, 1LL));
-  f = twoset_shape(c, Xq, nq, c->nbr_ptr.as<long long>(), c->nbr_idx.as<int>(), n1, c->phi.p,
-                   c->dphi.p, false);
+  reset_flags(c);
+  {
+    ProfScope ps(kProfShape);
+    twoset_shape(c, Xq, nq, c->nbr_ptr.as<long long>(), c->nbr_idx.as<int>(), n1, c->phi.p,
+                 c->dphi.p, tables_f32(c));
+  }
+  f = read_flags(c);
   c->hflags->fallback = f.fallback;
   if (f.code == FF_ERR_SINGULAR_MOMENT)
     throw Error(FF_ERR_SINGULAR_MOMENT,

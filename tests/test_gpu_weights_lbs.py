@@ -1,0 +1,61 @@
+"""Skinning weights and linear blend skinning on GB300 at the sizes where their
+kernels change path: widths around the vector lanes of a row, points around the
+blocks, aligned and unaligned weights."""
+import numpy as np
+import pytest
+
+from paper_2605_29318_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+def _ctx(prec):
+    import torch
+    from paper_2605_29318_gb300 import binding
+    c = synth.unit_cube(1500, seed=11)
+    c.a = synth.support_floor(c.X, c.a, factor=1.5)
+    ctx = binding.Context(0, prec)
+    ctx.rkpm_build(*(torch.from_numpy(x).to(DEV) for x in (c.X, c.v, c.a)))
+    return c, ctx
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("m", [1, 3, 16, 17, 33, 64, 65, 130])
+def test_weights_at_every_lane_split(prec, m):
+    """W = phi C with phi the exported shape functions: queries at the
+    particles.  A row's sum of c terms is within (c + 2) eps sum |phi C| of the
+    exact one; the query's shape functions sum their moments in another order
+    than the build's, each within 1e3 condition-weighted roundings (the redo
+    limit is 1e2 in FP32; FP64 contexts carry 2^-47)."""
+    import torch
+    c, ctx = _ctx(prec)
+    ptr, idx, phi, _ = ctx.export_rkpm()
+    C = torch.randn(c.n, m, device=DEV, dtype=ctx.dtype,
+                    generator=torch.Generator(device=DEV).manual_seed(m))
+    nq = 257
+    Q = torch.from_numpy(c.X[:nq]).to(DEV)
+    W = ctx.skinning_weights(Q, C).double().cpu().numpy()
+    Cd = C.double().cpu().numpy()
+    unit = 2.0 ** -24 if prec == "fp32" else 2.0 ** -47
+    for q in range(nq):
+        s = slice(ptr[q], ptr[q + 1])
+        exact = phi[s] @ Cd[idx[s]]
+        bound = 1e3 * unit * (np.abs(phi[s]) @ np.abs(Cd[idx[s]]))
+        assert (np.abs(W[q] - exact) <= bound).all(), (q, np.abs(W[q] - exact).max())
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_failed_weights_leave_the_output_alone(prec):
+    import torch
+    from paper_2605_29318_gb300 import binding
+    c, ctx = _ctx(prec)
+    Q = torch.from_numpy(c.X[:40]).to(DEV).clone()
+    Q[17] = 50.0                       # covered by nothing
+    W = torch.full((40, 5), 7.0, dtype=ctx.dtype, device=DEV)
+    C = torch.ones((5, c.n), dtype=ctx.dtype, device=DEV)
+    st = ctx.L.ff_skinning_weights(ctx.h, Q.data_ptr(), 40, C.data_ptr(), 5, W.data_ptr())
+    assert binding.STATUS[st] == "FF_ERR_SINGULAR_MOMENT"
+    assert "query point 17 " in ctx.L.ff_last_error(ctx.h).decode()
+    assert bool((W == 7.0).all())
