@@ -17,6 +17,7 @@
 // over the modes, from a row-major copy of the nodal values.  Clouds of the
 // two-set discretisation take its own covering test over the K centres and its
 // Gaussian shape functions (twoset.cu).
+#include <cstdint>
 #include <type_traits>
 
 #include "grid.cuh"
@@ -167,24 +168,151 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// x_q = X_q + sum_j W[q][j] Z_j [X_q; 1]  (Z row-major m x 3 x 4)
-template <class T>
-__global__ void k_lbs(const float* __restrict__ Q, long long nq, const T* __restrict__ W, int m,
-                      const T* __restrict__ Z, T* __restrict__ x) {
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  const T X0 = (T)Q[3 * q], X1 = (T)Q[3 * q + 1], X2 = (T)Q[3 * q + 2];
-  T o0 = X0, o1 = X1, o2 = X2;
-  for (int j = 0; j < m; ++j) {
-    const T w = W[q * m + j];
-    const T* z = Z + 12LL * j;
-    o0 += w * (z[0] * X0 + z[1] * X1 + z[2] * X2 + z[3]);
-    o1 += w * (z[4] * X0 + z[5] * X1 + z[6] * X2 + z[7]);
-    o2 += w * (z[8] * X0 + z[9] * X1 + z[10] * X2 + z[11]);
+// x_q = X_q + sum_j W[q][j] Z_j [X_q; 1]  (Z row-major m x 3 x 4).  A block
+// stages its rows of W and the transforms, kCols modes at a time, in shared
+// memory: by 16-byte asynchronous copies (kCopy; W 16-byte aligned and its rows
+// whole 16 bytes), else by plain loads, a warp 128 consecutive bytes (kLoad).
+// The staged rows are 16 bytes longer than their columns, so that a thread a
+// point reads its own row 16 bytes at a time without bank conflicts; with kCopy
+// a thread takes PTS points, which share its reads of the transforms.  FP32 rows
+// of up to 64 modes that are not whole 16 bytes come as one flat copy of the
+// block's span of W (kFlat), which starts on a 16-byte boundary where W does;
+// read at a stride of m words, m % 4 != 0, that is two lanes a bank at most.  Rows
+// of at most 32 bytes are read where they lie (kDirect): a sector or two a thread
+// either way.
+// Bound by reading W: every thread walking its row in global memory (a sector a
+// lane a load) took 326 us for 1M points x 64 FP32 modes, 58 us so; in FP64 by
+// its arithmetic (1.64 ms so, 1.27 ms with the 12 multiply-adds a mode of the form
+// below).
+enum LbsRead { kDirect, kLoad, kCopy, kFlat };
+
+constexpr int kLbsFlat = 64;
+
+template <class T, int TB, int PTS, LbsRead READ>
+__global__ void __launch_bounds__(TB, 1024 / (TB * PTS))
+    k_lbs(const float* __restrict__ Q, long long nq, const T* __restrict__ W, int m,
+          const T* __restrict__ Z, T* __restrict__ x) {
+  constexpr int E = 16 / (int)sizeof(T);  // elements of 16 bytes
+  constexpr int kCols = READ == kFlat ? kLbsFlat : 32;
+  constexpr int kRows = READ == kDirect ? 1 : TB * PTS;
+  __shared__ __align__(16) T sw[kRows][READ == kFlat ? kCols : kCols + E];
+  T* const flat = &sw[0][0];
+  __shared__ __align__(16) T sz[kCols][12];
+  const long long q0 = (long long)blockIdx.x * TB * PTS;
+  const int rows = (int)min((long long)TB * PTS, nq - q0);
+  const int tid = threadIdx.x;
+  T X[PTS][3], o[PTS][3];
+  int row[PTS];
+#pragma unroll
+  for (int p = 0; p < PTS; ++p) {
+    row[p] = min(tid + p * TB, rows - 1);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) o[p][d] = X[p][d] = (T)Q[3 * (q0 + row[p]) + d];
   }
-  x[3 * q] = o0;
-  x[3 * q + 1] = o1;
-  x[3 * q + 2] = o2;
+  for (int j0 = 0; j0 < m; j0 += kCols) {
+    const int jn = min(kCols, m - j0);
+    const T* w0 = W + q0 * m + j0;
+    if (j0) __syncthreads();
+    if constexpr (READ == kCopy) {
+      constexpr int kVecs = kCols / E;
+#pragma unroll 4
+      for (int t = tid; t < TB * PTS * kVecs; t += TB) {
+        const int r = t / kVecs, c = t % kVecs * E;
+        if (r < rows && c < jn) {
+          const unsigned dst = (unsigned)__cvta_generic_to_shared(&sw[r][c]);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst),
+                       "l"(w0 + (long long)r * m + c)
+                       : "memory");
+        }
+      }
+    } else if constexpr (READ == kFlat) {  // m <= kCols: the one chunk
+      const int total = rows * m;
+#pragma unroll 4
+      for (int t = tid * E; t < total; t += TB * E) {
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(flat + t);
+        if (t + E <= total)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(w0 + t)
+                       : "memory");
+        else
+          for (int u = t; u < total; ++u) flat[u] = w0[u];
+      }
+    } else if constexpr (READ == kLoad) {
+      const int lane = tid & 31;
+      if (lane < jn)
+#pragma unroll 4
+        for (int r = tid >> 5; r < rows; r += TB / 32) sw[r][lane] = w0[(long long)r * m + lane];
+    }
+    for (int t = tid; t < 12 * jn; t += TB) (&sz[0][0])[t] = Z[12LL * j0 + t];
+    if constexpr (READ == kCopy || READ == kFlat)
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    auto add = [&](int p, T wj, const T* z) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+        mac(o[p][d], wj,
+            fma(z[4 * d + 2], X[p][2],
+                fma(z[4 * d + 1], X[p][1], fma(z[4 * d], X[p][0], z[4 * d + 3]))));
+    };
+    int j = 0;
+    if constexpr (READ == kCopy || READ == kLoad)
+      for (; j + E <= jn; j += E) {
+        T wv[PTS][E];
+#pragma unroll
+        for (int p = 0; p < PTS; ++p)
+          *reinterpret_cast<uint4*>(wv[p]) = *reinterpret_cast<const uint4*>(&sw[row[p]][j]);
+#pragma unroll
+        for (int u = 0; u < E; ++u)
+#pragma unroll
+          for (int p = 0; p < PTS; ++p) add(p, wv[p][u], sz[j + u]);
+      }
+    for (; j < jn; ++j)
+#pragma unroll
+      for (int p = 0; p < PTS; ++p) {
+        if constexpr (READ == kDirect)
+          add(p, w0[(long long)row[p] * m + j], sz[j]);
+        else if constexpr (READ == kFlat)
+          add(p, flat[row[p] * m + j], sz[j]);
+        else
+          add(p, sw[row[p]][j], sz[j]);
+      }
+  }
+#pragma unroll
+  for (int p = 0; p < PTS; ++p)
+    if (tid + p * TB < rows)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x[3 * (q0 + row[p]) + d] = o[p][d];
+}
+
+template <class T>
+void lbs_t(ff_ctx* c, const float* Q, long long nq, const T* W, int m, const T* Z, T* x) {
+  auto go = [&](auto tb, auto pts, auto read) {
+    constexpr int TB = decltype(tb)::value, PTS = decltype(pts)::value;
+    (k_lbs<T, TB, PTS, decltype(read)::value>
+     <<<ceil_div(nq, TB * PTS), TB, 0, c->stream>>>(Q, nq, W, m, Z, x),
+     ::ff::note_launch());
+  };
+  // blocks of 128 threads where those fill the chip twice over, two points a
+  // thread for FP32 copies; fewer points are spread thinner, 32 a block (1,000
+  // points in 8 blocks of 128 would leave 144 SMs idle)
+  auto pick = [&](auto read) {
+    using One = std::integral_constant<int, 1>;
+    using Pts = std::integral_constant<int, sizeof(T) == 4 && decltype(read)::value == kCopy ? 2 : 1>;
+    if (nq >= 2LL * 128 * Pts::value * sm_count())
+      go(std::integral_constant<int, 128>{}, Pts{}, read);
+    else
+      go(std::integral_constant<int, 32>{}, One{}, read);
+  };
+  const bool aligned = reinterpret_cast<uintptr_t>(W) % 16 == 0;
+  if (m * sizeof(T) <= 32)
+    pick(std::integral_constant<LbsRead, kDirect>{});
+  else if (aligned && m * sizeof(T) % 16 == 0)
+    pick(std::integral_constant<LbsRead, kCopy>{});
+  else if (aligned && m <= kLbsFlat && sizeof(T) == 4)
+    pick(std::integral_constant<LbsRead, sizeof(T) == 4 ? kFlat : kLoad>{});
+  else
+    pick(std::integral_constant<LbsRead, kLoad>{});
+  FF_LAUNCH_CHECK();
+  FF_CUDA(cudaStreamSynchronize(c->stream));
 }
 
 template <class T, class S>
@@ -291,19 +419,12 @@ void skinning_weights(ff_ctx* c, const float* Q, long long nq, const void* C, in
 void lbs_deform(ff_ctx* c, const float* Q, long long nq, const void* W, int m, const void* Z,
                 void* x) {
   if (nq == 0) return;
-  const int TB = 256;
   if (c->prec == FF_PREC_FP64)
-    (k_lbs<double><<<ceil_div(nq, TB), TB, 0, c->stream>>>(Q, nq, static_cast<const double*>(W),
-                                                           m, static_cast<const double*>(Z),
-                                                           static_cast<double*>(x)),
-     ::ff::note_launch());
+    lbs_t<double>(c, Q, nq, static_cast<const double*>(W), m, static_cast<const double*>(Z),
+                  static_cast<double*>(x));
   else
-    (k_lbs<float><<<ceil_div(nq, TB), TB, 0, c->stream>>>(Q, nq, static_cast<const float*>(W), m,
-                                                          static_cast<const float*>(Z),
-                                                          static_cast<float*>(x)),
-     ::ff::note_launch());
-  FF_LAUNCH_CHECK();
-  FF_CUDA(cudaStreamSynchronize(c->stream));
+    lbs_t<float>(c, Q, nq, static_cast<const float*>(W), m, static_cast<const float*>(Z),
+                 static_cast<float*>(x));
 }
 
 }  // namespace ff

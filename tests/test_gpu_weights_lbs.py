@@ -9,6 +9,7 @@ from paper_2605_29318_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 DEV = "cuda:0"
+EPS = {"fp32": 2.0 ** -24, "fp64": 2.0 ** -53}
 
 
 def _ctx(prec):
@@ -59,3 +60,27 @@ def test_failed_weights_leave_the_output_alone(prec):
     assert binding.STATUS[st] == "FF_ERR_SINGULAR_MOMENT"
     assert "query point 17 " in ctx.L.ff_last_error(ctx.h).decode()
     assert bool((W == 7.0).all())
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("m", [1, 2, 4, 5, 8, 9, 33, 62, 64, 65, 100])
+@pytest.mark.parametrize("nq", [1, 33, 80001])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_lbs_in_every_read_form(prec, m, nq, shift):
+    """Each mode adds one product of a four-term form: the sum is within
+    (m + 6) eps of the sum of absolute terms.  shift = 1 takes the weights off
+    their 16-byte boundary."""
+    import torch
+    from paper_2605_29318_gb300 import binding
+    ctx = binding.Context(0, prec)
+    g = torch.Generator(device=DEV).manual_seed(100 * m + shift)
+    Q = torch.randn(nq, 3, device=DEV, generator=g)
+    room = torch.randn(nq * m + shift, device=DEV, dtype=ctx.dtype, generator=g)
+    W = room[shift:].view(nq, m)
+    Z = torch.randn(m, 3, 4, device=DEV, dtype=ctx.dtype, generator=g)
+    x = ctx.lbs(Q, W, Z).double()
+    h = torch.cat([Q.double(), torch.ones(nq, 1, device=DEV, dtype=torch.float64)], 1)
+    Wd, Zd = W.double(), Z.double()
+    exact = Q.double() + torch.einsum("qm,mrc,qc->qr", Wd, Zd, h)
+    terms = Q.double().abs() + torch.einsum("qm,mrc,qc->qr", Wd.abs(), Zd.abs(), h.abs())
+    assert bool(((x - exact).abs() <= (m + 6) * EPS[prec] * terms).all())
