@@ -22,18 +22,13 @@
 // patterns where they are ordered (non-negative doubles order like integers).
 //
 // Kernels:
-//   k_fps          one 8-block cluster: each block keeps its slice of points
-//                  and their running squared distance to the chosen set in
-//                  shared memory (global memory when it does not fit); per
-//                  chosen centre: update, block arg-max, one cluster barrier,
-//                  every block reduces the 8 published candidates itself
+//   k_fps_rounds   up to one block per SM, each with its slice of the points;
+//                  several centres a grid barrier
 //   k_radii        one warp per centre: the two smallest squared distances
 //   k_cover_rows   one thread per point: its covering centres, ascending
 //   k_cover_cols   one warp per centre: the points it covers, ascending, and
 //                  the centre's position in each point's row
 //   k_shape_twoset eight lanes per quadrature point, Eqs. 7, 9-10 with the Gaussian
-#include <cooperative_groups.h>
-
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -47,10 +42,8 @@
 namespace ff {
 namespace {
 
-constexpr int kFpsCS = 8;                    // blocks per cluster
-constexpr int kFpsT = 1024;                  // threads per block
+constexpr int kFpsT = 512;                   // threads per block
 constexpr int kFpsSmemMax = 200 * 1024;      // dynamic shared memory per block
-constexpr int kFpsGridMin = 200000;          // points from which the whole GPU samples
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ double d2_f64(float ax, float ay, float az, float bx, float by,
@@ -65,6 +58,13 @@ __device__ __forceinline__ float d2_f32(float ax, float ay, float az, float bx, 
                                         float bz) {
   const float dx = __fsub_rn(ax, bx), dy = __fsub_rn(ay, by), dz = __fsub_rn(az, bz);
   return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+}
+
+// the filter's form, within the same margin of the FP64 value
+__device__ __forceinline__ float d2_fma(float ax, float ay, float az, float bx, float by,
+                                        float bz) {
+  const float dx = ax - bx, dy = ay - by, dz = az - bz;
+  return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
 }
 
 // centre (p, l32 = fl32(lim), lim = t^2 r^2 or +inf) covers the point (x, y, z)
@@ -91,141 +91,10 @@ __global__ void k_validate_points(const float* __restrict__ X, const float* __re
 }
 
 // ------------------------------------------------------------------ farthest-point sampling
-struct FpsCand {
-  unsigned long long key;  // bit pattern of the squared distance (>= 0)
-  int idx;
-  float x, y, z;
-  int pad;
-};
-
-__device__ __forceinline__ void fps_pick(FpsCand& a, unsigned long long key, int idx, float x,
-                                         float y, float z) {
-  if (key > a.key || (key == a.key && idx < a.idx)) {
-    a.key = key;
-    a.idx = idx;
-    a.x = x;
-    a.y = y;
-    a.z = z;
-  }
-}
-
-__device__ __forceinline__ void fps_warp_max(FpsCand& a) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long k2 = __shfl_xor_sync(kFull, a.key, o);
-    const int i2 = __shfl_xor_sync(kFull, a.idx, o);
-    const float x2 = __shfl_xor_sync(kFull, a.x, o);
-    const float y2 = __shfl_xor_sync(kFull, a.y, o);
-    const float z2 = __shfl_xor_sync(kFull, a.z, o);
-    fps_pick(a, k2, i2, x2, y2, z2);
-  }
-}
-
-// Block b owns points [b S, min(n, (b + 1) S)).  cur = squared distance to the
-// chosen set (FP64), cur32 its FP32 rounding for the filter.  Every block
-// computes the same winner from the same 8 candidates, so all leave the loop
-// together; the published candidates alternate between two buffers, so the
-// one cluster barrier per step also orders their reuse.
-__global__ void __cluster_dims__(kFpsCS, 1, 1) __launch_bounds__(kFpsT, 1)
-    k_fps(const float* __restrict__ X, int n, int K, int start, int S, int in_smem,
-          float* __restrict__ gxyz, double* __restrict__ gcur, float* __restrict__ gcur32,
-          long long* __restrict__ chosen, DevFlags* __restrict__ flags) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank();
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int p0 = min(rank * S, n);
-  const int cnt = min(n - p0, S);
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  __shared__ FpsCand pub[2];
-  __shared__ FpsCand red[kFpsT / 32];
-  double* cur;
-  float *cur32, *xs, *ys, *zs;
-  if (in_smem) {
-    cur = reinterpret_cast<double*>(sm_raw);
-    cur32 = reinterpret_cast<float*>(cur + S);
-    xs = cur32 + S;
-    ys = xs + S;
-    zs = ys + S;
-  } else {
-    cur = gcur + p0;
-    cur32 = gcur32 + p0;
-    xs = gxyz + p0;
-    ys = gxyz + (size_t)n + p0;
-    zs = gxyz + 2 * (size_t)n + p0;
-  }
-  const float sx = X[3LL * start], sy = X[3LL * start + 1], sz = X[3LL * start + 2];
-  for (int p = tid; p < cnt; p += kFpsT) {
-    const long long g = (long long)p0 + p;
-    const float x = X[3 * g], y = X[3 * g + 1], z = X[3 * g + 2];
-    xs[p] = x;
-    ys[p] = y;
-    zs[p] = z;
-    const double d = d2_f64(x, y, z, sx, sy, sz);
-    cur[p] = d;
-    cur32[p] = (float)d;
-  }
-  if (rank == 0 && tid == 0) chosen[0] = start;
-  __syncthreads();
-  float cx = sx, cy = sy, cz = sz;
-  for (int j = 1; j < K; ++j) {
-    const int buf = j & 1;
-    FpsCand best{0ull, INT_MAX, 0.f, 0.f, 0.f, 0};
-    for (int p = tid; p < cnt; p += kFpsT) {
-      const float x = xs[p], y = ys[p], z = zs[p];
-      double c = cur[p];
-      if (j > 1) {  // fold in the centre chosen last (the start is in already)
-        const float c32 = cur32[p];
-        if (c32 < 1e-30f || d2_f32(x, y, z, cx, cy, cz) <= __fmul_rn(c32, 1.00001f)) {
-          const double d = d2_f64(x, y, z, cx, cy, cz);
-          if (d < c) {
-            c = d;
-            cur[p] = d;
-            cur32[p] = (float)d;
-          }
-        }
-      }
-      fps_pick(best, (unsigned long long)__double_as_longlong(c), p0 + p, x, y, z);
-    }
-    fps_warp_max(best);
-    if (lane == 0) red[wid] = best;
-    __syncthreads();
-    if (wid == 0) {
-      FpsCand b = red[lane];
-      fps_warp_max(b);
-      if (lane == 0) pub[buf] = b;
-    }
-    cl.sync();
-    FpsCand win{0ull, INT_MAX, 0.f, 0.f, 0.f, 0};
-#pragma unroll
-    for (int q = 0; q < kFpsCS; ++q) {
-      const FpsCand r = *cl.map_shared_rank(&pub[buf], q);
-      fps_pick(win, r.key, r.idx, r.x, r.y, r.z);
-    }
-    if (win.key == 0ull || win.idx == INT_MAX) {
-      // every remaining point coincides with a chosen centre
-      if (rank == 0 && tid == 0 && atomicCAS(&flags->code, 0, (int)FF_ERR_INVALID_ARG) == 0)
-        flags->index = j;
-      break;
-    }
-    if (rank == 0 && tid == 0) chosen[j] = win.idx;
-    cx = win.x;
-    cy = win.y;
-    cz = win.z;
-  }
-  cl.sync();  // no block leaves while another may still read its candidates
-}
-
-// The same sampling on the whole GPU: one block per SM in a cooperative
-// launch, each holding its slice of the points and their running distances in
-// shared memory (global memory when the slice does not fit).  Per centre:
-// update, block arg-max, the block's candidate published to global memory
-// (two buffers by parity), a grid barrier, and every block reduces all the
-// published candidates itself -- the same winner everywhere, so every block
-// leaves the loop at the same step.  The barrier is a monotone arrival counter
-// in global memory; its wait is bounded (about a second of clock cycles) and
-// a block that gives up records FF_ERR_TIMEOUT in the flags and in `abort`, and
-// every block leaves the loop at the next barrier it sees it at.
+// The grid barrier is a monotone arrival counter in global memory; its wait is
+// bounded (about a second of clock cycles) and a block that gives up records
+// FF_ERR_TIMEOUT in the flags and in `abort`, and every block leaves at the next
+// barrier it sees it at.
 constexpr long long kGridWaitCycles = 2000000000LL;
 
 __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int* abort,
@@ -258,104 +127,443 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int
   return s_abort == 0;
 }
 
+// Farthest-point sampling in rounds, a cooperative launch of up to one block per
+// SM.  Block b owns points [b S, min(n, (b + 1) S)) and keeps, in shared memory
+// (global memory when the slice does not fit), each point's position, the FP32
+// squared distance to its nearest chosen centre and that centre's index; the
+// exact (FP64) distance is computed from the two only where it decides.
+//
+// A distance only falls as centres are added, so the largest distance known
+// for a point bounds it for the rest of the run.  Each round
+//   1. folds the centres chosen last into the slice (FP32; FP64 within the
+//      margin of a near tie),
+//   2. publishes the block's `top` farthest points in the exact order
+//      (distance, then lowest index), and the next one as its bound,
+//   3. one grid barrier,
+//   4. every block chooses centres among the published points alone (two a
+//      thread; 256 threads of four points took 1.3 times as long), folding each into the others, while the
+//      farthest of them comes before every block's bound in that order: no
+//      unpublished point can then come before it, so it is the farthest of all
+//      points.  FP32 decides a choice unless two distances, or one and the
+//      bound, lie within its margin.
+// The first choice of a round always passes, so a round adds one centre at
+// least; holes of the covering are many once some tens of centres stand, and a
+// round adds up to kFpsNew.
+//
+// One centre a barrier was bound by the barrier and by FP64 updates (a warp
+// instruction costs the same for one lane as for 32): 8.19 ms for 1M points and
+// 1,000 centres, 6.45 ms for 228k grid points; 1.50 and 1.81 ms in 37
+// and 51 rounds.  Up to 1,024 points one block takes them all as
+// its published points and needs no round.
+struct FpsCand {
+  unsigned long long key;  // bit pattern of the squared distance (>= 0)
+  int idx;
+  float x, y, z;
+  int near;                // its nearest chosen centre
+  int pad;
+};
+
+constexpr int kFpsNew = 128;   // centres a round chooses at most
+constexpr int kPool = 2 * kFpsT;  // published points: two a thread
+constexpr unsigned long long kNoKey = ~0ull;
+
+// whether (ka, ia) comes before (kb, ib): larger key, ties to the lower index
+__device__ __forceinline__ bool fps_before(unsigned long long ka, int ia, unsigned long long kb,
+                                           int ib) {
+  return ka > kb || (ka == kb && ia < ib);
+}
+
+// the first of the warp's (key, idx) in every lane
+__device__ __forceinline__ void fps_warp_first(unsigned long long& key, int& idx) {
+  const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+  const unsigned mh = __reduce_max_sync(kFull, hi);
+  const unsigned ml = __reduce_max_sync(kFull, hi == mh ? lo : 0u);
+  idx = __reduce_min_sync(kFull, hi == mh && lo == ml ? idx : INT_MAX);
+  key = (unsigned long long)mh << 32 | ml;
+}
+
+// the first (key, idx) of the block, with its position, in every thread; red
+// alternates between two buffers, so one barrier a call also orders its reuse
+__device__ __forceinline__ FpsCand fps_block_first(FpsCand c, FpsCand (*red)[kFpsT / 32],
+                                                   int& buf) {
+  const int lane = threadIdx.x & 31;
+  FpsCand w = c;
+  fps_warp_first(w.key, w.idx);
+  const unsigned own = __ballot_sync(kFull, c.key == w.key && c.idx == w.idx);
+  if (lane == __ffs(own) - 1) red[buf][threadIdx.x >> 5] = c;
+  __syncthreads();
+  c = red[buf][lane % (kFpsT / 32)];
+  buf ^= 1;
+  w = c;
+  fps_warp_first(w.key, w.idx);
+  const int src = __ffs(__ballot_sync(kFull, c.key == w.key && c.idx == w.idx)) - 1;
+  w.x = __shfl_sync(kFull, c.x, src);
+  w.y = __shfl_sync(kFull, c.y, src);
+  w.z = __shfl_sync(kFull, c.z, src);
+  return w;
+}
+
+// (called, not inlined: the deciding paths are rare and the FP32 ones short)
+__device__ __noinline__ unsigned long long fps_key(float x, float y, float z,
+                                                      const float* __restrict__ X, int centre) {
+  return (unsigned long long)__double_as_longlong(
+      d2_f64(x, y, z, X[3LL * centre], X[3LL * centre + 1], X[3LL * centre + 2]));
+}
+
+// the FP32 distance up to which a new centre may be nearer than d: the filter's
+// margin above it, everything for tiny distances, nothing for d < 0
+__device__ __forceinline__ float fps_near(float d) {
+  return d >= 0.f && d < 1e-30f ? INFINITY : __fmul_rn(d, 1.00001f);
+}
+
+// the largest and second largest FP32 distance (bits) of a warp's published
+// points, and the point of the largest
+struct __align__(16) FpsPick {
+  int m1, m2, idx, pad;
+  float x, y, z, w;
+};
+
 __global__ void __launch_bounds__(kFpsT, 1)
-    k_fps_grid(const float* __restrict__ X, int n, int K, int start, int S, int in_smem,
-               float* __restrict__ gxyz, double* __restrict__ gcur, float* __restrict__ gcur32,
-               long long* __restrict__ chosen, FpsCand* __restrict__ cand, unsigned* bar,
-               int* abort, DevFlags* __restrict__ flags) {
+    k_fps_rounds(const float* __restrict__ X, int n, int K, int start, int S, int top,
+                 int in_smem, float* __restrict__ gslice, int* __restrict__ gnear,
+                 long long* __restrict__ chosen, FpsCand* __restrict__ cand, unsigned* bar,
+                 int* abort, DevFlags* __restrict__ flags) {
   const int G = gridDim.x, rank = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int p0 = min(rank * S, n);
+  const int p0 = (int)min((long long)rank * S, (long long)n);
   const int cnt = min(n - p0, S);
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  __shared__ FpsCand red[kFpsT / 32];
-  __shared__ FpsCand s_win;
-  double* cur;
-  float *cur32, *xs, *ys, *zs;
+  __shared__ FpsCand red[2][kFpsT / 32];
+  __shared__ float4 fresh[kFpsNew];  // the centres chosen last, w their index
+  __shared__ unsigned s_max[kFpsT / 16];
+  static_assert(kFpsT == 512, "the threshold takes 32 half-warps, one a lane");
+  __shared__ FpsPick pick[2][kFpsT / 32];
+  __shared__ FpsCand tie[2][kFpsT / 32];
+  float *xs, *ys, *zs, *cur;
+  int* near;
   if (in_smem) {
-    cur = reinterpret_cast<double*>(sm_raw);
-    cur32 = reinterpret_cast<float*>(cur + S);
-    xs = cur32 + S;
-    ys = xs + S;
-    zs = ys + S;
+    xs = reinterpret_cast<float*>(sm_raw);
+    near = reinterpret_cast<int*>(xs + 4 * (size_t)S);
   } else {
-    cur = gcur + p0;
-    cur32 = gcur32 + p0;
-    xs = gxyz + p0;
-    ys = gxyz + (size_t)n + p0;
-    zs = gxyz + 2 * (size_t)n + p0;
+    xs = gslice + 4 * (size_t)S * rank;
+    near = gnear + (size_t)S * rank;
   }
-  const float sx = X[3LL * start], sy = X[3LL * start + 1], sz = X[3LL * start + 2];
+  ys = xs + S;
+  zs = ys + S;
+  cur = zs + S;
   for (int p = tid; p < cnt; p += kFpsT) {
-    const long long g = (long long)p0 + p;
-    const float x = X[3 * g], y = X[3 * g + 1], z = X[3 * g + 2];
-    xs[p] = x;
-    ys[p] = y;
-    zs[p] = z;
-    const double d = d2_f64(x, y, z, sx, sy, sz);
-    cur[p] = d;
-    cur32[p] = (float)d;
+    const long long g = 3LL * (p0 + p);
+    xs[p] = X[g];
+    ys[p] = X[g + 1];
+    zs[p] = X[g + 2];
+    cur[p] = __int_as_float(0x7f800000);
+    near[p] = start;
   }
-  if (rank == 0 && tid == 0) chosen[0] = start;
+  if (tid == 0) {
+    fresh[0] = make_float4(X[3LL * start], X[3LL * start + 1], X[3LL * start + 2],
+                           __int_as_float(start));
+    if (rank == 0) chosen[0] = start;
+  }
   __syncthreads();
-  float cx = sx, cy = sy, cz = sz;
-  for (int j = 1; j < K; ++j) {
-    FpsCand best{0ull, INT_MAX, 0.f, 0.f, 0.f, 0};
-    for (int p = tid; p < cnt; p += kFpsT) {
-      const float x = xs[p], y = ys[p], z = zs[p];
-      double c = cur[p];
-      if (j > 1) {  // fold in the centre chosen last (the start is in already)
-        const float c32 = cur32[p];
-        if (c32 < 1e-30f || d2_f32(x, y, z, cx, cy, cz) <= __fmul_rn(c32, 1.00001f)) {
-          const double d = d2_f64(x, y, z, cx, cy, cz);
-          if (d < c) {
-            c = d;
-            cur[p] = d;
-            cur32[p] = (float)d;
+  int nnew = 1, j = 1, buf = 0, pbuf = 0, tbuf = 0;
+  const bool whole = G == 1 && n <= kPool;  // every point is a published one
+  const FpsCand* pool = nullptr;
+  unsigned long long bkey = 0ull;
+  int bidx = INT_MAX;
+  for (int round = 1; j < K; ++round) {
+    if (!whole) {
+      // ---- 1. fold in the fresh centres (four points a thread at a time)
+      unsigned fmax = 0;  // bits of the thread's largest FP32 distance
+      for (int q = tid; q < cnt; q += 4 * kFpsT) {
+        float x[4], y[4], z[4], d[4];
+        int c[4];
+  #pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int p = q + u * kFpsT;
+          const bool in = p < cnt;
+          x[u] = in ? xs[p] : 0.f;
+          y[u] = in ? ys[p] : 0.f;
+          z[u] = in ? zs[p] : 0.f;
+          d[u] = in ? cur[p] : -1.f;  // -1: below every squared distance
+          c[u] = in ? near[p] : 0;
+        }
+        float near_d[4];  // a distance up to this needs a closer look
+#pragma unroll
+        for (int u = 0; u < 4; ++u) near_d[u] = fps_near(d[u]);
+        for (int b = 0; b < nnew; ++b) {
+          const float4 f = fresh[b];
+          float dn[4];
+          bool look = false;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            dn[u] = d2_fma(x[u], y[u], z[u], f.x, f.y, f.z);
+            look |= dn[u] <= near_d[u];
+          }
+          if (!look) continue;
+          const int cn = __float_as_int(f.w);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (!(dn[u] <= near_d[u])) continue;
+            if ((dn[u] < __fmul_rn(d[u], 0.99999f) && d[u] >= 1e-30f) ||
+                fps_key(x[u], y[u], z[u], X, cn) < fps_key(x[u], y[u], z[u], X, c[u])) {
+              d[u] = dn[u];
+              c[u] = cn;
+              // a point that coincides with a centre has nothing left to fold
+              if (dn[u] < 1e-30f && fps_key(x[u], y[u], z[u], X, cn) == 0ull) d[u] = -1.f;
+              near_d[u] = fps_near(d[u]);
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int p = q + u * kFpsT;
+          if (p < cnt) {
+            cur[p] = d[u];
+            near[p] = c[u];
+            if (d[u] > 0.f) fmax = max(fmax, __float_as_uint(d[u]));
           }
         }
       }
-      fps_pick(best, (unsigned long long)__double_as_longlong(c), p0 + p, x, y, z);
+      // ---- 2. a threshold that `top` half-warps' points reach (all when the
+      // block has fewer), widened so that rounding hides no point
+      {
+        const unsigned hm = __reduce_max_sync(lane < 16 ? 0xffffu : 0xffff0000u, fmax);
+        if (lane % 16 == 0) s_max[tid / 16] = hm;
+      }
+      __syncthreads();
+      float tau;
+      {
+        unsigned v = s_max[lane], m = 0;
+        for (int t = 0; t < min(top, 32); ++t) {
+          m = __reduce_max_sync(kFull, v);
+          const unsigned first = __ballot_sync(kFull, v == m);
+          if (lane == __ffs(first) - 1) v = 0;
+        }
+        tau = __fmul_rn(__uint_as_float(m), 0.999997f);
+        if (tau < 1e-30f) tau = -1.f;
+      }
+      // the thread's first two points at or above the threshold, exactly
+      FpsCand a{0ull, INT_MAX, 0.f, 0.f, 0.f, 0, 0};
+      unsigned long long k2 = 0ull;
+      int i2 = INT_MAX;
+      int left = 0;  // those beyond the two
+      auto scan = [&](unsigned long long lk, int li) {  // those after (lk, li)
+        left = -2;
+        a.key = k2 = 0ull;
+        a.idx = i2 = INT_MAX;
+        for (int p = tid; p < cnt; p += kFpsT) {
+          if (!(cur[p] >= tau)) continue;
+          const unsigned long long k = fps_key(xs[p], ys[p], zs[p], X, near[p]);
+          const int g = p0 + p;
+          if (!fps_before(lk, li, k, g)) continue;
+          ++left;
+          if (fps_before(k, g, a.key, a.idx)) {
+            k2 = a.key;
+            i2 = a.idx;
+            a.key = k;
+            a.idx = g;
+          } else if (fps_before(k, g, k2, i2)) {
+            k2 = k;
+            i2 = g;
+          }
+        }
+      };
+      if (__uint_as_float(fmax) >= tau && tid < cnt) scan(~0ull, -1);
+      FpsCand* mine = cand + ((size_t)(round & 1) * G + rank) * (top + 1);
+      int t = 0;
+      FpsCand w = fps_block_first(a, red, buf);
+      for (; t < top && w.idx != INT_MAX; ++t) {
+        if (w.idx == a.idx) {  // the owner publishes it and offers its next
+          const int p = a.idx - p0;
+          mine[t] = FpsCand{a.key, a.idx, xs[p], ys[p], zs[p], near[p], 0};
+          if (i2 != INT_MAX) {
+            a.key = k2;
+            a.idx = i2;
+            i2 = INT_MAX;
+          } else if (left > 0) {
+            scan(w.key, w.idx);
+          } else {
+            a.key = 0ull;
+            a.idx = INT_MAX;
+          }
+        }
+        w = fps_block_first(a, red, buf);
+      }
+      if (tid == 0) {
+        // the bound: the next point, or what a point below the threshold may reach
+        FpsCand r{0ull, -1, 0.f, 0.f, 0.f, 0, 0};
+        if (tau > 0.f) r.key = (unsigned long long)__double_as_longlong((double)tau * 1.000002);
+        mine[top] = w.idx != INT_MAX && fps_before(w.key, w.idx, r.key, r.idx) ? w : r;
+        for (; t < top; ++t) mine[t] = FpsCand{0ull, INT_MAX, 0.f, 0.f, 0.f, 0, 0};
+      }
+      // ---- 3.
+      if (!grid_barrier(bar, (unsigned)round * (unsigned)G, abort, flags)) break;
+      // the first of the bounds (L1 bypassed)
+      pool = cand + (size_t)(round & 1) * G * (top + 1);
+      FpsCand bound{0ull, INT_MAX, 0.f, 0.f, 0.f, 0, 0};
+      for (int q = tid; q < G; q += kFpsT) {
+        const FpsCand* c = pool + (size_t)q * (top + 1) + top;
+        const unsigned long long k = __ldcg(&c->key);
+        const int i = __ldcg(&c->idx);
+        if (fps_before(k, i, bound.key, bound.idx)) {
+          bound.key = k;
+          bound.idx = i;
+        }
+      }
+      bound = fps_block_first(bound, red, buf);
+      bkey = bound.key;
+      bidx = bound.idx;
     }
-    fps_warp_max(best);
-    if (lane == 0) red[wid] = best;
-    __syncthreads();
-    if (wid == 0) {
-      FpsCand b = red[lane];
-      fps_warp_max(b);
-      if (lane == 0) cand[(size_t)(j & 1) * G + rank] = b;
+    // ---- 4. choose among the published points
+    bool stop = false;
+    int taken = 0;
+    {
+      float x[2], y[2], z[2], d[2];  // d < 0: none, or at a chosen centre
+      int id[2], nr[2];
+      unsigned long long ek[2];  // exact distances, computed when asked for
+      auto exact = [&](int u) {
+        if (ek[u] == kNoKey) ek[u] = fps_key(x[u], y[u], z[u], X, nr[u]);
+        return ek[u];
+      };
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int e = tid + u * kFpsT;
+        id[u] = INT_MAX;
+        nr[u] = start;
+        d[u] = -1.f;
+        ek[u] = kNoKey;
+        x[u] = y[u] = z[u] = 0.f;
+        if (whole && e < cnt) {
+          id[u] = e;
+          x[u] = xs[e];
+          y[u] = ys[e];
+          z[u] = zs[e];
+          d[u] = d2_f32(x[u], y[u], z[u], fresh[0].x, fresh[0].y, fresh[0].z);
+          if (d[u] < 1e-30f && exact(u) == 0ull) d[u] = -1.f;
+        } else if (!whole && e < G * top) {
+          const FpsCand* c = pool + e / top * (top + 1) + e % top;
+          id[u] = __ldcg(&c->idx);
+          if (id[u] != INT_MAX) {
+            x[u] = __ldcg(&c->x);
+            y[u] = __ldcg(&c->y);
+            z[u] = __ldcg(&c->z);
+            nr[u] = __ldcg(&c->near);
+            ek[u] = __ldcg(&c->key);
+            d[u] = ek[u] ? (float)__longlong_as_double((long long)ek[u]) : -1.f;
+          }
+        }
+      }
+      // an FP32 distance above this lies above the bound for certain
+      const float over = (float)__longlong_as_double((long long)bkey) * 1.000002f;
+      while (j < K && (whole || taken < kFpsNew)) {
+        int b1 = -1, b2 = -1, bu = 0;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int v = d[u] >= 0.f ? __float_as_int(d[u]) : -1;
+          if (v > b1) {
+            b2 = b1;
+            b1 = v;
+            bu = u;
+          } else if (v > b2) {
+            b2 = v;
+          }
+        }
+        const int m1 = __reduce_max_sync(kFull, b1);
+        const int own = __ffs(__ballot_sync(kFull, b1 == m1)) - 1;
+        const int m2 = __reduce_max_sync(kFull, lane == own ? b2 : b1);
+        if (lane == own) {
+          FpsPick r{m1, m2, INT_MAX, 0, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            if (u == bu) {
+              r.idx = id[u];
+              r.x = x[u];
+              r.y = y[u];
+              r.z = z[u];
+            }
+          pick[pbuf][wid] = r;
+        }
+        __syncthreads();
+        FpsPick r = pick[pbuf][lane % (kFpsT / 32)];
+        pbuf ^= 1;
+        const int M = __reduce_max_sync(kFull, r.m1);
+        const int src = __ffs(__ballot_sync(kFull, r.m1 == M)) - 1;
+        if (M < 0) {  // every published point is at a chosen centre: so is every
+                      // other one when no bound is above zero
+          stop = bkey == 0ull;
+          break;
+        }
+        const float far = __int_as_float(M);
+        float near_far = __fmul_rn(far, 0.999997f);
+        if (far < 1e-30f) near_far = 0.f;
+        const int other = lane == src ? r.m2 : lane < kFpsT / 32 ? r.m1 : -1;
+        const bool close =
+            __any_sync(kFull, other >= 0 && __int_as_float(other) >= near_far);
+        int wi = __shfl_sync(kFull, r.idx, src);
+        float wx = __shfl_sync(kFull, r.x, src);
+        float wy = __shfl_sync(kFull, r.y, src);
+        float wz = __shfl_sync(kFull, r.z, src);
+        if (close || far < 1e-30f || (taken > 0 && !(far > over))) {
+          // too close to call in FP32: the exact order of the points near the top
+          FpsCand a{0ull, INT_MAX, 0.f, 0.f, 0.f, 0, 0};
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            if (d[u] >= near_far) {
+              const unsigned long long k = exact(u);
+              if (fps_before(k, id[u], a.key, a.idx)) a = FpsCand{k, id[u], x[u], y[u], z[u], 0, 0};
+            }
+          FpsCand w = a;
+          fps_warp_first(w.key, w.idx);
+          const unsigned has = __ballot_sync(kFull, a.key == w.key && a.idx == w.idx);
+          if (lane == __ffs(has) - 1) tie[tbuf][wid] = a;
+          __syncthreads();
+          a = tie[tbuf][lane % (kFpsT / 32)];
+          tbuf ^= 1;
+          w = a;
+          fps_warp_first(w.key, w.idx);
+          const int from = __ffs(__ballot_sync(kFull, a.key == w.key && a.idx == w.idx)) - 1;
+          wi = w.idx;
+          wx = __shfl_sync(kFull, a.x, from);
+          wy = __shfl_sync(kFull, a.y, from);
+          wz = __shfl_sync(kFull, a.z, from);
+          if (w.key == 0ull) {
+            // every published point coincides with a chosen centre: so does
+            // every other one when no bound is above zero
+            stop = bkey == 0ull;
+            break;
+          }
+          if (taken > 0 && !fps_before(w.key, w.idx, bkey, bidx)) break;
+        }
+        if (tid == 0) {
+          if (!whole) fresh[taken] = make_float4(wx, wy, wz, __int_as_float(wi));
+          if (rank == 0) chosen[j] = wi;
+        }
+        ++taken;
+        ++j;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float dn = d2_fma(x[u], y[u], z[u], wx, wy, wz);
+          if (id[u] == wi) {
+            d[u] = -1.f;
+          } else if (dn <= fps_near(d[u])) {
+            if ((dn < __fmul_rn(d[u], 0.99999f) && d[u] >= 1e-30f) ||
+                fps_key(x[u], y[u], z[u], X, wi) < exact(u)) {
+              d[u] = dn;
+              nr[u] = wi;
+              ek[u] = kNoKey;
+              if (dn < 1e-30f && exact(u) == 0ull) d[u] = -1.f;
+            }
+          }
+        }
+      }
     }
-    if (!grid_barrier(bar, (unsigned)j * (unsigned)G, abort, flags)) break;
-    // every block reduces all the published candidates (L1 bypassed)
-    FpsCand w{0ull, INT_MAX, 0.f, 0.f, 0.f, 0};
-    const FpsCand* cj = cand + (size_t)(j & 1) * G;
-    for (int q = tid; q < G; q += kFpsT) {
-      const unsigned long long key = __ldcg(reinterpret_cast<const unsigned long long*>(&cj[q].key));
-      const int idx = __ldcg(&cj[q].idx);
-      const float x = __ldcg(&cj[q].x), y = __ldcg(&cj[q].y), z = __ldcg(&cj[q].z);
-      fps_pick(w, key, idx, x, y, z);
-    }
-    fps_warp_max(w);
-    if (lane == 0) red[wid] = w;
-    __syncthreads();
-    if (wid == 0) {
-      FpsCand b = red[lane];
-      fps_warp_max(b);
-      if (lane == 0) s_win = b;
-    }
-    __syncthreads();
-    const FpsCand win = s_win;
-    if (win.key == 0ull || win.idx == INT_MAX) {
-      // every remaining point coincides with a chosen centre
+    nnew = taken;
+    if (stop) {
       if (rank == 0 && tid == 0 && atomicCAS(&flags->code, 0, (int)FF_ERR_INVALID_ARG) == 0)
         flags->index = j;
       break;
     }
-    if (rank == 0 && tid == 0) chosen[j] = win.idx;
-    cx = win.x;
-    cy = win.y;
-    cz = win.z;
-    __syncthreads();  // s_win and red are rewritten in the next step
+    __syncthreads();  // fresh is read by every thread next
   }
 }
 
@@ -723,71 +931,42 @@ void build_twoset(ff_ctx* c, const float* Xq, const float* vq, long long nq, int
   c->twoset = true;
   c->trunc = trunc;
 
-  // ---- 2. farthest-point sampling: on the whole GPU (cooperative launch, one
-  // block per SM) when the points are many, else on one thread-block cluster
+  // ---- 2. farthest-point sampling: one block per 1,024 points up to one per
+  // SM; the points the blocks publish a round fill the 1,024 places that are
+  // chosen among (at most 16 a block: each costs a block reduction)
   const int n = (int)nq;
   long long* chosen = reinterpret_cast<long long*>(c->centre_idx.ensure(sizeof(long long) * K));
   reset_flags(c);
-  bool done = false;
   {
     ProfScope ps(kProfFps);
     int coop = 0;
     FF_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
-    const int G = sm_count();
-    if (coop && n >= kFpsGridMin) {
-      const int S = (n + G - 1) / G;
-      const size_t smem = 24 * (size_t)S;
-      const bool in_smem = smem <= (size_t)kFpsSmemMax;
-      if (in_smem) set_max_dyn_smem((const void*)k_fps_grid, (int)std::max<size_t>(smem, 16));
-      int per_sm = 0;
-      FF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fps_grid, kFpsT,
-                                                            in_smem ? smem : 0));
-      if (per_sm >= 1) {
-        float* gxyz = nullptr;
-        double* gcur = nullptr;
-        float* gcur32 = nullptr;
-        if (!in_smem) {
-          gxyz = reinterpret_cast<float*>(c->scratch[1].ensure(sizeof(float) * 3 * (size_t)n));
-          gcur = reinterpret_cast<double*>(c->scratch[2].ensure(sizeof(double) * (size_t)n));
-          gcur32 = reinterpret_cast<float*>(c->scratch[4].ensure(sizeof(float) * (size_t)n));
-        }
-        // candidates (two buffers of G), then the barrier counter and the abort word
-        unsigned char* sync = reinterpret_cast<unsigned char*>(
-            c->scratch[7].ensure(2 * sizeof(FpsCand) * G + 64));
-        FpsCand* cand = reinterpret_cast<FpsCand*>(sync);
-        unsigned* bar = reinterpret_cast<unsigned*>(sync + 2 * sizeof(FpsCand) * G);
-        int* abort = reinterpret_cast<int*>(bar + 4);
-        FF_CUDA(cudaMemsetAsync(bar, 0, 32, st));
-        int nn = n, KK = K, st0 = (int)start, SS = S, ism = in_smem ? 1 : 0;
-        DevFlags* fl = c->flags.as<DevFlags>();
-        void* args[] = {(void*)&Xq, &nn, &KK, &st0, &SS, &ism, &gxyz, &gcur, &gcur32,
-                        &chosen, &cand, &bar, &abort, &fl};
-        FF_CUDA(cudaLaunchCooperativeKernel((const void*)k_fps_grid, dim3(G), dim3(kFpsT), args,
-                                            in_smem ? smem : 0, st));
-        ::ff::note_launch();
-        done = true;
-      }
+    FF_REQUIRE(coop, FF_ERR_CUDA, "the device has no cooperative launch");
+    int G = std::min(std::min(sm_count(), kPool), (n + kPool - 1) / kPool);
+    int S = (n + G - 1) / G, top = std::min(16, kPool / G);
+    const size_t smem = 20 * (size_t)S;
+    int in_smem = smem <= (size_t)kFpsSmemMax ? 1 : 0;
+    if (in_smem) set_max_dyn_smem((const void*)k_fps_rounds, (int)smem);
+    float* gslice = nullptr;
+    int* gnear = nullptr;
+    if (!in_smem) {
+      gslice = reinterpret_cast<float*>(c->scratch[1].ensure(16 * (size_t)S * G));
+      gnear = reinterpret_cast<int*>(c->scratch[2].ensure(sizeof(int) * (size_t)S * G));
     }
-    if (!done) {
-      const int S = (n + kFpsCS - 1) / kFpsCS;
-      const size_t smem = 24 * (size_t)S;
-      const bool in_smem = smem <= (size_t)kFpsSmemMax;
-      float* gxyz = nullptr;
-      double* gcur = nullptr;
-      float* gcur32 = nullptr;
-      if (in_smem) {
-        set_max_dyn_smem((const void*)k_fps, (int)std::max<size_t>(smem, 16));
-      } else {
-        gxyz = reinterpret_cast<float*>(c->scratch[1].ensure(sizeof(float) * 3 * (size_t)n));
-        gcur = reinterpret_cast<double*>(c->scratch[2].ensure(sizeof(double) * (size_t)n));
-        gcur32 = reinterpret_cast<float*>(c->scratch[4].ensure(sizeof(float) * (size_t)n));
-      }
-      (k_fps<<<kFpsCS, kFpsT, in_smem ? smem : 0, st>>>(Xq, n, K, (int)start, S,
-                                                        in_smem ? 1 : 0, gxyz, gcur, gcur32,
-                                                        chosen, c->flags.as<DevFlags>()),
-       ::ff::note_launch());
-      FF_LAUNCH_CHECK();
-    }
+    // two buffers of published points, then the barrier counter and the abort word
+    const size_t pool = 2 * sizeof(FpsCand) * (size_t)G * (top + 1);
+    unsigned char* sync = reinterpret_cast<unsigned char*>(c->scratch[7].ensure(pool + 64));
+    FpsCand* cand = reinterpret_cast<FpsCand*>(sync);
+    unsigned* bar = reinterpret_cast<unsigned*>(sync + pool);
+    int* abort = reinterpret_cast<int*>(bar + 4);
+    FF_CUDA(cudaMemsetAsync(bar, 0, 32, st));
+    int nn = n, KK = K, st0 = (int)start;
+    DevFlags* fl = c->flags.as<DevFlags>();
+    void* args[] = {(void*)&Xq, &nn,  &KK,     &st0,  &S,   &top,   &in_smem, &gslice,
+                    &gnear,     &chosen, &cand, &bar, &abort, &fl};
+    FF_CUDA(cudaLaunchCooperativeKernel((const void*)k_fps_rounds, dim3(G), dim3(kFpsT), args,
+                                        in_smem ? smem : 0, st));
+    ::ff::note_launch();
   }
   DevFlags f = read_flags(c);
   FF_REQUIRE(f.code != FF_ERR_TIMEOUT, FF_ERR_TIMEOUT,
