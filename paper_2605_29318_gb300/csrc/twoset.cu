@@ -25,7 +25,9 @@
 //   k_fps_rounds   up to one block per SM, each with its slice of the points;
 //                  several centres a grid barrier
 //   k_radii        one warp per centre: the two smallest squared distances
-//   k_cover_rows   one thread per point: its covering centres, ascending
+//   k_cover_bits, k_cover_fill
+//                  each point's covering centres as bits, then as an ascending
+//                  list (k_cover_rows, one thread per point, for many centres)
 //   k_cover_cols   one warp per centre: the points it covers, ascending, and
 //                  the centre's position in each point's row
 //   k_shape_twoset eight lanes per quadrature point, Eqs. 7, 9-10 with the Gaussian
@@ -670,6 +672,119 @@ __global__ void __launch_bounds__(256)
   if (!MODE && live) cnt[i] = c;
 }
 
+// The covering of kBitPts points a block as bits, word-major (bits[w][i]: centres
+// 32 w .. 32 w + 31 of point i), and the count of each point.  Two points a thread
+// share the reads of a staged centre; a pair inside the FP32 margin is settled in
+// FP64 after its word.  Bound by the tests' issue: 14 instructions a pair.  With
+// k_cover_fill it stands for two passes of k_cover_rows (0.67 + 0.97 ms for 1M
+// points and 1,000 centres): 0.36 + 0.23 ms.
+constexpr int kBitPts = 512;
+
+__global__ void __launch_bounds__(kBitPts / 2)
+    k_cover_bits(const float* __restrict__ Xq, long long nq, const float4* __restrict__ cpos,
+                 const float* __restrict__ lim32, const double* __restrict__ lim, int K,
+                 int* __restrict__ cnt, unsigned* __restrict__ bits) {
+  constexpr int T = kBitPts / 2;
+  __shared__ float4 sp[T];   // position, upper limit of the FP32 margin
+  __shared__ float slo[T];   // lower limit
+  const int tid = threadIdx.x;
+  long long i[2];
+  float x[2], y[2], z[2];
+  int c[2] = {0, 0};
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    i[u] = (long long)blockIdx.x * kBitPts + u * T + tid;
+    const long long r = min(i[u], nq - 1);
+    x[u] = Xq[3 * r];
+    y[u] = Xq[3 * r + 1];
+    z[u] = Xq[3 * r + 2];
+  }
+  for (int k0 = 0; k0 < K; k0 += T) {
+    __syncthreads();
+    {
+      const int k = k0 + tid;
+      float4 p = make_float4(0.f, 0.f, 0.f, -1.f);  // covers nothing
+      float lo = -1.f;
+      if (k < K) {
+        p = cpos[k];
+        const float l32 = lim32[k];
+        // tiny limits: every pair in FP64
+        p.w = l32 >= 1e-30f ? __fmul_rn(l32, 1.00001f) : INFINITY;
+        lo = l32 >= 1e-30f ? __fmul_rn(l32, 0.99999f) : -1.f;
+      }
+      sp[tid] = p;
+      slo[tid] = lo;
+    }
+    __syncthreads();
+    for (int w0 = 0; w0 < T && k0 + w0 < K; w0 += 32) {
+      unsigned in[2] = {0u, 0u}, near[2] = {0u, 0u};
+#pragma unroll
+      for (int q = 0; q < 32; ++q) {
+        const float4 p = sp[w0 + q];
+        const float lo = slo[w0 + q];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float d = d2_fma(x[u], y[u], z[u], p.x, p.y, p.z);
+          if (d < lo) in[u] |= 1u << q;
+          if (d <= p.w) near[u] |= 1u << q;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        for (unsigned b = near[u] & ~in[u]; b; b &= b - 1) {
+          const int q = __ffs(b) - 1;
+          const float4 p = sp[w0 + q];
+          if (d2_f64(x[u], y[u], z[u], p.x, p.y, p.z) < lim[k0 + w0 + q]) in[u] |= 1u << q;
+        }
+        c[u] += __popc(in[u]);
+        if (i[u] < nq) bits[(long long)((k0 + w0) >> 5) * nq + i[u]] = in[u];
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    if (i[u] < nq) cnt[i[u]] = c[u];
+}
+
+// The lists of 32 points a block from their bits: the words staged transposed in
+// shared memory, then a warp a point, a lane a word.
+__global__ void __launch_bounds__(256)
+    k_cover_fill(const unsigned* __restrict__ bits, long long nq, int words,
+                 const long long* __restrict__ rptr, int* __restrict__ ridx) {
+  __shared__ unsigned sb[32][33];
+  const long long i0 = (long long)blockIdx.x * 32;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  long long at[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const long long i = i0 + wid + 8 * u;
+    at[u] = i < nq ? rptr[i] : 0;
+  }
+  for (int w0 = 0; w0 < words; w0 += 32) {
+    if (w0) __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int w = w0 + wid + 8 * u;
+      sb[wid + 8 * u][lane] = w < words && i0 + lane < nq ? bits[(long long)w * nq + i0 + lane] : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      unsigned b = sb[lane][wid + 8 * u];
+      const int h = __popc(b);
+      int off = h;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, off, o);
+        if (lane >= o) off += t;
+      }
+      long long p = at[u] + off - h;
+      at[u] += __shfl_sync(kFull, off, 31);
+      for (; b; b &= b - 1) ridx[p++] = 32 * (w0 + lane) + __ffs(b) - 1;
+    }
+  }
+}
+
 // MODE 0: count the points each centre covers; MODE 1: list them (ascending)
 // with the position of the centre in each point's (ascending) row
 template <int MODE>
@@ -783,10 +898,27 @@ long long twoset_cover(ff_ctx* c, const float* Q, long long nq, Buf& ptrb, Buf& 
   cudaStream_t st = c->stream;
   const int K = (int)c->n;
   int* cnt = reinterpret_cast<int*>(cntb.ensure(sizeof(int) * (nq + 1)));
-  (k_cover_rows<0><<<ceil_div(nq, 256), 256, 0, st>>>(
-       Q, nq, c->pos.as<float4>(), c->clim32.as<float>(), c->clim.as<double>(), K, cnt, nullptr,
-       nullptr),
-   ::ff::note_launch());
+  // as bits between the two passes while they take less room than the lists
+  // (K / 8 bytes a point against 4 a pair, ~100 pairs) and 1 GB at most; else, or
+  // without that room, the tests run twice
+  const int words = (K + 31) / 32;
+  const size_t room = sizeof(unsigned) * (size_t)words * nq;
+  unsigned* bits = nullptr;
+  if (K <= 3200 && room <= (1ull << 30)) {
+    try {
+      bits = reinterpret_cast<unsigned*>(c->scratch[6].ensure(room));
+    } catch (const Error&) {
+    }
+  }
+  if (bits)
+    (k_cover_bits<<<ceil_div(nq, kBitPts), kBitPts / 2, 0, st>>>(
+         Q, nq, c->pos.as<float4>(), c->clim32.as<float>(), c->clim.as<double>(), K, cnt, bits),
+     ::ff::note_launch());
+  else
+    (k_cover_rows<0><<<ceil_div(nq, 256), 256, 0, st>>>(
+         Q, nq, c->pos.as<float4>(), c->clim32.as<float>(), c->clim.as<double>(), K, cnt, nullptr,
+         nullptr),
+     ::ff::note_launch());
   FF_LAUNCH_CHECK();
   long long* ptr = reinterpret_cast<long long*>(ptrb.ensure(sizeof(long long) * (nq + 1)));
   scan_counts(cnt, ptr, nq, c, c->scratch[3]);
@@ -794,10 +926,14 @@ long long twoset_cover(ff_ctx* c, const float* Q, long long nq, Buf& ptrb, Buf& 
   FF_CUDA(cudaMemcpyAsync(&n1, ptr + nq, sizeof(long long), cudaMemcpyDeviceToHost, st));
   FF_CUDA(cudaStreamSynchronize(st));
   int* idx = reinterpret_cast<int*>(idxb.ensure(sizeof(int) * std::max(n1, 1LL)));
-  (k_cover_rows<1><<<ceil_div(nq, 256), 256, 0, st>>>(
-       Q, nq, c->pos.as<float4>(), c->clim32.as<float>(), c->clim.as<double>(), K, nullptr, ptr,
-       idx),
-   ::ff::note_launch());
+  if (bits)
+    (k_cover_fill<<<ceil_div(nq, 32), 256, 0, st>>>(bits, nq, words, ptr, idx),
+     ::ff::note_launch());
+  else
+    (k_cover_rows<1><<<ceil_div(nq, 256), 256, 0, st>>>(
+         Q, nq, c->pos.as<float4>(), c->clim32.as<float>(), c->clim.as<double>(), K, nullptr, ptr,
+         idx),
+     ::ff::note_launch());
   FF_LAUNCH_CHECK();
   return n1;
 }

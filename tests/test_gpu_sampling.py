@@ -61,3 +61,20 @@ def test_as_many_centres_as_distinct_points(repeat):
     assert np.array_equal(ctx.twoset()[1], twoset.farthest_point_sampling(X, 40, 0))
     with pytest.raises(binding.FreeformError, match="step 40"):
         ctx.rkpm_build_twoset(Xd, v, 41, 0.0, 0)
+
+
+@pytest.mark.parametrize("n,K,trunc", [(513, 31, 3.0), (512, 32, 3.0), (777, 33, 3.0),
+                                       (1300, 256, 3.0), (1300, 257, 2.5), (600, 64, 0.0),
+                                       (1025, 1024, 3.0), (3400, 3201, 3.0)])
+def test_covering_lists_at_the_edges_of_their_words(n, K, trunc):
+    """Lists from the bits (K up to 3,200) and from the two passes beyond, pair
+    by pair the oracle's."""
+    import torch
+    from paper_2605_29318_gb300 import binding
+    X = _random(n, n + K).astype(np.float32)
+    ctx = binding.Context(0, "fp32")
+    ctx.rkpm_build_twoset(torch.from_numpy(X).cuda(), torch.ones(n, device="cuda"), K, trunc, 0)
+    _, cen, rad = ctx.twoset()
+    ptr, idx = twoset.covering(X, X[cen], rad, trunc or None)
+    got_ptr, got_idx, _, _ = ctx.export_rkpm()
+    assert np.array_equal(got_ptr, ptr) and np.array_equal(got_idx, idx)
