@@ -1,5 +1,6 @@
 // Assembly of the weight-space Hessian H_w (Prop. 1) and the RKPM mass matrix
-// (Sec. 3.2, Eq. 14) in CSR, one warp per matrix row.
+// (Sec. 3.2, Eq. 14) in CSR, one warp per matrix row (in tiles of neighbouring
+// rows where the cloud's lists fit, k_tile_rows).
 //
 //   (H_w)_kl = sum_i v_i (lambda_i + 4 mu_i) grad phi_k(X_i) . grad phi_l(X_i)
 //   M_kl     = sum_i v_i phi_k(X_i) phi_l(X_i)
@@ -15,6 +16,7 @@
 // accumulates the values.  The diagonal of H_w is replaced by minus the sum of
 // the off-diagonal entries of its row, which makes H_w 1 = 0 exact in storage
 // (the constant mode of Supp. Sec. B is an exact null vector).
+#include <climits>
 #include <type_traits>
 
 #include "ff_internal.cuh"
@@ -231,6 +233,370 @@ size_t assemble_smem_per_warp(int tsize, int maxrow, size_t tbytes) {
   return (t + 15) & ~size_t(15);
 }
 
+// ------------------------------------------------------------------ tiles of rows
+// The same sums for the rows of a spatially sorted cloud, kTileRows consecutive
+// rows a block.  Neighbouring rows share most of their points and columns, so
+// the block first lists, once for all its rows,
+//   * the union of the points its nodes cover (a hash table: point -> local
+//     number), and
+//   * the union of those points' nodes (a hash table, then sorted: the rank of
+//     a column), with the rank of every entry of every point's list (`lr`);
+// each warp then takes rows: the ranks its points' entries mark become places in
+// the row, and it walks the points in ascending order as the row-owner pass does
+// (the same sums), a pair costing two 16-bit reads for its place where that pass
+// hashes the column twice.  The next point's table values are loaded
+// while the current ones are added.  Bound by issue and the latency of the
+// accumulators in shared memory, at two blocks an SM.  The row-owner pass took 1.81 +
+// 14.4 ms (count, values) for 200k particles in FP32, this 1.11 + 3.39 ms; in
+// double-float (50k) 0.48 + 4.07 ms, this 0.29 + 1.09 ms.
+// MODE 0 counts the rows' columns and reports the largest tile; MODE 1 writes
+// columns and values, its tables sized by that.
+constexpr int kTileRows = 16, kTileT = 256, kTileWarps = kTileT / 32;
+
+struct TileDims {
+  int pts, cols, pairs, row;  // capacities: points, columns and list entries of a
+                              // tile, columns of a row
+  int ptab, ctab;             // hash slots
+};
+struct TileMax {
+  int over, pts, cols, pairs, row;
+};
+constexpr TileDims kTileCap{512, 1536, 20480, 1536, 1024, 4096};
+
+// shared memory of a tile: what lasts (points, list entries, sorted columns),
+// then the column table, later the warps' rows
+struct TileSmem {
+  int ptab, plist, poff, scols, pid, lr, ctab, cid, cols, warp, per_warp, loc, total;
+  __host__ __device__ TileSmem(const TileDims& d, int mode, int tbytes) {
+    int at = 0;
+    auto take = [&](int bytes) {
+      const int o = at;
+      at += (bytes + 15) & ~15;
+      return o;
+    };
+    ptab = take(4 * d.ptab);
+    plist = take(4 * d.pts);
+    poff = take(4 * (d.pts + 1));
+    int room = 2;  // the sort's, a power of two
+    while (room < d.cols) room <<= 1;
+    scols = take(mode ? 4 * room : 0);
+    pid = take(2 * d.ptab);
+    lr = take(2 * d.pairs);
+    const int shared_from = at;
+    ctab = take(4 * d.ctab);
+    cid = take(2 * d.ctab);
+    cols = take(mode ? 4 * d.cols : 0);
+    const int tables = at;
+    // a warp: loc (MODE 0: marks), then the sums of H and M
+    loc = 0;
+    per_warp = mode ? ((2 * d.cols + 15) & ~15) + ((2 * d.row * tbytes + 15) & ~15)
+                    : (d.cols + 15) & ~15;
+    // MODE 0 marks while its table is dead too
+    warp = shared_from;
+    total = shared_from + per_warp * kTileWarps;
+    if (total < tables) total = tables;
+  }
+};
+
+template <int MODE, class T, class TO>
+__global__ void __launch_bounds__(kTileT, 2)
+    k_tile_rows(const long long* __restrict__ ptr, const int* __restrict__ idx,
+                const long long* __restrict__ tptr, const int* __restrict__ tidx,
+                const long long* __restrict__ tpos, const T* __restrict__ phi,
+                const T* __restrict__ dphi, long long n1, const float* __restrict__ vol,
+                const T* __restrict__ wh, long long n, TileDims dims, int* __restrict__ cnt,
+                TileMax* __restrict__ tmax, const long long* __restrict__ aptr,
+                int* __restrict__ acol, TO* __restrict__ aval, float* __restrict__ hf32,
+                float* __restrict__ hdiag) {
+  constexpr unsigned kAll = 0xffffffffu;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  __shared__ int s_np, s_nc, s_tot, s_over;
+  const TileSmem L(dims, MODE, (int)sizeof(T));
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const unsigned below = (1u << lane) - 1;
+  const long long k0 = (long long)blockIdx.x * kTileRows;
+  const long long k1 = min(k0 + kTileRows, n);
+  int* ptab = reinterpret_cast<int*>(sm_raw + L.ptab);
+  int* plist = reinterpret_cast<int*>(sm_raw + L.plist);
+  int* poff = reinterpret_cast<int*>(sm_raw + L.poff);
+  int* scols = reinterpret_cast<int*>(sm_raw + L.scols);
+  unsigned short* pid = reinterpret_cast<unsigned short*>(sm_raw + L.pid);
+  unsigned short* lr = reinterpret_cast<unsigned short*>(sm_raw + L.lr);
+  int* ctab = reinterpret_cast<int*>(sm_raw + L.ctab);
+  unsigned short* cid = reinterpret_cast<unsigned short*>(sm_raw + L.cid);
+  int* cols = reinterpret_cast<int*>(sm_raw + L.cols);
+  for (int q = tid; q < dims.ptab; q += kTileT) ptab[q] = kEmpty;
+  for (int q = tid; q < dims.ctab; q += kTileT) ctab[q] = kEmpty;
+  if (tid == 0) s_np = s_nc = s_tot = s_over = 0;
+  __syncthreads();
+  // ---- the tile's points, numbered as they are found
+  const long long a_end = tptr[k1];
+  for (long long a = tptr[k0] + tid; a < a_end; a += kTileT) {
+    if (*(volatile int*)&s_np > dims.pts) break;
+    bool fresh;
+    const int i = tidx[a];
+    const int slot = hset_insert(ptab, dims.ptab, i, fresh);
+    if (fresh) {
+      const int q = atomicAdd(&s_np, 1);
+      if (q < dims.pts) {
+        plist[q] = i;
+        pid[slot] = (unsigned short)q;
+      }
+    }
+  }
+  __syncthreads();
+  const int np = s_np;
+  bool over = np > dims.pts;
+  if (!over)
+    for (int p = tid; p < np; p += kTileT) {
+      const int i = plist[p];
+      poff[p] = atomicAdd(&s_tot, (int)(ptr[i + 1] - ptr[i]));
+    }
+  __syncthreads();
+  over = over || s_tot > dims.pairs;
+  // ---- their nodes: every list entry's slot in the column table (a warp a
+  // point; the entries of four points are loaded before they are inserted)
+  if (!over) {
+    for (int p0 = wid * 4; p0 < np; p0 += kTileWarps * 4) {
+      if (__any_sync(kAll, *(volatile int*)&s_nc > dims.cols)) break;
+      int key[4][2], len[4];
+      long long s[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = p0 + u < np ? plist[p0 + u] : -1;
+        s[u] = i >= 0 ? ptr[i] : 0;
+        len[u] = i >= 0 ? (int)(ptr[i + 1] - s[u]) : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+          key[u][v] = lane + 32 * v < len[u] ? idx[s[u] + lane + 32 * v] : -1;
+      auto put = [&](int c, int at) {  // every lane takes part
+        bool fresh = false;
+        int slot = 0;
+        if (c >= 0) {
+          slot = hset_insert(ctab, dims.ctab, c, fresh);
+          if (slot < 0) s_over = 1;
+          lr[at] = (unsigned short)slot;
+        }
+        const unsigned f = __ballot_sync(kAll, fresh);
+        if (f) {
+          int q = 0;
+          if (lane == 0) q = atomicAdd(&s_nc, __popc(f));
+          q = __shfl_sync(kAll, q, 0) + __popc(f & below);
+          if (fresh && q < dims.cols) {
+            cid[slot] = (unsigned short)q;
+            if (MODE) cols[q] = c;
+          }
+        }
+      };
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (p0 + u >= np || __any_sync(kAll, *(volatile int*)&s_nc > dims.cols)) break;
+        const int o = poff[p0 + u];
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+          if (32 * v < len[u]) put(key[u][v], o + lane + 32 * v);
+        for (int t0 = 64; t0 < len[u] && !__any_sync(kAll, *(volatile int*)&s_nc > dims.cols);
+             t0 += 32) {
+          const int t = t0 + lane;
+          put(t < len[u] ? idx[s[u] + t] : -1, o + t);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  const int nc = s_nc, tot = s_tot;
+  over = over || s_over || nc > dims.cols;
+  if (MODE == 0 && tid == 0) {
+    if (over) tmax->over = 1;
+    atomicMax(&tmax->pts, np);
+    atomicMax(&tmax->cols, nc);
+    atomicMax(&tmax->pairs, tot);
+  }
+  if (over) return;
+  if (MODE) {  // the columns in order (bitonic): a number becomes a rank
+    const int pow2 = 1 << (32 - __clz(max(nc - 1, 1)));
+    for (int q = tid; q < pow2; q += kTileT) scols[q] = q < nc ? cols[q] : INT_MAX;
+    __syncthreads();
+    for (int size = 2; size <= pow2; size <<= 1)
+      for (int step = size >> 1; step; step >>= 1) {
+        for (int q = tid; q < pow2 / 2; q += kTileT) {
+          const int lo = 2 * q - (q & (step - 1)), hi = lo + step;
+          const int x = scols[lo], y = scols[hi];
+          if ((x > y) == ((lo & size) == 0)) {
+            scols[lo] = y;
+            scols[hi] = x;
+          }
+        }
+        __syncthreads();
+      }
+    for (int r = tid; r < nc; r += kTileT)
+      cid[hset_find(ctab, dims.ctab, scols[r])] = (unsigned short)r;
+    __syncthreads();
+  }
+  for (int q = tid; q < tot; q += kTileT) lr[q] = cid[lr[q]];
+  __syncthreads();
+  // ---- the rows, a warp each
+  unsigned char* mine = sm_raw + L.warp + (size_t)wid * L.per_warp;
+  unsigned short* loc = reinterpret_cast<unsigned short*>(mine);
+  struct __align__(2 * sizeof(T)) Sums {
+    T h, m;
+  };
+  Sums* sums = reinterpret_cast<Sums*>(mine + (((size_t)2 * dims.cols + 15) & ~size_t(15)));
+  const int words = MODE ? (nc + 1) / 2 : (nc + 3) / 4;  // of the marks
+  for (long long k = k0 + wid; k < k1; k += kTileWarps) {
+    for (int w = lane; w < words; w += 32) reinterpret_cast<unsigned*>(mine)[w] = 0u;
+    __syncwarp();
+    const long long as = tptr[k];
+    const int np_row = (int)(tptr[k + 1] - as);
+    // the row's columns: the entries of its points marked
+    for (int a0 = 0; a0 < np_row; a0 += 32) {
+      const int here = min(32, np_row - a0);
+      int off = 0, len = 0;
+      if (lane < here) {
+        const int i = tidx[as + a0 + lane];
+        off = poff[pid[hset_find(ptab, dims.ptab, i)]];
+        len = (int)(ptr[i + 1] - ptr[i]);
+      }
+      for (int u = 0; u < here; ++u) {
+        const int o = __shfl_sync(kAll, off, u), e = __shfl_sync(kAll, len, u);
+        for (int t = lane; t < e; t += 32) {
+          const int r = lr[o + t];
+          if (MODE)
+            loc[r] = 1;
+          else
+            mine[r] = 1;
+        }
+      }
+    }
+    __syncwarp();
+    if constexpr (MODE == 0) {
+      int c = 0;
+      for (int w = lane; w < words; w += 32) c += __popc(reinterpret_cast<unsigned*>(mine)[w]);
+      c = __reduce_add_sync(kAll, c);
+      if (lane == 0) {
+        cnt[k] = c;
+        if (c > *(volatile int*)&tmax->row) atomicMax(&tmax->row, c);
+      }
+    } else {
+      // a rank becomes a place in the row
+      const long long at = aptr[k];
+      int m = 0, diag = -1;
+      for (int r0 = 0; r0 < nc; r0 += 32) {
+        const int r = r0 + lane;
+        const bool in = r < nc && loc[r];
+        const unsigned bal = __ballot_sync(kAll, in);
+        if (in) {
+          const int q = m + __popc(bal & below);
+          const int c = scols[r];
+          loc[r] = (unsigned short)q;
+          acol[at + q] = c;
+          if (c == (int)k) diag = q;
+        }
+        m += __popc(bal);
+      }
+      diag = __reduce_max_sync(kAll, diag);
+      for (int q = lane; q < m; q += 32) sums[q] = Sums{T(0), T(0)};
+      __syncwarp();
+      // the sums over the row's points, ascending
+      for (int a0 = 0; a0 < np_row; a0 += 32) {
+        const int here = min(32, np_row - a0);
+        // a lane a point: its list and the row's weighted values there
+        int off = 0, len = 0;
+        long long s = 0;
+        T h0(0), h1(0), h2(0), hm(0);
+        if (lane < here) {
+          const int i = tidx[as + a0 + lane];
+          off = poff[pid[hset_find(ptab, dims.ptab, i)]];
+          s = ptr[i];
+          len = (int)(ptr[i + 1] - s);
+          const long long e = tpos[as + a0 + lane];
+          const T w = wh[i];
+          h0 = w * dphi[e];
+          h1 = w * dphi[n1 + e];
+          h2 = w * dphi[2 * n1 + e];
+          hm = (T)vol[i] * phi[e];
+        }
+        // two entries a lane of the next point are in flight; longer lists take
+        // the rest in a loop
+        T g[2][4];
+        int rk[2], nlen = 0, noff = 0;
+        long long ns = 0;
+        auto load = [&](int u) {
+          nlen = __shfl_sync(kAll, len, u);
+          ns = __shfl_sync(kAll, s, u);
+          noff = __shfl_sync(kAll, off, u);
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            const int t = lane + 32 * v;
+            rk[v] = -1;
+            if (t < nlen) {
+              const long long e = ns + t;
+              rk[v] = loc[lr[noff + t]];
+              g[v][0] = dphi[e];
+              g[v][1] = dphi[n1 + e];
+              g[v][2] = dphi[2 * n1 + e];
+              g[v][3] = phi[e];
+            }
+          }
+        };
+        load(0);
+        for (int u = 0; u < here; ++u) {
+          const T c0 = __shfl_sync(kAll, h0, u), c1 = __shfl_sync(kAll, h1, u),
+                  c2 = __shfl_sync(kAll, h2, u), cm = __shfl_sync(kAll, hm, u);
+          const int mylen = nlen, myoff = noff;
+          const long long mys = ns;
+          T q[2][4];
+          int r2[2];
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            r2[v] = rk[v];
+#pragma unroll
+            for (int d = 0; d < 4; ++d) q[v][d] = g[v][d];
+          }
+          if (u + 1 < here) load(u + 1);
+          auto add = [&](int r, T x0, T x1, T x2, T xm) {
+            Sums z = sums[r];
+            if constexpr (std::is_same_v<T, dfloat>) {  // unnormalised, finished below
+              df_mac(z.h, c0, x0);
+              df_mac(z.h, c1, x1);
+              df_mac(z.h, c2, x2);
+              df_mac(z.m, cm, xm);
+            } else {
+              z.h += c0 * x0 + c1 * x1 + c2 * x2;
+              z.m += cm * xm;
+            }
+            sums[r] = z;
+          };
+#pragma unroll
+          for (int v = 0; v < 2; ++v)
+            if (r2[v] >= 0) add(r2[v], q[v][0], q[v][1], q[v][2], q[v][3]);
+          for (int t = lane + 64; t < mylen; t += 32) {
+            const long long e = mys + t;
+            add(loc[lr[myoff + t]], dphi[e], dphi[n1 + e], dphi[2 * n1 + e], phi[e]);
+          }
+          __syncwarp();
+        }
+      }
+      T sum(0);
+      for (int q = lane; q < m; q += 32)
+        if (q != diag) sum += finish(sums[q].h);
+#pragma unroll
+      for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(kAll, sum, o);
+      for (int q = lane; q < m; q += 32) {
+        const TO h = q == diag ? (TO)(-sum) : (TO)finish(sums[q].h);
+        aval[2 * (at + q)] = h;
+        aval[2 * (at + q) + 1] = (TO)finish(sums[q].m);
+        hf32[at + q] = (float)h;
+      }
+      if (lane == 0) hdiag[k] = (float)(TO)(-sum);
+    }
+    __syncwarp();
+  }
+}
+
 __global__ void k_round_f32(const double* __restrict__ x, float* __restrict__ y, long long m) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < m) y[t] = (float)x[t];
@@ -307,79 +673,112 @@ void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, doubl
     finish_matrices(c);
     return;
   }
-  // pass 1: unique columns per row, in a table of 2048 slots per warp (4 warps
-  // per block); clouds of uneven density (wide supports reaching into dense
-  // regions) retry with 16384 slots per warp (2 warps per block)
   int* cnt = reinterpret_cast<int*>(c->scratch[5].ensure(sizeof(int) * (n + 1)));
-  int tsize1 = 2048;
+  const long long* ptr = c->nbr_ptr.as<long long>();
+  const int* idx = c->nbr_idx.as<int>();
+  const long long* tptr = c->nbrT_ptr.as<long long>();
+  const int* tidx = c->nbrT_idx.as<int>();
+  const long long* tpos = c->nbrT_pos.as<long long>();
+  const float* vol = c->vol.as<float>();
   ProfScope ps_pattern(kProfPattern);
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    tsize1 = attempt == 0 ? 2048 : 16384;
+  // nodal clouds in tiles of rows; a tile beyond kTileCap (wide supports, clouds
+  // of very uneven density) sends the whole cloud to the row-owner passes below
+  TileMax tmax{1, 0, 0, 0, 0};
+  if (!c->twoset) {
+    TileMax* dmax = reinterpret_cast<TileMax*>(c->scratch[6].ensure(sizeof(TileMax)));
+    FF_CUDA(cudaMemsetAsync(dmax, 0, sizeof(TileMax), st));
+    const int smem = TileSmem(kTileCap, 0, 4).total;
+    set_max_dyn_smem((const void*)k_tile_rows<0, float, float>, smem);
+    (k_tile_rows<0, float, float><<<ceil_div(n, kTileRows), kTileT, smem, st>>>(
+         ptr, idx, tptr, tidx, tpos, nullptr, nullptr, n1, vol, nullptr, n, kTileCap, cnt, dmax,
+         nullptr, nullptr, nullptr, nullptr, nullptr),
+     ::ff::note_launch());
+    FF_LAUNCH_CHECK();
+    FF_CUDA(cudaMemcpyAsync(&tmax, dmax, sizeof(TileMax), cudaMemcpyDeviceToHost, st));
+    f = read_flags(c);
+    if (f.code == FF_ERR_INVALID_ARG)
+      throw Error(FF_ERR_INVALID_ARG, "invalid material (need E > 0, 0 <= nu < 0.5) at point " +
+                                          std::to_string(f.index));
+  }
+  const bool tiles = !tmax.over;
+  // row-owner pass 1: unique columns per row, in a table of 2048 slots per warp
+  // (4 warps per block); clouds of uneven density (wide supports reaching into
+  // dense regions) retry with 16384 slots per warp (2 warps per block)
+  for (int attempt = 0; !tiles && attempt < 2; ++attempt) {
+    const int tsize1 = attempt == 0 ? 2048 : 16384;
     const int wpb1 = attempt == 0 ? 4 : 2;
     const size_t smem1 = sizeof(int) * tsize1 * wpb1;
     if (smem1 > 48 * 1024) set_max_dyn_smem((const void*)k_pattern_count, (int)smem1);
     if (attempt > 0) reset_flags(c);
     int grid1 = (int)std::min<long long>(ceil_div(n, wpb1), (long long)sm_count() * 16);
-    (k_pattern_count<<<grid1, 32 * wpb1, smem1, st>>>(
-        c->nbr_ptr.as<long long>(), c->nbr_idx.as<int>(), c->nbrT_ptr.as<long long>(),
-        c->nbrT_idx.as<int>(), n, tsize1, cnt, c->flags.as<DevFlags>()), ::ff::note_launch());
+    (k_pattern_count<<<grid1, 32 * wpb1, smem1, st>>>(ptr, idx, tptr, tidx, n, tsize1, cnt,
+                                                     c->flags.as<DevFlags>()),
+     ::ff::note_launch());
     FF_LAUNCH_CHECK();
     f = read_flags(c);
     const bool overflow =
         f.code == FF_ERR_INVALID_ARG && f.max_row > 0 && f.max_row * 2 > tsize1;
     if (!overflow) break;
+    if (attempt == 1)
+      throw Error(FF_ERR_INVALID_ARG, "a Hessian row has more than " + std::to_string(tsize1 / 2) +
+                                          " distinct columns (support too large)");
   }
   ps_pattern.close();
-  if (f.code == FF_ERR_INVALID_ARG) {
-    throw Error(FF_ERR_INVALID_ARG,
-                f.max_row > 0 && f.max_row * 2 > tsize1
-                    ? "a Hessian row has more than " + std::to_string(tsize1 / 2) +
-                          " distinct columns (support too large)"
-                    : "invalid material (need E > 0, 0 <= nu < 0.5) at point " +
-                          std::to_string(f.index));
-  }
-  const int maxrow = std::max(f.max_row, 1);
+  if (f.code == FF_ERR_INVALID_ARG)
+    throw Error(FF_ERR_INVALID_ARG, "invalid material (need E > 0, 0 <= nu < 0.5) at point " +
+                                        std::to_string(f.index));
   long long* aptr = reinterpret_cast<long long*>(c->a_ptr.ensure(sizeof(long long) * (n + 1)));
   scan_counts(cnt, aptr, n, c, c->scratch[3]);
   long long n2 = 0;
   FF_CUDA(cudaMemcpyAsync(&n2, aptr + n, sizeof(long long), cudaMemcpyDeviceToHost, st));
   FF_CUDA(cudaStreamSynchronize(st));
   c->n2 = n2;
-  c->a_col.ensure(sizeof(int) * n2);
+  int* acol = reinterpret_cast<int*>(c->a_col.ensure(sizeof(int) * n2));
   c->a_val.ensure(2 * tb * n2);
-  c->h_f32.ensure(sizeof(float) * n2);
-  c->hdiag_f32.ensure(sizeof(float) * n);
-  int tsize2 = 64;
-  while (tsize2 < 2 * maxrow) tsize2 <<= 1;
-  size_t pw = assemble_smem_per_warp(tsize2, maxrow, tdf ? 8 : 4);
-  int wpb2 = (int)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / pw));
-  size_t smem = pw * wpb2;
-  int grid2 = (int)std::min<long long>(ceil_div(n, wpb2), (long long)sm_count() * 32);
+  float* hf32 = reinterpret_cast<float*>(c->h_f32.ensure(sizeof(float) * n2));
+  float* hdiag = reinterpret_cast<float*>(c->hdiag_f32.ensure(sizeof(float) * n));
   ProfScope ps_values(kProfAsmValues);
-  if (f64 && !tdf) {  // FP32 tables and sums, FP64 storage
-    set_max_dyn_smem((const void*)k_assemble<float, double>,
-                     (int)std::max<size_t>(smem, 48 * 1024));
-    (k_assemble<float, double><<<grid2, 32 * wpb2, smem, st>>>(
-        c->nbr_ptr.as<long long>(), c->nbr_idx.as<int>(), c->nbrT_ptr.as<long long>(),
-        c->nbrT_idx.as<int>(), c->nbrT_pos.as<long long>(), c->phi.as<float>(),
-        c->dphi.as<float>(), n1, c->vol.as<float>(), c->wh.as<float>(), n, tsize2, maxrow, aptr,
-        c->a_col.as<int>(), c->a_val.as<double>(), c->h_f32.as<float>(), c->hdiag_f32.as<float>()), ::ff::note_launch());
-  } else if (f64) {
-    set_max_dyn_smem((const void*)k_assemble<dfloat, double>,
-                     (int)std::max<size_t>(smem, 48 * 1024));
-    (k_assemble<dfloat, double><<<grid2, 32 * wpb2, smem, st>>>(
-        c->nbr_ptr.as<long long>(), c->nbr_idx.as<int>(), c->nbrT_ptr.as<long long>(),
-        c->nbrT_idx.as<int>(), c->nbrT_pos.as<long long>(), c->phi.as<dfloat>(),
-        c->dphi.as<dfloat>(), n1, c->vol.as<float>(), c->wh.as<dfloat>(), n, tsize2, maxrow, aptr,
-        c->a_col.as<int>(), c->a_val.as<double>(), c->h_f32.as<float>(), c->hdiag_f32.as<float>()), ::ff::note_launch());
-  } else {
-    set_max_dyn_smem((const void*)k_assemble<float>, (int)std::max<size_t>(smem, 48 * 1024));
-    (k_assemble<float><<<grid2, 32 * wpb2, smem, st>>>(
-        c->nbr_ptr.as<long long>(), c->nbr_idx.as<int>(), c->nbrT_ptr.as<long long>(),
-        c->nbrT_idx.as<int>(), c->nbrT_pos.as<long long>(), c->phi.as<float>(),
-        c->dphi.as<float>(), n1, c->vol.as<float>(), c->wh.as<float>(), n, tsize2, maxrow, aptr,
-        c->a_col.as<int>(), c->a_val.as<float>(), c->h_f32.as<float>(), c->hdiag_f32.as<float>()), ::ff::note_launch());
-  }
+  auto values = [&](auto ttag, auto totag) {
+    using TT = decltype(ttag);
+    using TO = decltype(totag);
+    const TT *phi = c->phi.as<TT>(), *dphi = c->dphi.as<TT>(), *wh = c->wh.as<TT>();
+    TO* aval = c->a_val.as<TO>();
+    if (tiles) {
+      auto slots = [](int m) {
+        int t = 64;
+        while (t < 2 * m) t <<= 1;
+        return t;
+      };
+      auto up = [](int m) { return (m + 7) & ~7; };
+      const TileDims d{up(tmax.pts), up(tmax.cols), up(tmax.pairs), up(tmax.row),
+                       slots(tmax.pts), slots(tmax.cols)};
+      const int smem = TileSmem(d, 1, (int)sizeof(TT)).total;
+      set_max_dyn_smem((const void*)k_tile_rows<1, TT, TO>, smem);
+      (k_tile_rows<1, TT, TO><<<ceil_div(n, kTileRows), kTileT, smem, st>>>(
+           ptr, idx, tptr, tidx, tpos, phi, dphi, n1, vol, wh, n, d, nullptr, nullptr, aptr, acol,
+           aval, hf32, hdiag),
+       ::ff::note_launch());
+      return;
+    }
+    const int maxrow = std::max(f.max_row, 1);
+    int tsize2 = 64;
+    while (tsize2 < 2 * maxrow) tsize2 <<= 1;
+    const size_t pw = assemble_smem_per_warp(tsize2, maxrow, sizeof(TT));
+    const int wpb2 = (int)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / pw));
+    const size_t smem = pw * wpb2;
+    const int grid2 = (int)std::min<long long>(ceil_div(n, wpb2), (long long)sm_count() * 32);
+    set_max_dyn_smem((const void*)k_assemble<TT, TO>, (int)std::max<size_t>(smem, 48 * 1024));
+    (k_assemble<TT, TO><<<grid2, 32 * wpb2, smem, st>>>(ptr, idx, tptr, tidx, tpos, phi, dphi, n1,
+                                                       vol, wh, n, tsize2, maxrow, aptr, acol,
+                                                       aval, hf32, hdiag),
+     ::ff::note_launch());
+  };
+  if (f64 && !tdf)  // FP32 tables and sums, FP64 storage
+    values(float{}, double{});
+  else if (f64)
+    values(dfloat{}, double{});
+  else
+    values(float{}, float{});
   FF_LAUNCH_CHECK();
   ps_values.close();
   finish_matrices(c);
