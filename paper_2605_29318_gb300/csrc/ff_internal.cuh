@@ -137,8 +137,8 @@ struct ff_ctx {
 
   ff::Grid grid{};
   // particles in internal (cell) order
-  // (two-set: the centres in their farthest-point order, pos.w = 1 / r_k^2; the
-  // radii are kept in FP64 in crad)
+  // (two-set: the centres in their farthest-point order, pos.w = the square of
+  // r_k's FP32 rounding; the radii are kept in FP64 in crad)
   ff::Buf perm;      // int[n]   internal -> caller index
   ff::Buf iperm;     // int[n]   caller -> internal index
   ff::Buf pos;       // float4[n] (x, y, z, a)
@@ -147,7 +147,7 @@ struct ff_ctx {
   // two-set centres
   ff::Buf centre_idx;// int64[K]  quadrature point chosen as centre k
   ff::Buf crad;      // double[K] r_k
-  ff::Buf cinv;      // dfloat[K] 1 / r_k^2 (its FP32 rounding: pos.w)
+  ff::Buf cinv;      // dfloat[K] 1 / r_k^2
   ff::Buf clim;      // double[K] t^2 r_k^2 (+inf untruncated)
   ff::Buf clim32;    // float[K]  its FP32 rounding (filter)
   ff::Buf qpts;      // float[3 nq] the quadrature points (x, y, z), caller order

@@ -46,35 +46,37 @@ __device__ __forceinline__ double gauss_exp(double x) { return exp(x); }
 __device__ __forceinline__ dfloat gauss_exp(dfloat x) { return df_exp(x); }
 
 // Gauss: exp(-|X - p_k|^2 / r_k^2) (Sec. 3.2) with the FP64 radii r_k of the
-// two-set construction; grad_X = (2 w / r_k^2)(p_k - X).  FP32 and double-float
-// take 1 / r_k^2 rounded once from FP64 per centre (p.w, inv): a multiplication
-// where the radius would cost two conversions from FP64, a square and a
-// division a pair.  In double-float the exponential is df_exp (reduction by
-// ln 2 and a Taylor polynomial on the FP32 pipes).
+// two-set construction; grad_X = (2 w / r_k^2)(p_k - X).  FP32 takes the square
+// of the rounded radius (p.w), double-float 1 / r_k^2 rounded from FP64 (inv),
+// once per centre: where the radius would cost two conversions from FP64 and more
+// a pair.  In double-float the exponential is df_exp (reduction by ln 2 and a
+// Taylor polynomial on the FP32 pipes).
 struct Gauss {
   static constexpr bool kStash = true;
   const double* rad;
   const dfloat* inv;
   template <class C>
-  __device__ __forceinline__ C inv_r2(int k, float4 p) const {
+  __device__ __forceinline__ C slope(int k, float4 p, C w) const {
     if constexpr (sizeof(C) == 4) {
-      return p.w;
+      return C(2) * w / p.w;
     } else if constexpr (std::is_same_v<C, dfloat>) {
-      return inv[k];
+      return C(2) * w * inv[k];
     } else {
       const double rk = rad[k];
-      return 1.0 / (rk * rk);
+      return 2.0 * w / (rk * rk);
     }
   }
   template <class C>
-  __device__ __forceinline__ C slope(int k, float4 p, C w) const {
-    return C(2) * w * inv_r2<C>(k, p);
-  }
-  template <class C>
   __device__ __forceinline__ void eval(int k, float4 p, C d2, C& w, C& gs) const {
-    const C iv = inv_r2<C>(k, p);
-    w = gauss_exp(-(d2 * iv));
-    gs = C(2) * w * iv;
+    if constexpr (sizeof(C) == 4) {
+      w = gauss_exp(-(d2 / p.w));
+    } else if constexpr (std::is_same_v<C, dfloat>) {
+      w = gauss_exp(-(d2 * inv[k]));
+    } else {
+      const double rk = rad[k];
+      w = gauss_exp(-(d2 / (rk * rk)));
+    }
+    gs = slope<C>(k, p, w);
   }
 };
 
@@ -262,6 +264,188 @@ __device__ __forceinline__ int shape_rows(const float4* __restrict__ pos, long l
       for (int a = 1; a < 4; ++a) mac(PdC, P[a], dC[d][a]);
       PdC = finish(PdC);
       dphi[d * n1 + t] = (T)(g[d] * PC + w * PdC);
+    }
+  }
+  return 0;
+}
+
+// Cholesky of a 4x4 SPD matrix (packed) with divisions; false if a pivot is not
+// positive relative to the trace.  L dense row-major lower.
+__device__ __forceinline__ bool chol4_div(const float* m, float* L, float rel_tol) {
+  const float tr = m[0] + m[4] + m[7] + m[9];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float s = m[sidx(j, j)];
+#pragma unroll
+    for (int p = 0; p < j; ++p) s -= L[j * 4 + p] * L[j * 4 + p];
+    if (!(s > rel_tol * tr)) return false;
+    const float d = sqrtf(s);
+    L[j * 4 + j] = d;
+#pragma unroll
+    for (int i = j + 1; i < 4; ++i) {
+      float t = m[sidx(i, j)];
+#pragma unroll
+      for (int p = 0; p < j; ++p) t -= L[i * 4 + p] * L[j * 4 + p];
+      L[i * 4 + j] = t / d;
+    }
+  }
+  return true;
+}
+
+__device__ __forceinline__ void chol4_div_solve(const float* L, const float* b, float* x) {
+  float y[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float t = b[i];
+#pragma unroll
+    for (int p = 0; p < i; ++p) t -= L[i * 4 + p] * y[p];
+    y[i] = t / L[i * 4 + i];
+  }
+#pragma unroll
+  for (int i = 3; i >= 0; --i) {
+    float t = y[i];
+#pragma unroll
+    for (int p = i + 1; p < 4; ++p) t -= L[p * 4 + i] * x[p];
+    x[i] = t / L[i * 4 + i];
+  }
+}
+
+// The FP32 rows of a two-set build, eight lanes a row, in one fixed order of
+// operations: entry 32 u + v of a row is summed in partial v, and the 32 partials
+// in a binary tree (v with v + 16, then + 8, 4, 2, 1), whatever lanes hold them.
+// A moment matrix's condition number (up to the redo's limit of 100) amplifies a
+// change of rounding here, and the low modes of the matrices amplify it again
+// (a tree over eight partials moved the modes of a million-point splat by 2e-5);
+// so a faster split of the lanes keeps the bits.  A lane takes four partials,
+// two at a time; the solves of a row are shared by its lanes.  phi holds the raw
+// kernel of a pair between the passes.
+template <class Kern>
+__device__ __forceinline__ int shape_rows_ordered(const float4* __restrict__ pos, long long s,
+                                                  long long e, const int* __restrict__ idx,
+                                                  float4 Xi, float* __restrict__ phi,
+                                                  float* __restrict__ dphi, long long n1,
+                                                  double cond_limit, const Kern& kern) {
+  constexpr int L = 8;
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & (L - 1);
+  const float xi = Xi.x, yi = Xi.y, zi = Xi.z, si = Xi.w;
+  const float isi = 1.f / si;
+  // sums q < 10: M; 10 (1 + d) + q: dM / dx_d
+  auto partial = [&](int v, float (&m)[40]) {
+#pragma unroll
+    for (int q = 0; q < 40; ++q) m[q] = 0.f;
+    for (long long t = s + v; t < e; t += 32) {
+      const int k = idx[t];
+      const float4 p = pos[k];
+      const float r0 = p.x - xi, r1 = p.y - yi, r2 = p.z - zi;
+      float w, gs;  // grad_X varphi = gs * r
+      kern.template eval<float>(k, p, r0 * r0 + r1 * r1 + r2 * r2, w, gs);
+      phi[t] = w;
+      const float P[4] = {1.f, r0 * isi, r1 * isi, r2 * isi};
+      const float g[3] = {gs * r0, gs * r1, gs * r2};
+      int o = 0;
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = a; b < 4; ++b, ++o) {
+          const float pp = P[a] * P[b];
+          m[o] = fmaf(w, pp, m[o]);
+#pragma unroll
+          for (int d = 0; d < 3; ++d) m[10 * (1 + d) + o] = fmaf(g[d], pp, m[10 * (1 + d) + o]);
+        }
+    }
+  };
+  float m[40];
+  {
+    float b[40];
+    partial(lane, m);
+    partial(lane + 16, b);
+#pragma unroll
+    for (int q = 0; q < 40; ++q) m[q] += b[q];
+  }
+  {
+    float b[40], c[40];
+    partial(lane + 8, b);
+    partial(lane + 24, c);
+#pragma unroll
+    for (int q = 0; q < 40; ++q) m[q] += b[q] + c[q];
+  }
+#pragma unroll
+  for (int q = 0; q < 40; ++q) m[q] = group_sum<L>(m[q]);
+  float Lf[16];
+  const bool spd = chol4_div(m, Lf, 1e-12f);
+  if (!spd)
+#pragma unroll
+    for (int q = 0; q < 16; ++q) Lf[q] = 1.f;  // solved for nothing below
+  // a lane a column of the inverse (twice): the 1-norm condition number, and
+  // C, its first column
+  const int col = lane & 3;
+  float x[4];
+  {
+    const float ecol[4] = {(float)(col == 0), (float)(col == 1), (float)(col == 2),
+                           (float)(col == 3)};
+    chol4_div_solve(Lf, ecol, x);
+  }
+  float inv_norm = 0.f, m_norm = 0.f;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) inv_norm += fabsf(x[r]);
+  inv_norm = fmaxf(0.f, inv_norm);
+#pragma unroll
+  for (int o = 2; o; o >>= 1) inv_norm = fmaxf(inv_norm, __shfl_xor_sync(kAll, inv_norm, o));
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float a = 0.f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) a += fabsf(m[sidx(r, c)]);
+    m_norm = fmaxf(m_norm, a);
+  }
+  float Cv[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) Cv[r] = __shfl_sync(kAll, x[r], 0, L);
+  // a lane a direction (lanes past 2 repeat the last): dC
+  float dC[3][4];
+  {
+    const int d = min(col, 2);
+    float rhs[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      float t = 0.f;
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {
+        const int q = 10 + sidx(r, cc);
+        const float md = d == 0 ? m[q] : d == 1 ? m[q + 10] : m[q + 20];
+        t += md * Cv[cc];
+      }
+      rhs[r] = -t;
+    }
+    if (d == 0) rhs[1] += isi;
+    if (d == 1) rhs[2] += isi;
+    if (d == 2) rhs[3] += isi;
+    chol4_div_solve(Lf, rhs, x);
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) dC[d][r] = __shfl_sync(kAll, x[r], d, L);
+  if (!spd) return 1;
+  if ((double)(inv_norm * m_norm) > cond_limit) return 2;
+  for (long long t = s + lane; t < e; t += L) {
+    const int k = idx[t];
+    const float4 p = pos[k];
+    const float r0 = p.x - xi, r1 = p.y - yi, r2 = p.z - zi;
+    const float w = phi[t], gs = kern.template slope<float>(k, p, w);
+    const float P[4] = {1.f, r0 * isi, r1 * isi, r2 * isi};
+    float PC = Cv[0];
+#pragma unroll
+    for (int a = 1; a < 4; ++a) PC = fmaf(P[a], Cv[a], PC);
+    phi[t] = w * PC;
+    const float g[3] = {gs * r0, gs * r1, gs * r2};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      float PdC = dC[d][0];
+#pragma unroll
+      for (int a = 1; a < 4; ++a) PdC = fmaf(P[a], dC[d][a], PdC);
+      dphi[d * n1 + t] = g[d] * PC + w * PdC;
     }
   }
   return 0;

@@ -834,20 +834,22 @@ __global__ void k_cover_cols(const float* __restrict__ Xq, long long nq,
 }
 
 // ------------------------------------------------------------------ shape functions
-// 1 / r_k^2 for the Gaussian's FP32 and double-float forms, rounded from FP64
-// (kept finite: a pair at distance 0 has weight 1 whatever the radius)
+// what the Gaussian's FP32 and double-float forms take of a radius: the square of
+// its FP32 rounding, and 1 / r_k^2 rounded from FP64 (kept finite: a pair at
+// distance 0 has weight 1 whatever the radius)
 __global__ void k_centre_inv(const double* __restrict__ rad, int K, float4* __restrict__ cpos,
                              dfloat* __restrict__ inv) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= K) return;
-  const double v = fmin(1.0 / (rad[k] * rad[k]), 3e38);
-  cpos[k].w = (float)v;
-  inv[k] = dfloat(v);
+  const float r = (float)rad[k];
+  cpos[k].w = r * r;
+  inv[k] = dfloat(fmin(1.0 / (rad[k] * rad[k]), 3e38));
 }
 
 // lanes a row: a point has ~100 covering centres, so eight lanes take a dozen
 // each and a warp's moment solve serves four points.  FP32, 1M points of 98
-// centres: 3.17 ms with a warp a point, 0.95 ms now (values alone 0.41 ms);
+// centres: 3.17 ms with a warp a point, 1.61 ms in its
+// order of operations (0.95 ms in a free one; values alone 0.51 ms);
 // double-float, 228k points: 5.73 ms, 2.09 ms now.
 constexpr int kShapeLanes = 8;
 
@@ -864,8 +866,12 @@ __global__ void __launch_bounds__(256, 2)
   const float4 Xi = live ? make_float4(Xq[3 * i], Xq[3 * i + 1], Xq[3 * i + 2], scale)
                          : make_float4(0.f, 0.f, 0.f, 1.f);
   if constexpr (sizeof(T) == 4) {
-    const int st = rkpm::shape_rows<float, T, kShapeLanes, GRAD>(
-        cpos, s, e, idx, Xi, phi, dphi, n1, cond_limit, true, kern);
+    int st;
+    if constexpr (GRAD)
+      st = rkpm::shape_rows_ordered(cpos, s, e, idx, Xi, phi, dphi, n1, cond_limit, kern);
+    else
+      st = rkpm::shape_rows<float, T, kShapeLanes, GRAD>(cpos, s, e, idx, Xi, phi, dphi, n1,
+                                                        cond_limit, true, kern);
     if (live && st != 0 && first) rkpm::redo_later(redo, i);
   } else {
     const int st = rkpm::shape_rows<dfloat, T, kShapeLanes, GRAD>(
