@@ -955,6 +955,236 @@ __global__ void __launch_bounds__(kCT) k_rr_house_cluster(int n, RRWork<R> w) {
     for (int i = tid; i < n; i += kCT) w.e2[i] = w.e[i] * w.e[i];
 }
 
+// ------------------------------------------------------------------ 1c. one-block Householder
+// The same reduction by one block with the matrix in registers, for the sizes
+// they hold.  Warp tr and lane tc hold rows tr + NW i and columns tc + 32 q; a
+// step has two block barriers and no traffic between SMs:
+//   1. every warp forms the reflector from column j (a lane holds the column's
+//      entries tc + 32 q, and entry tr + NW lane for the warp's own rows) and its
+//      rows' share of A v, which by symmetry is a sum over rows for every column;
+//      the lane that holds column j + 1 publishes it as it stands;
+//   2. after a barrier, a thread a column sums the warps' shares and p^T v;
+//   3. after a barrier, every warp forms w = tau p - K v for its columns and
+//      rows, column j + 1 as the update will leave it, and updates its entries.
+// Blocks of columns and rows that are done are skipped.  The cluster pays a
+// cluster barrier and a round of remote loads a step; alone, in FP32: n = 60 43
+// us against the cluster's 129, n = 120 108 against 270, n = 216 319 against 539;
+// in double-float n = 60 138 against 210, n = 90 287 against 328.
+// w = tau (A v) - K v and the next column o - (v w_n + w v_1), rounded the same
+// wherever they are formed: rows and columns must see one reflector
+__device__ __forceinline__ float house_w(float t, float p, float K, float v) {
+  return __fmaf_rn(-K, v, __fmul_rn(t, p));
+}
+__device__ __forceinline__ dfloat house_w(dfloat t, dfloat p, dfloat K, dfloat v) {
+  return t * p - K * v;
+}
+__device__ __forceinline__ float house_col(float o, float v, float wn, float w, float v1) {
+  return __fsub_rn(o, __fmaf_rn(v, wn, __fmul_rn(w, v1)));
+}
+__device__ __forceinline__ dfloat house_col(dfloat o, dfloat v, dfloat wn, dfloat w, dfloat v1) {
+  return o - (v * wn + w * v1);
+}
+
+template <class R, int NW, int RI, int CJ>
+__global__ void __launch_bounds__(32 * NW) k_rr_house_reg(int n, RRWork<R> w) {
+  // stride of a warp's rows in the row-wise vectors: two lanes a bank at most
+  // when they are read by columns
+  constexpr int kHS = RI <= 20 ? 20 : RI <= 28 ? 28 : 36;
+  static_assert(RI <= 32 && RI % 2 == 0 && CJ <= NW && NW * RI >= 32 * CJ, "layout");
+  struct __align__(2 * sizeof(R)) Pair {
+    R v, w;
+  };
+  __shared__ R part[NW][32 * CJ];        // the warps' shares of A v
+  __shared__ R oldc[2][NW * kHS];        // column j + 1 before the update
+  __shared__ R pvec[NW * kHS];           // A v
+  __shared__ Pair vw[NW][RI];            // v and w of a warp's own rows
+  __shared__ R ksum[NW];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  auto at = [](int l) { return (l % NW) * kHS + l / NW; };
+  const int rl = wid + NW * lane;        // the row whose vectors this lane keeps
+  R a[RI][CJ], cc[CJ];
+#pragma unroll
+  for (int i = 0; i < RI; ++i)
+#pragma unroll
+    for (int q = 0; q < CJ; ++q) {
+      const int r = wid + NW * i, c = lane + 32 * q;
+      a[i][q] = r < n && c < n ? w.As[(size_t)r * n + c] : R(0.0);
+    }
+#pragma unroll
+  for (int q = 0; q < CJ; ++q) cc[q] = lane + 32 * q < n ? w.As[lane + 32 * q] : R(0.0);
+  R rc = lane < RI && rl < n ? w.As[rl] : R(0.0);  // column j at row rl
+  // entry l of a vector held by columns, in every lane
+  auto pick = [&](const R (&x)[CJ], int l) {
+    R t = x[0];
+#pragma unroll
+    for (int q = 1; q < CJ; ++q)
+      if (q == l / 32) t = x[q];
+    return __shfl_sync(0xffffffffu, t, l % 32);
+  };
+  // one step; blocks of columns before Q0 = (j + 1) / 32 are done
+  auto step = [&](int j, auto first) {
+    constexpr int Q0 = decltype(first)::value;
+    const int buf = j & 1, j1 = j + 1;
+    const bool low = j1 < NW * (RI / 2);  // the first half of the rows is not done
+    // 1. the reflector
+    R ss = R(0.0);
+#pragma unroll
+    for (int q = Q0 > 0 ? Q0 - 1 : 0; q < CJ; ++q)
+      if (lane + 32 * q > j) ss += cc[q] * cc[q];
+    ss = warp_sum(ss);
+    const R x0 = pick(cc, j1);
+    const R alpha = sqrt(ss);
+    const bool refl = alpha > Prec<R>::tiny;
+    const R beta = x0 >= R(0.0) ? -alpha : alpha;
+    const R tj = refl ? (beta - x0) / beta : R(0.0);
+    const R scale = refl ? R(1.0) / (x0 - beta) : R(0.0);
+    const R v1 = refl ? R(1.0) : R(0.0);
+    if (wid == j % NW) {
+      const R dj = pick(cc, j);
+      if (lane == 0) {
+        const R ej = refl ? beta : x0;
+        w.dg[j] = dj;
+        w.tau[j] = tj;
+        w.e[j] = ej;
+        w.e2[j] = ej * ej;
+      }
+    }
+#pragma unroll
+    for (int q = Q0; q < CJ; ++q) {  // cc becomes v
+      const int c = lane + 32 * q;
+      cc[q] = c > j1 ? cc[q] * scale : c == j1 ? v1 : R(0.0);
+      if (wid == j % NW && c > j && c < n) w.ref[(size_t)j * n + c] = cc[q];
+    }
+    const R rv = rl > j1 ? rc * scale : rl == j1 ? v1 : R(0.0);
+    if (lane < RI) vw[wid][lane].v = rv;
+    __syncwarp();
+    R s[CJ];
+#pragma unroll
+    for (int q = Q0; q < CJ; ++q) s[q] = R(0.0);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (h == 0 && !low) continue;
+#pragma unroll
+      for (int i = h * (RI / 2); i < (h + 1) * (RI / 2); ++i) {
+        const R vi = vw[wid][i].v;
+#pragma unroll
+        for (int q = Q0; q < CJ; ++q) s[q] += a[i][q] * vi;
+      }
+    }
+#pragma unroll
+    for (int q = Q0; q < CJ; ++q) part[wid][lane + 32 * q] = s[q];
+    if (lane == j1 % 32)
+#pragma unroll
+      for (int i = 0; i < RI; ++i) oldc[buf][wid * kHS + i] = a[i][Q0];
+    __syncthreads();
+    // 2. A v and its product with v, a thread a column
+    if (wid < CJ && wid >= Q0) {
+      R p = R(0.0);
+#pragma unroll
+      for (int u = 0; u < NW; ++u) p += part[u][tid];
+      pvec[at(tid)] = p;
+      R vc = cc[Q0];
+#pragma unroll
+      for (int q = Q0 + 1; q < CJ; ++q)
+        if (q == wid) vc = cc[q];
+      const R kp = warp_sum(p * vc);
+      if (lane == 0) ksum[wid] = kp;
+    }
+    __syncthreads();
+    // 3. w, the next column, the update
+    R K = R(0.0);
+#pragma unroll
+    for (int q = Q0; q < CJ; ++q) K += ksum[q];
+    K = R(0.5) * tj * tj * K;
+    const R wn = house_w(tj, pvec[at(j1)], K, v1);
+    if (lane < RI) {
+      const R rw = rl > j ? house_w(tj, pvec[wid * kHS + lane], K, rv) : R(0.0);
+      vw[wid][lane].w = rw;
+      rc = house_col(oldc[buf][wid * kHS + lane], rv, wn, rw, v1);
+    }
+    __syncwarp();
+    R wc[CJ];
+#pragma unroll
+    for (int q = Q0; q < CJ; ++q) {
+      const int c = lane + 32 * q;
+      wc[q] = c > j ? house_w(tj, pvec[at(c)], K, cc[q]) : R(0.0);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (h == 0 && !low) continue;
+#pragma unroll
+      for (int i = h * (RI / 2); i < (h + 1) * (RI / 2); ++i) {
+        const Pair z = vw[wid][i];
+#pragma unroll
+        for (int q = Q0; q < CJ; ++q) a[i][q] -= z.v * wc[q] + z.w * cc[q];
+      }
+    }
+#pragma unroll
+    for (int q = Q0; q < CJ; ++q)
+      cc[q] = house_col(oldc[buf][at(lane + 32 * q)], cc[q], wn, wc[q], v1);
+    __syncwarp();
+  };
+  int j = 0;
+  auto run = [&](auto first) {
+    constexpr int Q0 = decltype(first)::value;
+    if constexpr (Q0 < CJ)
+      for (; j + 2 < n && (j + 1) / 32 == Q0; ++j) step(j, first);
+  };
+  run(std::integral_constant<int, 0>{});
+  run(std::integral_constant<int, 1>{});
+  run(std::integral_constant<int, 2>{});
+  run(std::integral_constant<int, 3>{});
+  run(std::integral_constant<int, 4>{});
+  run(std::integral_constant<int, 5>{});
+  run(std::integral_constant<int, 6>{});
+  static_assert(CJ <= 7, "column blocks");
+  // the last 2 x 2 block
+  const R d2 = pick(cc, n - 2), e2 = pick(cc, n - 1);
+  if (tid == 0) {
+    w.dg[n - 2] = d2;
+    w.e[n - 2] = e2;
+    w.e2[n - 2] = e2 * e2;
+    w.tau[n - 2] = w.tau[n - 1] = R(0.0);
+    w.e[n - 1] = w.e2[n - 1] = R(0.0);
+  }
+#pragma unroll
+  for (int i = 0; i < RI; ++i)
+#pragma unroll
+    for (int q = 0; q < CJ; ++q)
+      if (wid + NW * i == n - 1 && lane + 32 * q == n - 1) w.dg[n - 1] = a[i][q];
+}
+
+// launches it when the registers hold an n x n matrix (false: the cluster's)
+template <class R>
+bool launch_house_reg(int n, RRWork<R> w, cudaStream_t st) {
+  if (n < 3) return false;
+  auto go = [&](auto nw, auto ri, auto cj) {
+    constexpr int NW = decltype(nw)::value;
+    (k_rr_house_reg<R, NW, decltype(ri)::value, decltype(cj)::value>
+     <<<1, 32 * NW, 0, st>>>(n, w),
+     ::ff::note_launch());
+    return true;
+  };
+#define FF_HOUSE(NW, RI, CJ)                                                       \
+  go(std::integral_constant<int, NW>{}, std::integral_constant<int, RI>{},         \
+     std::integral_constant<int, CJ>{})
+  // eight warps (sixteen at n = 216: 426 us against 319); double-float takes
+  // twice the registers and twelve times the arithmetic, and past n = 96 the
+  // cluster's sixteen SMs are the faster (n = 120: 549 us against 470)
+  if constexpr (std::is_same_v<R, float> || std::is_same_v<R, dfloat>) {
+    if (n <= 64) return FF_HOUSE(8, 8, 2);
+    if (n <= 96) return FF_HOUSE(8, 12, 3);
+  }
+  if constexpr (std::is_same_v<R, float>) {
+    if (n <= 128) return FF_HOUSE(8, 16, 4);
+    if (n <= 160) return FF_HOUSE(8, 20, 5);
+    if (n <= 192) return FF_HOUSE(8, 24, 6);
+    if (n <= 224) return FF_HOUSE(8, 28, 7);
+  }
+#undef FF_HOUSE
+  return false;
+}
+
 // ------------------------------------------------------------------ 2b. eigenvalues, one block each
 // FP64 multisection with the division-free Sturm count: one warp per
 // eigenvalue, 32 probes per round (a 33-fold shrink of the bracket per round).
@@ -1765,7 +1995,7 @@ void rr_run(cudaStream_t st, const double* A, const double* B, RRDims d, T* YZ, 
                                                                 tri_smem, use_cluster ? 0 : 1, Yg),
    ::ff::note_launch());
   FF_LAUNCH_CHECK();
-  if (use_cluster) {
+  if (use_cluster && !launch_house_reg<R>(d.ns, w, st)) {
     if (cs == 16)
       launch_house<R, 16>(d.ns, w, cl_bytes, st);
     else
