@@ -59,6 +59,7 @@ ff_status eigenmodes_batched(int device, int precision, ff_batch_item* items, in
       cudaStreamDestroy(st);
       return;
     }
+    c->beside_others = nw > 1;
     for (;;) {
       const int q = next.fetch_add(1);
       if (q >= count) break;

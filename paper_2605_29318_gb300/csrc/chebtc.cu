@@ -317,6 +317,188 @@ __global__ void __launch_bounds__(32 * WB)
   }
 }
 
+// All the steps of a polynomial in one cooperative launch, for matrices of few
+// row blocks (one block of 16 warps each, all resident): a block keeps its A
+// fragments, union columns, residual and x in registers for the whole polynomial
+// and only the directions pass through memory, with a grid barrier between steps.
+// The same sums in the same order as k_cheb_step_tc<NT, 16>, bit for bit.  A
+// step by itself is a launch, the loads of tiles and columns, and a tail: for
+// 3,001 rows and 24 columns 7.8 us, 3.5 so; for the 1,000 x 1,000 pencil of the
+// splat and 72 columns 9.6 us, 5.0 so.  Not for solves beside others on the GPU (a
+// batch): a cooperative launch waits until all its blocks fit, and four objects of
+// 2,000 to 20,000 particles took 108 ms with it against 103 without.
+// Each warp's k-steps must fit its registers (kPolyK of them).
+constexpr int kPolyK = 4;        // k-steps of a warp: unions up to 1,024 columns
+constexpr int kPolyMax = 64;     // steps a launch
+struct PolyCoef {
+  float c1[kPolyMax], c2[kPolyMax];
+};
+
+// Arrivals counted up to `target` (modulo 2^32); false when the wait ran out
+// (about a second: a block of the grid was not running)
+__device__ __forceinline__ bool poly_barrier(unsigned* bar, unsigned target) {
+  __shared__ int s_late;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+    const long long t0 = clock64();
+    int late = 0;
+    unsigned v;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (clock64() - t0 > 2000000000LL) late = 1;
+    } while ((int)(v - target) < 0 && !late);
+    __threadfence();
+    s_late = late;
+  }
+  __syncthreads();
+  return s_late == 0;
+}
+
+constexpr size_t poly_smem(int NT, int ksteps) {
+  return std::max<size_t>((size_t)16 * ksteps * kTcRows * 8 * NT * 2, (size_t)16 * 32 * 4 * NT * 4);
+}
+
+template <int NT>
+__global__ void __launch_bounds__(512, NT <= 5 ? 2 : 1)
+    k_cheb_poly_tc(const int* __restrict__ kofs, const int* __restrict__ ucol,
+                   const uint4* __restrict__ tile, const float* __restrict__ hs,
+                   const float* __restrict__ hdiag, int n, __nv_bfloat16* d0, __nv_bfloat16* d1,
+                   float* __restrict__ x, const float* __restrict__ res, int steps, PolyCoef coef,
+                   int ksteps, unsigned* bar, unsigned base) {
+  constexpr int kWB = 16;
+  constexpr int m = 8 * NT, PIECES = kTcRows * NT, ITERS = (PIECES + 31) / 32;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int b = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __nv_bfloat16* stage = reinterpret_cast<__nv_bfloat16*>(smem) + (size_t)w * ksteps * kTcRows * m;
+  float* red = reinterpret_cast<float*>(smem);  // [kWB][32][4 NT]
+  const int s0 = kofs[b], ns = kofs[b + 1] - s0;
+  uint4 A[kPolyK];
+  int U[kPolyK];
+#pragma unroll
+  for (int p = 0; p < kPolyK; ++p) {
+    const int s = w + p * kWB;
+    A[p] = s < ns ? __ldg(tile + (long long)(s0 + s) * 32 + lane) : make_uint4(0u, 0u, 0u, 0u);
+    U[p] = s < ns && lane < 16 ? __ldg(ucol + (long long)(s0 + s) * 16 + lane) : 0;
+  }
+  // warp j finishes column tile j: rows g and g + 8, columns 8 j + 2 t and the next
+  const int g = lane >> 2, t = lane & 3;
+  float2 r[2], xx[2], dk[2];
+  float dinv[2] = {0.f, 0.f}, hsk[2] = {0.f, 0.f};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int k = b * kTcRows + g + 8 * h;
+    r[h] = xx[h] = dk[h] = make_float2(0.f, 0.f);
+    if (w < NT && k < n) {
+      const long long o = (long long)k * m + 8 * w + 2 * t;
+      dinv[h] = 1.0f / hdiag[k];
+      hsk[h] = hs[k];
+      r[h] = *reinterpret_cast<const float2*>(res + o);
+      xx[h] = *reinterpret_cast<const float2*>(x + o);
+      dk[h] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(d0 + o));
+    }
+  }
+  bool ok = true;
+  for (int it = 0; it < steps; ++it) {
+    const __nv_bfloat16* din = it & 1 ? d1 : d0;
+    __nv_bfloat16* dout = it & 1 ? d0 : d1;
+#pragma unroll
+    for (int p = 0; p < kPolyK; ++p) {
+      if (w + p * kWB < ns) {
+        __nv_bfloat16* dst = stage + p * kTcRows * m;
+#pragma unroll
+        for (int q = 0; q < ITERS; ++q) {
+          const int e = q * 32 + lane;
+          const int rr = min(e / NT, kTcRows - 1), pc = e % NT;
+          const int row = __shfl_sync(kFullMask, U[p], rr);
+          if (e < PIECES) cp_async16(dst + rr * m + pc * 8, din + (long long)row * m + pc * 8);
+        }
+      }
+      cp_commit();
+    }
+    float acc[NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+#pragma unroll
+    for (int p = 0; p < kPolyK; ++p) {
+      if (p == 0) asm volatile("cp.async.wait_group %0;\n" ::"n"(kPolyK - 1) : "memory");
+      if (p == 1) asm volatile("cp.async.wait_group %0;\n" ::"n"(kPolyK - 2) : "memory");
+      if (p == 2) asm volatile("cp.async.wait_group %0;\n" ::"n"(kPolyK - 3) : "memory");
+      if (p == 3) asm volatile("cp.async.wait_group %0;\n" ::"n"(0) : "memory");
+      __syncwarp();
+      if (w + p * kWB >= ns) continue;
+      const unsigned sbase = (unsigned)__cvta_generic_to_shared(stage + p * kTcRows * m);
+      const int mat = lane >> 3, krow = (mat & 1) * 8 + (lane & 7);
+#pragma unroll
+      for (int j = 0; j + 1 < NT; j += 2) {
+        unsigned r0, r1, r2, r3;
+        const unsigned addr = sbase + (unsigned)(krow * m * 2 + (j + (mat >> 1)) * 16);
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                     : "r"(addr));
+        mma_bf16(acc[j], A[p], r0, r1);
+        mma_bf16(acc[j + 1], A[p], r2, r3);
+      }
+      if (NT & 1) {
+        constexpr int j = NT - 1;
+        unsigned r0, r1;
+        const unsigned addr =
+            sbase + (unsigned)(((lane >> 3) & 1) * 8 * m * 2 + (lane & 7) * m * 2 + j * 16);
+        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
+                     : "=r"(r0), "=r"(r1)
+                     : "r"(addr));
+        mma_bf16(acc[j], A[p], r0, r1);
+      }
+    }
+    __syncthreads();  // every warp is done with its staging buffers
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+      *reinterpret_cast<float4*>(red + (w * 32 + lane) * 4 * NT + 4 * j) =
+          make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+    __syncthreads();
+    if (w < NT) {
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int v = 0; v < kWB; ++v) {
+        const float4 y =
+            *reinterpret_cast<const float4*>(red + (v * 32 + lane) * 4 * NT + 4 * w);
+        c[0] += y.x;
+        c[1] += y.y;
+        c[2] += y.z;
+        c[3] += y.w;
+      }
+      const float c1 = coef.c1[it], c2 = coef.c2[it];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = b * kTcRows + g + 8 * h;
+        if (k >= n) continue;
+        r[h].x -= (c[2 * h] - hsk[h] * dk[h].x) * dinv[h];
+        r[h].y -= (c[2 * h + 1] - hsk[h] * dk[h].y) * dinv[h];
+        const __nv_bfloat16 q0 = __float2bfloat16(c1 * dk[h].x + c2 * r[h].x);
+        const __nv_bfloat16 q1 = __float2bfloat16(c1 * dk[h].y + c2 * r[h].y);
+        dk[h] = make_float2(__bfloat162float(q0), __bfloat162float(q1));
+        xx[h].x += dk[h].x;
+        xx[h].y += dk[h].y;
+        __nv_bfloat162 qq;
+        qq.x = q0;
+        qq.y = q1;
+        *reinterpret_cast<__nv_bfloat162*>(dout + (long long)k * m + 8 * w + 2 * t) = qq;
+      }
+    }
+    if (it + 1 < steps) ok = poly_barrier(bar, base + (unsigned)(it + 1) * gridDim.x);
+    if (!ok) break;
+  }
+  if (w < NT)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = b * kTcRows + g + 8 * h;
+      // a wait that ran out leaves NaN, which the solver reports
+      if (!ok) xx[h] = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+      if (k < n) *reinterpret_cast<float2*>(x + (long long)k * m + 8 * w + 2 * t) = xx[h];
+    }
+}
+
 }  // namespace
 
 bool cheb_tc_build(ff_ctx* c) {
@@ -344,6 +526,7 @@ bool cheb_tc_build(ff_ctx* c) {
     if (ofs[b + 1] >= (1 << 26)) return false;
   }
   const long long S = ofs[nblk];
+  c->tc_kmax = *std::max_element(h.begin(), h.end());
   int* kofs = reinterpret_cast<int*>(c->tc_kofs.ensure(sizeof(int) * (nblk + 1)));
   FF_CUDA(cudaMemcpyAsync(kofs, ofs.data(), sizeof(int) * (nblk + 1), cudaMemcpyHostToDevice, st));
   int* uc = reinterpret_cast<int*>(c->tc_ucol.ensure(sizeof(int) * 16 * (size_t)std::max(S, 1LL)));
@@ -409,6 +592,71 @@ bool cheb_step_tc(cudaStream_t st, const ff_ctx* c, int m, const void* din, void
 #undef FF_TC
   FF_LAUNCH_CHECK();
   return true;
+}
+
+// The steps c1[j], c2[j] (count of them) on d (bin first, bout its other buffer)
+// in one launch each of up to kPolyMax; false (nothing launched) when the row
+// blocks do not all fit the GPU at once or a block's union is too wide.
+bool cheb_poly_tc(cudaStream_t st, ff_ctx* c, int m, void* din, void* dout, float* x, float* res,
+                  const float* c1, const float* c2, int count) {
+  const int nblk = (int)((c->n + kTcRows - 1) / kTcRows);
+  const int ksteps = (c->tc_kmax + 15) / 16;
+  if (c->beside_others || c->tc_ksteps <= 0 || m % 8 != 0 || m < 8 || m > 120 ||
+      nblk >= 2 * sm_count() ||
+      ksteps > kPolyK || count < 2 || count > kPolyMax)
+    return false;
+  bool done = false;
+  auto go = [&](auto nt) {
+    constexpr int NT = decltype(nt)::value;
+    const size_t sm = poly_smem(NT, ksteps);
+    if (sm > 200 * 1024) return;
+    const void* fn = (const void*)k_cheb_poly_tc<NT>;
+    set_max_dyn_smem(fn, (int)sm);
+    int per_sm = 0;
+    FF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cheb_poly_tc<NT>, 512, sm));
+    if (per_sm * sm_count() < nblk) return;
+    if (!c->poly_bar.p) {
+      c->poly_bar.ensure(64);
+      FF_CUDA(cudaMemsetAsync(c->poly_bar.p, 0, 64, st));
+    }
+    ProfScope ps(kProfPrecond);
+    const int* kofs = c->tc_kofs.as<int>();
+    const int* ucol = c->tc_ucol.as<int>();
+    const uint4* tile = c->tc_tile.as<uint4>();
+    const float *hs = c->tc_hs.as<float>(), *hdiag = c->hdiag_f32.as<float>();
+    int n = (int)c->n, ks = ksteps, steps = count;
+    PolyCoef coef;
+    std::copy(c1, c1 + count, coef.c1);
+    std::copy(c2, c2 + count, coef.c2);
+    unsigned* bar = c->poly_bar.as<unsigned>();
+    unsigned base = c->poly_base;
+    void* args[] = {&kofs, &ucol, &tile, &hs,   &hdiag, &n,  &din, &dout,
+                    &x,    &res,  &steps, &coef, &ks,    &bar, &base};
+    FF_CUDA(cudaLaunchCooperativeKernel(fn, dim3(nblk), dim3(512), args, sm, st));
+    ::ff::note_launch();
+    c->poly_base += (unsigned)(count - 1) * (unsigned)nblk;
+    done = true;
+  };
+#define FF_TC(NT) go(std::integral_constant<int, NT>{})
+  switch (m / 8) {
+    case 1: FF_TC(1); break;
+    case 2: FF_TC(2); break;
+    case 3: FF_TC(3); break;
+    case 4: FF_TC(4); break;
+    case 5: FF_TC(5); break;
+    case 6: FF_TC(6); break;
+    case 7: FF_TC(7); break;
+    case 8: FF_TC(8); break;
+    case 9: FF_TC(9); break;
+    case 10: FF_TC(10); break;
+    case 11: FF_TC(11); break;
+    case 12: FF_TC(12); break;
+    case 13: FF_TC(13); break;
+    case 14: FF_TC(14); break;
+    default: FF_TC(15); break;
+  }
+#undef FF_TC
+  return done;
 }
 
 }  // namespace ff

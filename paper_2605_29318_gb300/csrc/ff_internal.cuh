@@ -178,6 +178,10 @@ struct ff_ctx {
   ff::Buf tc_tile;   // uint4[32 * ksteps] A fragments
   ff::Buf tc_hs;     // float[n] row sums of the rounded entries
   long long tc_ksteps = 0;
+  int tc_kmax = 0;   // the most k-steps of a block
+  ff::Buf poly_bar;  // arrivals of the polynomial's grid barrier, counted on over launches
+  unsigned poly_base = 0;
+  bool beside_others = false;  // solves of other contexts run beside this one's (batch)
   ff::Buf hdiag_f32; // float[n] diag(H)
   // skinning weights at query points (scratch of the last call)
   ff::Buf sk_cnt;    // int[nq + 1]

@@ -29,6 +29,12 @@ bool cheb_tc_build(ff_ctx* c);
 bool cheb_step_tc(cudaStream_t st, const ff_ctx* c, int m, const void* din, void* dout, float* x,
                   float* res, float c1, float c2);
 
+// All steps of a polynomial in one cooperative launch where the row blocks are
+// few (false: nothing launched); din holds the first directions, dout is the
+// other buffer.
+bool cheb_poly_tc(cudaStream_t st, ff_ctx* c, int m, void* din, void* dout, float* x, float* res,
+                  const float* c1, const float* c2, int count);
+
 // out (p x q, row-major with leading dimension ldo (default q), FP64)
 // (+)= alpha * A^T B over n rows
 template <class T>

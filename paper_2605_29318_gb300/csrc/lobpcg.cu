@@ -507,6 +507,11 @@ ff_status solve(ff_ctx* c, int k, const ff_eig_opts& o, Phase& ph, const T* X0,
   const int TB = 256;
   auto blocks = [&](long long work) { return (unsigned)((work + TB - 1) / TB); };
 
+  // the polynomial's barrier counts from zero again in every phase (a wait that
+  // ran out would leave its count short)
+  if (c->poly_bar.p) FF_CUDA(cudaMemsetAsync(c->poly_bar.p, 0, 64, st));
+  c->poly_base = 0;
+
   // ---- constant mode: c0 = 1 / sqrt(1^T M 1)
   (k_fill<T><<<blocks(n), TB, 0, st>>>(s.c0, n, T(1)), ::ff::note_launch());
   spmm_hm_raw<T>(st, c->a_ptr.as<long long>(), c->a_col.as<int>(), s.aval, n, s.c0, 1, nullptr,
@@ -753,9 +758,20 @@ ff_status solve(ff_ctx* c, int k, const ff_eig_opts& o, Phase& ph, const T* X0,
       float* dout = s.cd1;
       __nv_bfloat16* bin = s.cb0;
       __nv_bfloat16* bout = s.cb1;
-      for (int j = 1; j < deg; ++j) {
+      std::vector<float> k1(deg - 1), k2(deg - 1);
+      for (int j = 0; j + 1 < deg; ++j) {
         const double rn = 1.0 / (2.0 * sigma1 - rho);
-        const float c1 = (float)(rn * rho), c2 = (float)(2.0 * rn / delta);
+        k1[j] = (float)(rn * rho);
+        k2[j] = (float)(2.0 * rn / delta);
+        rho = rn;
+      }
+      // the whole polynomial in one launch where the row blocks are few
+      const bool whole = b16 && o.precond_tc &&
+                         cheb_poly_tc(st, c, mc, bin, bout, s.cx, s.cres, k1.data(), k2.data(),
+                                      deg - 1);
+      if (whole) s.spmv_calls += deg - 1;
+      for (int j = 1; j < deg && !whole; ++j) {
+        const float c1 = k1[j - 1], c2 = k2[j - 1];
         // the tensor-core step when its tiles exist, else the CUDA-core ones
         const bool tc =
             b16 && o.precond_tc && cheb_step_tc(st, c, mc, bin, bout, s.cx, s.cres, c1, c2);
@@ -767,7 +783,6 @@ ff_status solve(ff_ctx* c, int k, const ff_eig_opts& o, Phase& ph, const T* X0,
                     c->hdiag_f32.as<float>(), n, mc, mc, din, dout, s.cx, s.cres, c1, c2);
         }
         ++s.spmv_calls;
-        rho = rn;
         std::swap(din, dout);
         std::swap(bin, bout);
       }
