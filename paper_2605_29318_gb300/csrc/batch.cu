@@ -42,7 +42,11 @@ ff_status eigenmodes_batched(int device, int precision, ff_batch_item* items, in
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(),
                    [&](int a, int b) { return items[a].n > items[b].n; });
-  const int nw = std::min(count, workers > 0 ? workers : 8);
+  // Four by default: past that the host threads wait for one another in the
+  // driver's launch path (~2,500 launches an object).  2, 4, 6 and 8 workers: 206,
+  // 171, 189 and 203 ms for 8 objects of 2,000-20,000 particles; 531, 409, 434 and
+  // 457 ms for 24; 1463, 1350, 1356 and 1386 ms for 16 of 2,000-200,000.
+  const int nw = std::min(count, workers > 0 ? workers : 4);
   std::atomic<int> next{0};
   auto work = [&]() {
     if (cudaSetDevice(device) != cudaSuccess) {
