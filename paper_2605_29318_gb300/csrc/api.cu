@@ -10,7 +10,8 @@ void warmstart_block(ff_ctx* c, ff_net* w, int k, const ff_eig_opts& o, void* X0
 template <class T>
 void gather_block(ff_ctx* c, const T* X0, int m, T* X, int ld);
 template <class T>
-void scatter_block(ff_ctx* c, const T* X, int ld, int m, T* out);
+void scatter_blocks(ff_ctx* c, const T* A, const T* B, int ld, int m, T* outA, T* outB,
+                    const DevFlags* flags = nullptr);
 }  // namespace ff
 
 namespace {
@@ -492,13 +493,13 @@ ff_status ff_apply_operators(ff_ctx* c, const void* X, int m, void* YH, void* YM
     const long long n = c->n;
     auto run = [&](auto tag) {
       using T = decltype(tag);
-      T* in = reinterpret_cast<T*>(c->scratch[4].ensure(sizeof(T) * n * m));
-      T* oh = reinterpret_cast<T*>(c->scratch[6].ensure(sizeof(T) * n * m));
-      T* om = reinterpret_cast<T*>(c->scratch[7].ensure(sizeof(T) * n * m));
-      ff::gather_block<T>(c, static_cast<const T*>(X), m, in, m);
-      ff::spmm_hm<T>(c, in, m, oh, om, m, m);
-      if (YH) ff::scatter_block<T>(c, oh, m, m, static_cast<T*>(YH));
-      if (YM) ff::scatter_block<T>(c, om, m, m, static_cast<T*>(YM));
+      const int ld = ff::spmm_ld<T>(m);
+      T* in = reinterpret_cast<T*>(c->scratch[4].ensure(sizeof(T) * n * ld));
+      T* oh = reinterpret_cast<T*>(c->scratch[6].ensure(sizeof(T) * n * ld));
+      T* om = reinterpret_cast<T*>(c->scratch[7].ensure(sizeof(T) * n * ld));
+      ff::gather_block<T>(c, static_cast<const T*>(X), m, in, ld);
+      ff::spmm_hm<T>(c, in, oh, om, ld, m);
+      ff::scatter_blocks<T>(c, oh, om, ld, m, static_cast<T*>(YH), static_cast<T*>(YM));
       FF_CUDA(cudaStreamSynchronize(c->stream));
     };
     if (c->prec == FF_PREC_FP64)

@@ -615,8 +615,14 @@ __global__ void k_split_df(const double* __restrict__ x, float2* __restrict__ y,
 
 void finish_matrices(ff_ctx* c);
 
+void check_material(const DevFlags& f) {
+  if (f.code == FF_ERR_INVALID_ARG)
+    throw Error(FF_ERR_INVALID_ARG, "invalid material (need E > 0, 0 <= nu < 0.5) at point " +
+                                        std::to_string(f.index));
+}
+
 // v_i (lambda_i + 4 mu_i) per quadrature point into wh (double-float pairs in
-// FP64 contexts, FP32 otherwise); throws FF_ERR_INVALID_ARG on a bad material
+// FP64 contexts, FP32 otherwise)
 void material_weights(ff_ctx* c, const float* E, const float* nu, double E0, double nu0,
                       void* wh) {
   cudaStream_t st = c->stream;
@@ -635,10 +641,6 @@ void material_weights(ff_ctx* c, const float* E, const float* nu, double E0, dou
                                                     c->flags.as<DevFlags>()),
      ::ff::note_launch());
   FF_LAUNCH_CHECK();
-  const DevFlags f = read_flags(c);
-  if (f.code == FF_ERR_INVALID_ARG)
-    throw Error(FF_ERR_INVALID_ARG, "invalid material (need E > 0, 0 <= nu < 0.5) at point " +
-                                        std::to_string(f.index));
 }
 
 void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, double nu0) {
@@ -648,27 +650,14 @@ void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, doubl
   const bool f64 = c->prec == FF_PREC_FP64;
   const bool tdf = !tables_f32(c);  // double-float tables, weights and sums
   const size_t tb = f64 ? 8 : 4;
-  reset_flags(c);
   DevFlags f{};
   // material weights per quadrature point (the nodal points are in cell
   // order, the two-set quadrature points in the caller's)
-  c->wh.ensure((tdf ? 8 : 4) * nq);
-  const int* qperm = c->twoset ? nullptr : c->perm.as<int>();
-  if (tdf)  // FP64 contexts: material weights in double-float, like the shape functions
-    (k_material<dfloat><<<ceil_div(nq, T), T, 0, st>>>(qperm, nq, c->vol.as<float>(), E, nu, E0,
-                                                     nu0, c->wh.as<dfloat>(),
-                                                     c->flags.as<DevFlags>()), ::ff::note_launch());
-  else
-    (k_material<float><<<ceil_div(nq, T), T, 0, st>>>(qperm, nq, c->vol.as<float>(), E, nu, E0,
-                                                    nu0, c->wh.as<float>(),
-                                                    c->flags.as<DevFlags>()), ::ff::note_launch());
-  FF_LAUNCH_CHECK();
+  material_weights(c, E, nu, E0, nu0, c->wh.ensure((tdf ? 8 : 4) * nq));
   if (c->twoset && tset_assembly_fits(n)) {
     // two-set clouds: dense tiles of points grouped by their nearest centre
     f = read_flags(c);
-    if (f.code == FF_ERR_INVALID_ARG)
-      throw Error(FF_ERR_INVALID_ARG, "invalid material (need E > 0, 0 <= nu < 0.5) at point " +
-                                          std::to_string(f.index));
+    check_material(f);
     tset_assemble(c);
     finish_matrices(c);
     return;
@@ -696,9 +685,7 @@ void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, doubl
     FF_LAUNCH_CHECK();
     FF_CUDA(cudaMemcpyAsync(&tmax, dmax, sizeof(TileMax), cudaMemcpyDeviceToHost, st));
     f = read_flags(c);
-    if (f.code == FF_ERR_INVALID_ARG)
-      throw Error(FF_ERR_INVALID_ARG, "invalid material (need E > 0, 0 <= nu < 0.5) at point " +
-                                          std::to_string(f.index));
+    check_material(f);
   }
   const bool tiles = !tmax.over;
   // row-owner pass 1: unique columns per row, in a table of 2048 slots per warp
@@ -724,9 +711,7 @@ void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, doubl
                                           " distinct columns (support too large)");
   }
   ps_pattern.close();
-  if (f.code == FF_ERR_INVALID_ARG)
-    throw Error(FF_ERR_INVALID_ARG, "invalid material (need E > 0, 0 <= nu < 0.5) at point " +
-                                        std::to_string(f.index));
+  check_material(f);
   long long* aptr = reinterpret_cast<long long*>(c->a_ptr.ensure(sizeof(long long) * (n + 1)));
   scan_counts(cnt, aptr, n, c, c->scratch[3]);
   long long n2 = 0;

@@ -245,9 +245,11 @@ void scan_counts_i32(const int* in, int* out, long long n, ff_ctx* c, Buf& tmp);
 void build_neighbours(ff_ctx* c, const float* X, const float* v, const float* a, int64_t n);
 void build_shape(ff_ctx* c);
 void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, double nu0);
-// v_i (lambda_i + 4 mu_i) per quadrature point (context precision) into wh
+// v_i (lambda_i + 4 mu_i) per quadrature point into wh; the flags, reset here, hold
+// a bad material for check_material once the stream is done
 void material_weights(ff_ctx* c, const float* E, const float* nu, double E0, double nu0,
                       void* wh);
+void check_material(const DevFlags& f);
 // the grid barrier's bounded wait run out on purpose (one arrival missing)
 ff_status selftest_device_wait(int device, long long wait_cycles);
 // the transposed lists of a two-set cloud (built on demand)
@@ -277,9 +279,17 @@ void skinning_weights(ff_ctx* c, const float* Q, long long nq, const void* C, in
 void lbs_deform(ff_ctx* c, const float* Q, long long nq, const void* W, int m, const void* Z,
                 void* x);
 
-// operator application on internal-order row-major panels
+// operator application on internal-order row-major panels of m columns and
+// leading dimension ld: spmm_ld(m) columns fill whole 16 bytes a row, which the
+// vector kernels take (the columns past m are computed from whatever they hold);
+// ld = m runs the general kernel where m is not such a number
 template <class T>
-void spmm_hm(ff_ctx* c, const T* X, int ldx, T* YH, T* YM, int ldy, int m);
+inline int spmm_ld(int m) {
+  constexpr int v = 16 / (int)sizeof(T);
+  return (m + v - 1) / v * v;
+}
+template <class T>
+void spmm_hm(ff_ctx* c, const T* X, T* YH, T* YM, int ld, int m);
 
 // eigen solver
 ff_status run_eigenmodes(ff_ctx* c, int k, const ff_eig_opts& o, const void* X0,

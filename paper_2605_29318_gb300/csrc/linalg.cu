@@ -741,6 +741,11 @@ __global__ void k_spmm_hm_f64x4(const long long* __restrict__ ptr, const int* __
   for (long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += warps) {
     const long long s = ptr[k], e = ptr[k + 1];
     double ah[4] = {0, 0, 0, 0}, am[4] = {0, 0, 0, 0}, hs = 0.0;
+    // the row sum, a lane an entry: summed beside the products it would be a ninth
+    // of their FP64 instructions
+    for (long long t = s + lane; t < e; t += 32) hs += val[2 * t];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) hs += __shfl_xor_sync(kFull, hs, o);
     long long e0 = act ? s + g : e;
     for (; e0 + P < e; e0 += 2 * P) {
       const int l0 = col[e0], l1 = col[e0 + P];
@@ -749,7 +754,6 @@ __global__ void k_spmm_hm_f64x4(const long long* __restrict__ ptr, const int* __
       const double2* p0 = reinterpret_cast<const double2*>(X + (long long)l0 * ldx + cv);
       const double2* p1 = reinterpret_cast<const double2*>(X + (long long)l1 * ldx + cv);
       const double2 a0 = __ldg(p0), b0 = __ldg(p0 + 1), a1 = __ldg(p1), b1 = __ldg(p1 + 1);
-      hs += hm0.x + hm1.x;
       ah[0] = fma(hm0.x, a0.x, ah[0]); ah[1] = fma(hm0.x, a0.y, ah[1]);
       ah[2] = fma(hm0.x, b0.x, ah[2]); ah[3] = fma(hm0.x, b0.y, ah[3]);
       am[0] = fma(hm0.y, a0.x, am[0]); am[1] = fma(hm0.y, a0.y, am[1]);
@@ -764,7 +768,6 @@ __global__ void k_spmm_hm_f64x4(const long long* __restrict__ ptr, const int* __
       const double2 hm0 = *reinterpret_cast<const double2*>(val + 2 * e0);
       const double2* p0 = reinterpret_cast<const double2*>(X + (long long)l0 * ldx + cv);
       const double2 a0 = __ldg(p0), b0 = __ldg(p0 + 1);
-      hs += hm0.x;
       ah[0] = fma(hm0.x, a0.x, ah[0]); ah[1] = fma(hm0.x, a0.y, ah[1]);
       ah[2] = fma(hm0.x, b0.x, ah[2]); ah[3] = fma(hm0.x, b0.y, ah[3]);
       am[0] = fma(hm0.y, a0.x, am[0]); am[1] = fma(hm0.y, a0.y, am[1]);
@@ -780,8 +783,6 @@ __global__ void k_spmm_hm_f64x4(const long long* __restrict__ ptr, const int* __
           am[u] += tm;
         }
       }
-      const double ts = __shfl_down_sync(kFull, hs, q * G);
-      if (g == 0) hs += ts;
     }
     if (g == 0) {
       const double2* pk = reinterpret_cast<const double2*>(X + k * ldx + cv);
@@ -822,6 +823,13 @@ __global__ void __launch_bounds__(256)
     dfloat ah[4], am[4], hs(0);
 #pragma unroll
     for (int u = 0; u < 4; ++u) ah[u] = am[u] = dfloat(0);
+    // the row sum, a lane an entry
+    for (int t = lane; t < cnt; t += 32) {
+      const float2 h = __ldg(reinterpret_cast<const float2*>(vr + t));
+      df_acc(hs, dfloat(h.x, h.y));
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) hs = df_add(df_norm(hs), df_norm(__shfl_xor_sync(kFull, hs, o)));
     int e = act ? g : cnt;
     for (; e + P < cnt; e += 2 * P) {
       const int l0 = __ldg(cr + e), l1 = __ldg(cr + e + P);
@@ -834,8 +842,6 @@ __global__ void __launch_bounds__(256)
       const dfloat x1[4] = {dfloat(a1.x, a1.y), dfloat(a1.z, a1.w), dfloat(b1.x, b1.y),
                             dfloat(b1.z, b1.w)};
       const dfloat h0(v0.x, v0.y), m0(v0.z, v0.w), h1(v1.x, v1.y), m1(v1.z, v1.w);
-      df_acc(hs, h0);
-      df_acc(hs, h1);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         df_mac(ah[u], h0, x0[u]);
@@ -852,7 +858,6 @@ __global__ void __launch_bounds__(256)
       const dfloat x0[4] = {dfloat(a0.x, a0.y), dfloat(a0.z, a0.w), dfloat(b0.x, b0.y),
                             dfloat(b0.z, b0.w)};
       const dfloat h0(v0.x, v0.y), m0(v0.z, v0.w);
-      df_acc(hs, h0);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         df_mac(ah[u], h0, x0[u]);
@@ -869,8 +874,6 @@ __global__ void __launch_bounds__(256)
           df_acc(am[u], tm);
         }
       }
-      const dfloat ts = __shfl_down_sync(kFull, hs, q * G);
-      if (g == 0) df_acc(hs, ts);
     }
     if (g == 0) {
       const long long o = (long long)k * ldy + cv;
@@ -1073,7 +1076,7 @@ __global__ void __launch_bounds__(32 * kSW)
 
 template <class T>
 void spmm_hm_raw(cudaStream_t st, const long long* ptr, const int* col, const T* val, long long n,
-                 const T* X, int ldx, T* YH, T* YM, int ldy, int m) {
+                 const T* X, int ldx, T* YH, T* YM, int ldy, int m, bool diff) {
   ProfScope ps(kProfSpmm);
   const int T_ = 256;
   long long blocks = std::min<long long>((n * 32 + T_ - 1) / T_, (long long)sm_count() * 64);
@@ -1103,7 +1106,10 @@ void spmm_hm_raw(cudaStream_t st, const long long* ptr, const int* col, const T*
                         (!YH || reinterpret_cast<uintptr_t>(YH) % 16 == 0) &&
                         (!YM || reinterpret_cast<uintptr_t>(YM) % 16 == 0);
     if constexpr (std::is_same_v<T, double>) {
-      if (vec_ok && m % 4 == 0 && m <= 128 && reinterpret_cast<uintptr_t>(val) % 16 == 0) {
+      const bool x4_ok = ldx % 2 == 0 && ldy % 2 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
+                         (!YH || reinterpret_cast<uintptr_t>(YH) % 16 == 0) &&
+                         (!YM || reinterpret_cast<uintptr_t>(YM) % 16 == 0);
+      if (!diff && x4_ok && m % 4 == 0 && m <= 128 && reinterpret_cast<uintptr_t>(val) % 16 == 0) {
         (k_spmm_hm_f64x4<<<(unsigned)blocks, T_, 0, st>>>(ptr, col, val, n, X, ldx, YH, YM, ldy,
                                                          m),
          ::ff::note_launch());
@@ -1480,9 +1486,9 @@ void block_update(cudaStream_t st, const T* A, int lda, int p, const T* Y, int q
 }
 
 template void spmm_hm_raw<float>(cudaStream_t, const long long*, const int*, const float*,
-                                 long long, const float*, int, float*, float*, int, int);
+                                 long long, const float*, int, float*, float*, int, int, bool);
 template void spmm_hm_raw<double>(cudaStream_t, const long long*, const int*, const double*,
-                                  long long, const double*, int, double*, double*, int, int);
+                                  long long, const double*, int, double*, double*, int, int, bool);
 template void gram<float>(cudaStream_t, const float*, int, int, const float*, int, int, long long,
                           double*, double, bool, Buf&, int);
 template void gram<double>(cudaStream_t, const double*, int, int, const double*, int, int,
@@ -1496,7 +1502,7 @@ template void block_update<float>(cudaStream_t, const float*, int, int, const fl
 template void block_update<double>(cudaStream_t, const double*, int, int, const double*, int,
                                    double*, int, long long, double, int, int, int);
 template void spmm_hm_raw<dfloat>(cudaStream_t, const long long*, const int*, const dfloat*,
-                                  long long, const dfloat*, int, dfloat*, dfloat*, int, int);
+                                  long long, const dfloat*, int, dfloat*, dfloat*, int, int, bool);
 template void gram<dfloat>(cudaStream_t, const dfloat*, int, int, const dfloat*, int, int,
                            long long, double*, double, bool, Buf&, int);
 template void gram_rr<dfloat>(cudaStream_t, const dfloat*, const dfloat*, const dfloat*, int, int,

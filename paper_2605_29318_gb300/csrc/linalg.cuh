@@ -8,7 +8,7 @@ namespace ff {
 
 template <class T>
 void spmm_hm_raw(cudaStream_t st, const long long* ptr, const int* col, const T* val, long long n,
-                 const T* X, int ldx, T* YH, T* YM, int ldy, int m);
+                 const T* X, int ldx, T* YH, T* YM, int ldy, int m, bool diff = false);
 
 void cheb_step(cudaStream_t st, const long long* ptr, const int* col, const float* hv,
                const float* hdiag, long long n, int m, int ld, const float* din, float* dout,

@@ -67,6 +67,23 @@ __global__ void k_scatter_block(const T* __restrict__ X, int ld, long long n, in
   out[(long long)(c + col0) * ldo + perm[r]] = (To)X[r * ld + c];
 }
 
+// two panels to the caller's order at once (either output may be NULL); nothing
+// is written when flags (if given) hold an error
+template <class T>
+__global__ void k_scatter_blocks(const T* __restrict__ A, const T* __restrict__ B, int ld,
+                                 long long n, int m, const int* __restrict__ perm,
+                                 T* __restrict__ outA, T* __restrict__ outB,
+                                 const DevFlags* __restrict__ flags) {
+  if (flags && flags->code != 0) return;
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n * m) return;
+  const long long r = t / m;
+  const int c = (int)(t % m);
+  const long long o = (long long)c * n + perm[r];
+  if (outA) outA[o] = A[r * ld + c];
+  if (outB) outB[o] = B[r * ld + c];
+}
+
 template <class T>
 __global__ void k_fill(T* x, long long n, T v) {
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1028,12 +1045,19 @@ ff_status run_eigenmodes(ff_ctx* c, int k, const ff_eig_opts& o, const void* X0,
 }
 
 template <class T>
-void spmm_hm(ff_ctx* c, const T* X, int ldx, T* YH, T* YM, int ldy, int m) {
-  spmm_hm_raw<T>(c->stream, c->a_ptr.as<long long>(), c->a_col.as<int>(), c->a_val.as<T>(), c->n,
-                 X, ldx, YH, YM, ldy, m);
+void spmm_hm(ff_ctx* c, const T* X, T* YH, T* YM, int ld, int m) {
+  // FP64 blocks of whole fours keep the summed form of their kernel, others the
+  // difference form they had in the general kernel; wide blocks go in the widest
+  // pieces the vector kernels take
+  const bool diff = sizeof(T) == 8 && m % 4 != 0;
+  const int piece = sizeof(T) == 4 || !diff ? 128 : 64;
+  const int cols = ld > m ? ld : m;
+  for (int c0 = 0; c0 < cols; c0 += piece)
+    spmm_hm_raw<T>(c->stream, c->a_ptr.as<long long>(), c->a_col.as<int>(), c->a_val.as<T>(), c->n,
+                   X + c0, ld, YH + c0, YM + c0, ld, std::min(piece, cols - c0), diff);
 }
-template void spmm_hm<float>(ff_ctx*, const float*, int, float*, float*, int, int);
-template void spmm_hm<double>(ff_ctx*, const double*, int, double*, double*, int, int);
+template void spmm_hm<float>(ff_ctx*, const float*, float*, float*, int, int);
+template void spmm_hm<double>(ff_ctx*, const double*, double*, double*, int, int);
 
 // caller-order column-major block <-> internal row-major panel (used by ff_apply_operators)
 template <class T>
@@ -1043,14 +1067,18 @@ void gather_block(ff_ctx* c, const T* X0, int m, T* X, int ld) {
   FF_LAUNCH_CHECK();
 }
 template <class T>
-void scatter_block(ff_ctx* c, const T* X, int ld, int m, T* out) {
-  (k_scatter_block<T><<<(unsigned)((c->n * m + 255) / 256), 256, 0, c->stream>>>(
-      X, ld, c->n, m, c->perm.as<int>(), out, c->n, 0), ::ff::note_launch());
+void scatter_blocks(ff_ctx* c, const T* A, const T* B, int ld, int m, T* outA, T* outB,
+                    const DevFlags* flags) {
+  if (!outA && !outB) return;
+  (k_scatter_blocks<T><<<(unsigned)((c->n * m + 255) / 256), 256, 0, c->stream>>>(
+      A, B, ld, c->n, m, c->perm.as<int>(), outA, outB, flags), ::ff::note_launch());
   FF_LAUNCH_CHECK();
 }
 template void gather_block<float>(ff_ctx*, const float*, int, float*, int);
 template void gather_block<double>(ff_ctx*, const double*, int, double*, int);
-template void scatter_block<float>(ff_ctx*, const float*, int, int, float*);
-template void scatter_block<double>(ff_ctx*, const double*, int, int, double*);
+template void scatter_blocks<float>(ff_ctx*, const float*, const float*, int, int, float*, float*,
+                                    const DevFlags*);
+template void scatter_blocks<double>(ff_ctx*, const double*, const double*, int, int, double*,
+                                     double*, const DevFlags*);
 
 }  // namespace ff

@@ -28,7 +28,8 @@ namespace ff {
 template <class T>
 void gather_block(ff_ctx* c, const T* X0, int m, T* X, int ld);
 template <class T>
-void scatter_block(ff_ctx* c, const T* X, int ld, int m, T* out);
+void scatter_blocks(ff_ctx* c, const T* A, const T* B, int ld, int m, T* outA, T* outB,
+                    const DevFlags* flags = nullptr);
 }  // namespace ff
 
 namespace {
@@ -75,7 +76,11 @@ extern "C" ff_status ff_apply_operators_noalloc(ff_ctx* c, const void* X, int m,
     FF_REQUIRE(c->stage >= 2, FF_ERR_STATE, "matrices not assembled");
     FF_REQUIRE(X && m >= 1 && m <= 512, FF_ERR_INVALID_ARG, "bad block");
     const size_t esz = c->prec == FF_PREC_FP64 ? 8 : 4;
-    const size_t panel = ((size_t)c->n * m * esz + 255) / 256 * 256;
+    auto panel_of = [&](int ld) { return ((size_t)c->n * ld * esz + 255) / 256 * 256; };
+    // rows of whole 16 bytes while the three panels still fit
+    int ld = esz == 8 ? ff::spmm_ld<double>(m) : ff::spmm_ld<float>(m);
+    if (3 * panel_of(ld) > kStaticScratchBytes) ld = m;
+    const size_t panel = panel_of(ld);
     if (3 * panel > kStaticScratchBytes)
       throw ff::Error(FF_ERR_INVALID_ARG,
                       "block too large for the static scratch: n * m * " + std::to_string(esz) +
@@ -87,10 +92,9 @@ extern "C" ff_status ff_apply_operators_noalloc(ff_ctx* c, const void* X, int m,
       T* in = reinterpret_cast<T*>(base);
       T* oh = reinterpret_cast<T*>(base + panel);
       T* om = reinterpret_cast<T*>(base + 2 * panel);
-      ff::gather_block<T>(c, static_cast<const T*>(X), m, in, m);
-      ff::spmm_hm<T>(c, in, m, oh, om, m, m);
-      if (YH) ff::scatter_block<T>(c, oh, m, m, static_cast<T*>(YH));
-      if (YM) ff::scatter_block<T>(c, om, m, m, static_cast<T*>(YM));
+      ff::gather_block<T>(c, static_cast<const T*>(X), m, in, ld);
+      ff::spmm_hm<T>(c, in, oh, om, ld, m);
+      ff::scatter_blocks<T>(c, oh, om, ld, m, static_cast<T*>(YH), static_cast<T*>(YM));
       FF_CUDA(cudaStreamSynchronize(c->stream));
     };
     if (c->prec == FF_PREC_FP64)
