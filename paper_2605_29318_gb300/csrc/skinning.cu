@@ -30,54 +30,126 @@ void gather_block(ff_ctx* c, const T* X0, int m, T* X, int ld);
 
 namespace {
 
-// MODE 0: count the nodes covering each query point; MODE 1: list them.  One
-// warp a point, a lane a cell; a lane tests up to 32 nodes of its cell a round,
-// and the list takes each round's hits in cell order, then node order
-// (deterministic).  A thread a point (27 dependent walks, 1.3 blocks an SM at
-// 50,000 points) took 306 us a pass, 125 us now.
-template <int MODE>
-__global__ void __launch_bounds__(256)
-    k_query_search(const float* __restrict__ Q, long long nq, const float4* __restrict__ pos,
-                   GridDev g, const int* __restrict__ cstart, int* __restrict__ cnt,
-                   const long long* __restrict__ qptr, int* __restrict__ qidx) {
-  const long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (q >= nq) return;
-  const int lane = threadIdx.x & 31;
-  const float4 X = make_float4(Q[3 * q], Q[3 * q + 1], Q[3 * q + 2], 0.f);
-  const int x = cell_coord(X.x, g.o0, g.h, g.d0) + lane % 3 - 1;
-  const int y = cell_coord(X.y, g.o1, g.h, g.d1) + lane / 3 % 3 - 1;
-  const int z = cell_coord(X.z, g.o2, g.h, g.d2) + lane / 9 - 1;
-  int i = 0, end = 0;
+// A warp takes kQueries points, whose cells it finds at once, a lane a coordinate:
+// the FP64 division of a cell coordinate costs a warp the same for one lane as for
+// 32.
+constexpr int kQueries = 8;
+
+__device__ __forceinline__ int query_coords(const float* __restrict__ Q, long long q0,
+                                            long long nq, const GridDev& g, int lane) {
+  const int d = lane % 3;
+  const long long q = q0 + lane / 3;
+  if (lane >= 3 * kQueries || q >= nq) return 0;
+  return cell_coord(Q[3 * q + d], d == 0 ? g.o0 : d == 1 ? g.o1 : g.o2, g.h,
+                    d == 0 ? g.d0 : d == 1 ? g.d1 : g.d2);
+}
+
+// the cell this lane searches for point u of the warp: nodes [i, end)
+__device__ __forceinline__ void query_cell(int coords, int u, const GridDev& g,
+                                           const int* __restrict__ cstart, int lane, int& i,
+                                           int& end) {
+  const int x = __shfl_sync(0xffffffffu, coords, 3 * u) + lane % 3 - 1;
+  const int y = __shfl_sync(0xffffffffu, coords, 3 * u + 1) + lane / 3 % 3 - 1;
+  const int z = __shfl_sync(0xffffffffu, coords, 3 * u + 2) + lane / 9 - 1;
+  i = end = 0;
   if (lane < 27 && x >= 0 && x < g.d0 && y >= 0 && y < g.d1 && z >= 0 && z < g.d2) {
     const long long key = cell_key(g, x, y, z);
     i = cstart[key];
     end = cstart[key + 1];
   }
-  int c = 0;
-  long long base = MODE ? qptr[q] : 0;
-  while (__any_sync(0xffffffffu, i < end)) {
-    const int n = min(end - i, 32);
-    unsigned hit = 0;
-    for (int u = 0; u < n; ++u) hit |= (unsigned)covers(X, pos[i + u]) << u;
-    const int h = __popc(hit);
-    if (MODE) {
-      int off = h;
+}
+
+// a round's hits to the list, in cell order then node order; base moves on
+__device__ __forceinline__ void query_put(unsigned hit, int i, int lane, long long& base,
+                                          int* __restrict__ qidx) {
+  const int h = __popc(hit);
+  int off = h;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, off, o);
-        if (lane >= o) off += t;
-      }
-      long long at = base + off - h;
-      base += __shfl_sync(0xffffffffu, off, 31);
-      for (unsigned b = hit; b; b &= b - 1) qidx[at++] = i + __ffs(b) - 1;
-    } else {
-      c += h;
-    }
-    i += max(n, 0);
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, off, o);
+    if (lane >= o) off += t;
   }
-  if (!MODE) {
-    c = __reduce_add_sync(0xffffffffu, c);
-    if (lane == 0) cnt[q] = c;
+  long long at = base + off - h;
+  base += __shfl_sync(0xffffffffu, off, 31);
+  for (unsigned b = hit; b; b &= b - 1) qidx[at++] = i + __ffs(b) - 1;
+}
+
+// MODE 0: count the nodes covering each query point, and keep the hits of its
+// first kMaskRounds rounds (masks, 32 words a round; the last word of a point's
+// first round is the number of rounds); MODE 1: list them, from the masks where they
+// hold all the rounds.  A lane a cell tests up to 32 of its nodes a round
+// (deterministic: rounds, then cells, then nodes).  A cell's edge is the largest
+// support, so 27 cells hold ~250 nodes, ~900 where supports are uneven; bound by a
+// load's 27 sectors.  A thread a point took 306 us a pass for 50,000 points of the
+// latter kind, this 126 + 36 us; half warps on consecutive nodes, two cells at a
+// time, 127 + 70 us.
+constexpr int kMaskRounds = 3;
+
+template <int MODE>
+__global__ void __launch_bounds__(256)
+    k_query_search(const float* __restrict__ Q, long long nq, const float4* __restrict__ pos,
+                   GridDev g, const int* __restrict__ cstart, int* __restrict__ cnt,
+                   unsigned* __restrict__ masks, const long long* __restrict__ qptr,
+                   int* __restrict__ qidx) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const long long q0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kQueries;
+  if (q0 >= nq) return;
+  const int lane = threadIdx.x & 31;
+  const int coords = query_coords(Q, q0, nq, g, lane);
+  for (int v = 0; v < kQueries && q0 + v < nq; ++v) {
+    const long long q = q0 + v;
+    const float4 X = make_float4(Q[3 * q], Q[3 * q + 1], Q[3 * q + 2], 0.f);
+    int i, end;
+    query_cell(coords, v, g, cstart, lane, i, end);
+    unsigned* mine = masks ? masks + 32LL * kMaskRounds * q : nullptr;
+    long long base = MODE ? qptr[q] : 0;
+    int c = 0, round = 0;
+    if (MODE == 1 && masks) {
+      const int rounds = (int)mine[31];
+      if (rounds <= kMaskRounds) {
+        for (; round < rounds; ++round) {
+          const unsigned hit = mine[32 * round + lane];
+          query_put(lane < 27 ? hit : 0u, i + 32 * round, lane, base, qidx);
+        }
+        continue;
+      }
+    }
+    while (__any_sync(kAll, i < end)) {
+      const int n = min(end - i, 32);
+      unsigned hit = 0, near = 0;
+      for (int u0 = 0; u0 < n; u0 += 4) {
+        float4 p[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) p[u] = pos[min(i + u0 + u, end - 1)];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          // the predicate of covers(): FP32 outside a margin, settled below inside
+          const float dx = X.x - p[u].x, dy = X.y - p[u].y, dz = X.z - p[u].z;
+          const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx)), a2 = p[u].w * p[u].w;
+          if (u0 + u < n) {
+            if (d2 < a2 * 0.99999f) hit |= 1u << (u0 + u);
+            if (d2 <= a2 * 1.00001f) near |= 1u << (u0 + u);
+          }
+        }
+      }
+      for (unsigned b = near & ~hit; b; b &= b - 1) {
+        const int u = __ffs(b) - 1;
+        if (covers(X, pos[i + u])) hit |= 1u << u;
+      }
+      if (MODE) {
+        query_put(hit, i, lane, base, qidx);
+      } else {
+        c += __popc(hit);
+        if (mine && round < kMaskRounds) mine[32 * round + lane] = hit;
+      }
+      ++round;
+      i += max(n, 0);
+    }
+    if (!MODE) {
+      if (mine && lane == 31) mine[31] = (unsigned)round;  // lane 31 has no cell
+      c = __reduce_add_sync(kAll, c);
+      if (lane == 0) cnt[q] = c;
+    }
   }
 }
 
@@ -366,18 +438,26 @@ void weights_t(ff_ctx* c, const float* Q, long long nq, const T* C, int m, T* W)
                      g.bdims[0], g.bdims[1], g.bdims[2]};
     int* cnt = reinterpret_cast<int*>(c->sk_cnt.ensure(sizeof(int) * (nq + 1)));
     long long* ptr = reinterpret_cast<long long*>(c->sk_ptr.ensure(sizeof(long long) * (nq + 1)));
-    (k_query_search<0><<<ceil_div(nq * 32, TB), TB, 0, st>>>(Q, nq, c->pos.as<float4>(), gd,
-                                                             c->cell_start.as<int>(), cnt,
-                                                             nullptr, nullptr),
+    // the hits kept between the passes while they are small; without them the
+    // second pass searches again
+    unsigned* masks = nullptr;
+    const size_t room = sizeof(unsigned) * 32 * kMaskRounds * (size_t)nq;
+    if (room <= (1ull << 30)) {
+      try {
+        masks = reinterpret_cast<unsigned*>(c->scratch[6].ensure(room));
+      } catch (const Error&) {
+      }
+    }
+    (k_query_search<0><<<ceil_div(nq * 32, TB * kQueries), TB, 0, st>>>(
+         Q, nq, c->pos.as<float4>(), gd, c->cell_start.as<int>(), cnt, masks, nullptr, nullptr),
      ::ff::note_launch());
     FF_LAUNCH_CHECK();
     scan_counts(cnt, ptr, nq, c, c->scratch[3]);
     FF_CUDA(cudaMemcpyAsync(&nq1, ptr + nq, sizeof(long long), cudaMemcpyDeviceToHost, st));
     FF_CUDA(cudaStreamSynchronize(st));
     int* idx = reinterpret_cast<int*>(c->sk_idx.ensure(sizeof(int) * std::max(nq1, 1LL)));
-    (k_query_search<1><<<ceil_div(nq * 32, TB), TB, 0, st>>>(Q, nq, c->pos.as<float4>(), gd,
-                                                             c->cell_start.as<int>(), nullptr,
-                                                             ptr, idx),
+    (k_query_search<1><<<ceil_div(nq * 32, TB * kQueries), TB, 0, st>>>(
+         Q, nq, c->pos.as<float4>(), gd, c->cell_start.as<int>(), nullptr, masks, ptr, idx),
      ::ff::note_launch());
     FF_LAUNCH_CHECK();
     qptr = ptr;

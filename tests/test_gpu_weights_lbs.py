@@ -84,3 +84,30 @@ def test_lbs_in_every_read_form(prec, m, nq, shift):
     exact = Q.double() + torch.einsum("qm,mrc,qc->qr", Wd, Zd, h)
     terms = Q.double().abs() + torch.einsum("qm,mrc,qc->qr", Wd.abs(), Zd.abs(), h.abs())
     assert bool(((x - exact).abs() <= (m + 6) * EPS[prec] * terms).all())
+
+
+@pytest.mark.parametrize("crowd", [0, 40, 130])
+def test_query_lists_in_and_past_the_kept_rounds(crowd):
+    """Weights at the particles are phi C of the build's own lists: with cells of
+    about ten nodes, of some forty (two rounds of 32) and of more than three rounds'
+    worth, which are searched twice.  The bound of the lane-split test."""
+    import torch
+    from paper_2605_29318_gb300 import binding
+    c = synth.unit_cube(1500, seed=12)
+    rng = np.random.default_rng(crowd)
+    near = (0.5 + 0.02 * rng.standard_normal((crowd, 3))).astype(np.float32)
+    X = np.concatenate([c.X, near])
+    v = np.concatenate([c.v, np.full(crowd, 1e-6, np.float32)])
+    a = np.concatenate([c.a, np.full(crowd, 0.1, np.float32)])
+    a = synth.support_floor(X, a, factor=1.5)
+    ctx = binding.Context(0, "fp64")
+    ctx.rkpm_build(*(torch.from_numpy(x).to(DEV) for x in (X, v, a)))
+    ptr, idx, phi, _ = ctx.export_rkpm()
+    C = torch.randn(len(X), 7, device=DEV, dtype=torch.float64,
+                    generator=torch.Generator(device=DEV).manual_seed(crowd))
+    W = ctx.skinning_weights(torch.from_numpy(X).to(DEV), C).cpu().numpy()
+    Cd = C.cpu().numpy()
+    for q in range(len(X)):
+        s = slice(ptr[q], ptr[q + 1])
+        bound = 1e3 * 2.0 ** -47 * (np.abs(phi[s]) @ np.abs(Cd[idx[s]]))
+        assert (np.abs(W[q] - phi[s] @ Cd[idx[s]]) <= bound).all(), q
