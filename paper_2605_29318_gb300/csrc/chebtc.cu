@@ -180,18 +180,31 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, unsigned
 // w, w + WB, ...: three staging buffers per warp keep the union rows of two
 // later steps in flight while a step is multiplied (their union columns and
 // A fragments loaded earlier still).  The warps' partial 16 x m products are
-// summed through the same shared memory and each warp finishes a share of the
-// column tiles: res -= D^-1 (H d), d' = c1 d + c2 res (BF16), x += d'.
+// summed through the same shared memory, then res -= D^-1 (H d),
+// d' = c1 d + c2 res (BF16), x += d'.
 // WB = 4 where the row blocks fill the GPU; WB = 16 where they are few (a
 // K x K pencil of a two-set cloud: 63 row blocks for K = 1,000), so that each
 // warp's chain of k-steps is four times shorter.
+// Bound by the latency of its chains (a warp has about seven k-steps): the block's
+// own rows of res, x and d therefore come with the third step's group and are
+// finished as the contiguous run they are, 64 registers let eight blocks share an
+// SM, and a step's kernel starts while the one before drains, reading its tables
+// before it waits for that one's vectors.  50,000 rows, 40 columns: 31.7 us a step
+// without these, 27.2 so, and 3 us less between steps.  Gathers that keep lines in
+// L1 (29.5 us), and two (30.8) or four (33.1) row blocks in a block to share them,
+// were slower.
+__host__ __device__ constexpr size_t tc_rows_bytes(int NT) { return (size_t)kTcRows * (8 * NT * 10 + 8); }
+__host__ __device__ constexpr int tc_red_ld(int NT) { return 8 * NT + (NT % 2 ? 0 : 8); }  // conflict-free for 8 rows
+
 template <int WB>
 constexpr size_t tc_step_smem(int NT) {
-  return std::max<size_t>((size_t)WB * 3 * kTcRows * 8 * NT * 2, (size_t)WB * 32 * 4 * NT * 4);
+  return std::max<size_t>((size_t)WB * 3 * kTcRows * 8 * NT * 2,
+                          (size_t)WB * kTcRows * tc_red_ld(NT) * 4) +
+         tc_rows_bytes(NT);
 }
 
 template <int NT, int WB>
-__global__ void __launch_bounds__(32 * WB)
+__global__ void __launch_bounds__(32 * WB, WB == 4 && NT <= 5 ? 8 : 1)
     k_cheb_step_tc(const int* __restrict__ kofs, const int* __restrict__ ucol,
                    const uint4* __restrict__ tile, const float* __restrict__ hs,
                    const float* __restrict__ hdiag, int n, const __nv_bfloat16* __restrict__ din,
@@ -199,10 +212,19 @@ __global__ void __launch_bounds__(32 * WB)
                    float* __restrict__ res, float c1, float c2) {
   constexpr int kWB = WB;
   constexpr int m = 8 * NT, PIECES = kTcRows * NT, ITERS = (PIECES + 31) / 32, NB = 3;
+  constexpr int P = tc_red_ld(NT);
   extern __shared__ __align__(16) unsigned char smem[];
   const int b = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __nv_bfloat16* stage = reinterpret_cast<__nv_bfloat16*>(smem) + w * NB * kTcRows * m;
+  // the block's own rows of res, x and d, and 1 / diagonal and row sum of each row
+  float* own_r = reinterpret_cast<float*>(smem);
+  float* own_x = own_r + kTcRows * m;
+  __nv_bfloat16* own_d = reinterpret_cast<__nv_bfloat16*>(own_x + kTcRows * m);
+  float* own_h = reinterpret_cast<float*>(own_d + kTcRows * m);
+  unsigned char* work = smem + tc_rows_bytes(NT);
+  __nv_bfloat16* stage = reinterpret_cast<__nv_bfloat16*>(work) + w * NB * kTcRows * m;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int s0 = kofs[b], ns = kofs[b + 1] - s0;
+  const int k0 = b * kTcRows, nrow = min(kTcRows, n - k0);
   float acc[NT][4];
 #pragma unroll
   for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
@@ -227,13 +249,29 @@ __global__ void __launch_bounds__(32 * WB)
   // columns of the step staged in phase p; each is reloaded right after use
   // for the step three phases on.
   int s = w;
-  if (s < ns) stage_step(0, ucol_of(s));
-  cp_commit();
-  if (s + kWB < ns) stage_step(1, ucol_of(s + kWB));
-  cp_commit();
+  const int u0 = ucol_of(s), u1 = ucol_of(s + kWB);
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
   uint4 A[3] = {tile_of(s, zero4), tile_of(s + kWB, zero4), tile_of(s + 2 * kWB, zero4)};
   int U[3] = {ucol_of(s + 2 * kWB), ucol_of(s + 3 * kWB), ucol_of(s + 4 * kWB)};
+  if (threadIdx.x < nrow) {
+    own_h[threadIdx.x] = 1.0f / hdiag[k0 + threadIdx.x];
+    own_h[kTcRows + threadIdx.x] = hs[k0 + threadIdx.x];
+  }
+  // only the vectors come from the step before
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (s < ns) stage_step(0, u0);
+  cp_commit();
+  if (s + kWB < ns) stage_step(1, u1);
+  cp_commit();
+  {  // in the group of the third step
+    const long long o = (long long)k0 * m;
+    for (int q = threadIdx.x; q < nrow * (m / 4); q += 32 * kWB) {
+      cp_async16(own_r + 4 * q, res + o + 4 * q);
+      cp_async16(own_x + 4 * q, x + o + 4 * q);
+    }
+    for (int q = threadIdx.x; q < nrow * NT; q += 32 * kWB)
+      cp_async16(own_d + 8 * q, din + o + 8 * q);
+  }
   auto phase = [&](const int p) {
     if (s + 2 * kWB < ns) stage_step((p + 2) % 3, U[p]);
     cp_commit();
@@ -275,45 +313,41 @@ __global__ void __launch_bounds__(32 * WB)
   }
   cp_wait0();
   __syncthreads();  // every warp is done with its staging buffers
-  float* red = reinterpret_cast<float*>(smem);  // [kWB][32][4 NT]
+  float* red = reinterpret_cast<float*>(work);  // [kWB][16][P]
+  const int g = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int j = 0; j < NT; ++j)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) red[(w * 32 + lane) * 4 * NT + 4 * j + q] = acc[j][q];
+    for (int h = 0; h < 2; ++h)
+      *reinterpret_cast<float2*>(red + (w * kTcRows + g + 8 * h) * P + 8 * j + 2 * t) =
+          make_float2(acc[j][2 * h], acc[j][2 * h + 1]);
   __syncthreads();
-  // warp w finishes the column tiles j = w, w + kWB, ...
-  const int g = lane >> 2, t = lane & 3;
-  for (int j = w; j < NT; j += kWB) {
-    float c[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float t = 0.f;
-      for (int v = 0; v < kWB; ++v) t += red[(v * 32 + lane) * 4 * NT + 4 * j + q];
-      c[q] = t;
+  // the block's rows are contiguous: a thread takes pairs of columns of them
+  for (int e = threadIdx.x; e < nrow * (m / 2); e += 32 * kWB) {
+    const int row = e / (m / 2), col = 2 * (e % (m / 2));
+    float2 c = make_float2(0.f, 0.f);
+    for (int v = 0; v < kWB; ++v) {
+      const float2 p = *reinterpret_cast<const float2*>(red + (v * kTcRows + row) * P + col);
+      c.x += p.x;
+      c.y += p.y;
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = b * kTcRows + g + 8 * h;
-      if (k >= n) continue;
-      const float dinv = 1.0f / hdiag[k], hsk = hs[k];
-      const long long o = (long long)k * m + 8 * j + 2 * t;
-      const __nv_bfloat162 dk2 = *reinterpret_cast<const __nv_bfloat162*>(din + o);
-      const float2 dk = __bfloat1622float2(dk2);
-      float2 r = *reinterpret_cast<const float2*>(res + o);
-      float2 xx = *reinterpret_cast<const float2*>(x + o);
-      r.x -= (c[2 * h] - hsk * dk.x) * dinv;
-      r.y -= (c[2 * h + 1] - hsk * dk.y) * dinv;
-      const __nv_bfloat16 q0 = __float2bfloat16(c1 * dk.x + c2 * r.x);
-      const __nv_bfloat16 q1 = __float2bfloat16(c1 * dk.y + c2 * r.y);
-      xx.x += __bfloat162float(q0);
-      xx.y += __bfloat162float(q1);
-      *reinterpret_cast<float2*>(res + o) = r;
-      *reinterpret_cast<float2*>(x + o) = xx;
-      __nv_bfloat162 qq;
-      qq.x = q0;
-      qq.y = q1;
-      *reinterpret_cast<__nv_bfloat162*>(dout + o) = qq;
-    }
+    const float dinv = own_h[row], hsk = own_h[kTcRows + row];
+    const float2 dk = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(own_d)[e]);
+    float2 r = reinterpret_cast<const float2*>(own_r)[e];
+    float2 xx = reinterpret_cast<const float2*>(own_x)[e];
+    r.x -= (c.x - hsk * dk.x) * dinv;
+    r.y -= (c.y - hsk * dk.y) * dinv;
+    const __nv_bfloat16 q0 = __float2bfloat16(c1 * dk.x + c2 * r.x);
+    const __nv_bfloat16 q1 = __float2bfloat16(c1 * dk.y + c2 * r.y);
+    xx.x += __bfloat162float(q0);
+    xx.y += __bfloat162float(q1);
+    const long long o = (long long)k0 * m + 2 * e;
+    *reinterpret_cast<float2*>(res + o) = r;
+    *reinterpret_cast<float2*>(x + o) = xx;
+    __nv_bfloat162 qq;
+    qq.x = q0;
+    qq.y = q1;
+    *reinterpret_cast<__nv_bfloat162*>(dout + o) = qq;
   }
 }
 
@@ -553,23 +587,31 @@ bool cheb_step_tc(cudaStream_t st, const ff_ctx* c, int m, const void* din, void
   const bool few = nblk < 2 * sm_count();
   auto go = [&](auto nt) {
     constexpr int NT = decltype(nt)::value;
-    if (few) {
-      const size_t sm = tc_step_smem<16>(NT);
-      set_max_dyn_smem((const void*)k_cheb_step_tc<NT, 16>, (int)sm);
-      (k_cheb_step_tc<NT, 16><<<nblk, 32 * 16, sm, st>>>(
-           c->tc_kofs.as<int>(), c->tc_ucol.as<int>(),
-           reinterpret_cast<const uint4*>(c->tc_tile.p), c->tc_hs.as<float>(),
-           c->hdiag_f32.as<float>(), (int)c->n, bi, bo, x, res, c1, c2),
-       ::ff::note_launch());
-    } else {
-      const size_t sm = tc_step_smem<4>(NT);
-      set_max_dyn_smem((const void*)k_cheb_step_tc<NT, 4>, (int)sm);
-      (k_cheb_step_tc<NT, 4><<<nblk, 32 * 4, sm, st>>>(
-           c->tc_kofs.as<int>(), c->tc_ucol.as<int>(),
-           reinterpret_cast<const uint4*>(c->tc_tile.p), c->tc_hs.as<float>(),
-           c->hdiag_f32.as<float>(), (int)c->n, bi, bo, x, res, c1, c2),
-       ::ff::note_launch());
-    }
+    // a step's tables are fetched while the step before it drains
+    cudaLaunchAttribute early;
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nblk);
+    cfg.stream = st;
+    cfg.attrs = &early;
+    cfg.numAttrs = 1;
+    auto launch = [&](auto fn, int warps, size_t sm) {
+      set_max_dyn_smem((const void*)fn, (int)sm);
+      cfg.blockDim = dim3(32 * warps);
+      cfg.dynamicSmemBytes = sm;
+      FF_CUDA(cudaLaunchKernelEx(&cfg, fn, (const int*)c->tc_kofs.as<int>(),
+                                 (const int*)c->tc_ucol.as<int>(),
+                                 reinterpret_cast<const uint4*>(c->tc_tile.p),
+                                 (const float*)c->tc_hs.as<float>(),
+                                 (const float*)c->hdiag_f32.as<float>(), (int)c->n, bi, bo, x, res,
+                                 c1, c2));
+      ::ff::note_launch();
+    };
+    if (few)
+      launch(k_cheb_step_tc<NT, 16>, 16, tc_step_smem<16>(NT));
+    else
+      launch(k_cheb_step_tc<NT, 4>, 4, tc_step_smem<4>(NT));
   };
 #define FF_TC(NT) go(std::integral_constant<int, NT>{})
   switch (m / 8) {
