@@ -654,17 +654,28 @@ __global__ void __launch_bounds__(32 * kRedWarps)
 }
 
 // C = beta C + A Y for blocks with p, q, lda, ldc, split, off2 multiples of 4:
-// each thread computes a 4 x 4 register block (4 consecutive rows, 4
+// each thread computes an RR x 4 register block (RR consecutive rows, 4
 // consecutive output columns) from 16-byte row loads of A and of the Y tile
 // staged in shared memory; TD = TW / 4 threads span a TW-column tile and
 // RG = 256 / TD row groups share a block.  Columns at or past `split` are
-// written at off2 + (j - split).
-template <class T, int TW>
+// written at off2 + (j - split).  blockIdx.z: one of up to three pairs of A and C
+// under the same Y (the same sums whatever RR and the pairs).  Bound by the latency
+// of a thread's walk along its rows where the blocks do not fill the GPU: fewer rows
+// a thread there, and the pairs beside each other.  1,000 rows, 216 columns to 144:
+// three pairs 96 us in FP32 one after the other at four rows a thread, 31 us together
+// at one; 3,000 rows, 60 columns to 40: 41 and 12.8 us.
+template <class T>
+struct UpdatePairs {
+  const T* a[3];
+  T* c[3];
+};
+template <class T, int TW, int RR>
 __global__ void __launch_bounds__(256)
-    k_block_update_rt(const T* __restrict__ A, int lda, int p, const T* __restrict__ Y, int ldy,
-                      int q, T* __restrict__ C, int ldc, long long n, T beta, int split,
-                      int off2) {
-  constexpr int TD = TW / 4, RG = 256 / TD, RR = 4;
+    k_block_update_rt(UpdatePairs<T> pairs, int lda, int p, const T* __restrict__ Y, int ldy,
+                      int q, int ldc, long long n, T beta, int split, int off2) {
+  constexpr int TD = TW / 4, RG = 256 / TD;
+  const T* __restrict__ A = pairs.a[blockIdx.z];
+  T* __restrict__ C = pairs.c[blockIdx.z];
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sy = reinterpret_cast<T*>(smraw);  // p x TW
   const int c0 = blockIdx.y * TW;
@@ -1435,8 +1446,8 @@ void gram_rr(cudaStream_t st, const T* S, const T* HS, const T* MS, int ld, int 
 }
 
 template <class T>
-void block_update(cudaStream_t st, const T* A, int lda, int p, const T* Y, int q, T* C, int ldc,
-                  long long n, T beta, int split, int off2, int ldy) {
+void block_updates(cudaStream_t st, int pairs, const T* const* A, T* const* C, int lda, int p,
+                   const T* Y, int q, int ldc, long long n, T beta, int split, int off2, int ldy) {
   if (q <= 0 || n <= 0) return;
   ProfScope ps(kProfUpdate);
   if (p <= 0) {
@@ -1446,25 +1457,48 @@ void block_update(cudaStream_t st, const T* A, int lda, int p, const T* Y, int q
   const bool w40 = q % 40 == 0;
   const int TW = w40 ? 40 : 32;
   size_t smem = sizeof(T) * (size_t)p * TW;
-  const int sp = split < 0 ? q : split;
+  const int sp = split < 0 ? q : split, ly = ldy < 0 ? q : ldy;
+  bool al = true;
+  for (int i = 0; i < pairs; ++i) al = al && al16(A[i]) && al16(C[i]);
+  if (!al && pairs > 1) {  // each by its own alignment
+    for (int i = 0; i < pairs; ++i)
+      block_updates<T>(st, 1, A + i, C + i, lda, p, Y, q, ldc, n, beta, split, off2, ldy);
+    return;
+  }
   if (p % 4 == 0 && q % 4 == 0 && lda % 4 == 0 && ldc % 4 == 0 && sp % 4 == 0 && off2 % 4 == 0 &&
-      al16(A) && al16(C) && smem <= 200 * 1024) {
-    if (smem > 48 * 1024)
-      set_max_dyn_smem(w40 ? (const void*)k_block_update_rt<T, 40>
-                           : (const void*)k_block_update_rt<T, 32>,
-                       200 * 1024);
+      al && smem <= 200 * 1024) {
+    UpdatePairs<T> up = {};
+    for (int i = 0; i < pairs; ++i) {
+      up.a[i] = A[i];
+      up.c[i] = C[i];
+    }
     const int TD = TW / 4, RG = 256 / TD;
-    const long long rows_per_block = (long long)RG * 4;
-    dim3 grid((unsigned)std::min<long long>((n + rows_per_block - 1) / rows_per_block, (long long)sm_count() * 8),
-              (unsigned)((q + TW - 1) / TW));
+    const unsigned tiles = (unsigned)((q + TW - 1) / TW);
+    auto go = [&](auto tw, auto rr) {
+      constexpr int W = decltype(tw)::value, RR = decltype(rr)::value;
+      if (smem > 48 * 1024) set_max_dyn_smem((const void*)k_block_update_rt<T, W, RR>, 200 * 1024);
+      const long long per = (long long)RG * RR;
+      dim3 grid((unsigned)std::min<long long>((n + per - 1) / per, (long long)sm_count() * 8), tiles,
+                (unsigned)pairs);
+      (k_block_update_rt<T, W, RR><<<grid, TD * RG, smem, st>>>(up, lda, p, Y, ly, q, ldc, n, beta,
+                                                               sp, off2),
+       ::ff::note_launch());
+    };
+    auto rows = [&](auto tw) {
+      const long long four = (n + RG * 4 - 1) / (RG * 4) * tiles * pairs;
+      // blocks at four rows a thread: with less than one an SM one row is the
+      // fastest (above), from two on four (a tile of Y is read for more rows)
+      if (four < sm_count())
+        go(tw, std::integral_constant<int, 1>{});
+      else if (four < 2 * sm_count())
+        go(tw, std::integral_constant<int, 2>{});
+      else
+        go(tw, std::integral_constant<int, 4>{});
+    };
     if (w40)
-      (k_block_update_rt<T, 40><<<grid, TD * RG, smem, st>>>(A, lda, p, Y, ldy < 0 ? q : ldy, q, C,
-                                                            ldc, n, beta, sp, off2),
-       ::ff::note_launch());
+      rows(std::integral_constant<int, 40>{});
     else
-      (k_block_update_rt<T, 32><<<grid, TD * RG, smem, st>>>(A, lda, p, Y, ldy < 0 ? q : ldy, q, C,
-                                                            ldc, n, beta, sp, off2),
-       ::ff::note_launch());
+      rows(std::integral_constant<int, 32>{});
     FF_LAUNCH_CHECK();
     return;
   }
@@ -1474,15 +1508,23 @@ void block_update(cudaStream_t st, const T* A, int lda, int p, const T* Y, int q
                      227 * 1024);
   dim3 grid((unsigned)std::min<long long>((n + rpb - 1) / rpb, (long long)sm_count() * 16),
             (unsigned)((q + TW - 1) / TW));
-  if (w40)
-    (k_block_update<T, 40><<<grid, 40 * rpb, smem, st>>>(A, lda, p, Y, ldy < 0 ? q : ldy, q, C,
-                                                        ldc, n, beta, split < 0 ? q : split, off2),
-     ::ff::note_launch());
-  else
-    (k_block_update<T, 32><<<grid, 32 * rpb, smem, st>>>(A, lda, p, Y, ldy < 0 ? q : ldy, q, C,
-                                                        ldc, n, beta, split < 0 ? q : split, off2),
-     ::ff::note_launch());
-  FF_LAUNCH_CHECK();
+  for (int i = 0; i < pairs; ++i) {
+    if (w40)
+      (k_block_update<T, 40><<<grid, 40 * rpb, smem, st>>>(A[i], lda, p, Y, ly, q, C[i], ldc, n,
+                                                          beta, sp, off2),
+       ::ff::note_launch());
+    else
+      (k_block_update<T, 32><<<grid, 32 * rpb, smem, st>>>(A[i], lda, p, Y, ly, q, C[i], ldc, n,
+                                                          beta, sp, off2),
+       ::ff::note_launch());
+    FF_LAUNCH_CHECK();
+  }
+}
+
+template <class T>
+void block_update(cudaStream_t st, const T* A, int lda, int p, const T* Y, int q, T* C, int ldc,
+                  long long n, T beta, int split, int off2, int ldy) {
+  block_updates<T>(st, 1, &A, &C, lda, p, Y, q, ldc, n, beta, split, off2, ldy);
 }
 
 template void spmm_hm_raw<float>(cudaStream_t, const long long*, const int*, const float*,
@@ -1497,8 +1539,12 @@ template void gram_rr<float>(cudaStream_t, const float*, const float*, const flo
                              long long, double*, double*, Buf&);
 template void gram_rr<double>(cudaStream_t, const double*, const double*, const double*, int, int,
                               int, long long, double*, double*, Buf&);
+template void block_updates<float>(cudaStream_t, int, const float* const*, float* const*, int, int,
+                            const float*, int, int, long long, float, int, int, int);
 template void block_update<float>(cudaStream_t, const float*, int, int, const float*, int, float*,
                                   int, long long, float, int, int, int);
+template void block_updates<double>(cudaStream_t, int, const double* const*, double* const*, int, int,
+                            const double*, int, int, long long, double, int, int, int);
 template void block_update<double>(cudaStream_t, const double*, int, int, const double*, int,
                                    double*, int, long long, double, int, int, int);
 template void spmm_hm_raw<dfloat>(cudaStream_t, const long long*, const int*, const dfloat*,
@@ -1507,6 +1553,8 @@ template void gram<dfloat>(cudaStream_t, const dfloat*, int, int, const dfloat*,
                            long long, double*, double, bool, Buf&, int);
 template void gram_rr<dfloat>(cudaStream_t, const dfloat*, const dfloat*, const dfloat*, int, int,
                               int, long long, double*, double*, Buf&);
+template void block_updates<dfloat>(cudaStream_t, int, const dfloat* const*, dfloat* const*, int, int,
+                            const dfloat*, int, int, long long, dfloat, int, int, int);
 template void block_update<dfloat>(cudaStream_t, const dfloat*, int, int, const dfloat*, int,
                                    dfloat*, int, long long, dfloat, int, int, int);
 

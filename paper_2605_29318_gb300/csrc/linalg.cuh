@@ -66,6 +66,11 @@ void gram_mirror(cudaStream_t st, double* A, double* B, int ns, int nb);
 template <class T>
 void block_update(cudaStream_t st, const T* A, int lda, int p, const T* Y, int q, T* C, int ldc,
                   long long n, T beta, int split = -1, int off2 = 0, int ldy = -1);
+// the same for `pairs` (at most three) blocks A[i], C[i] under one Y
+template <class T>
+void block_updates(cudaStream_t st, int pairs, const T* const* A, T* const* C, int lda, int p,
+                   const T* Y, int q, int ldc, long long n, T beta, int split = -1, int off2 = 0,
+                   int ldy = -1);
 
 // small dense Rayleigh-Ritz (dense.cu)
 struct RRDims {

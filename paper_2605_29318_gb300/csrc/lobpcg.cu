@@ -868,15 +868,14 @@ ff_status solve(ff_ctx* c, int k, const ff_eig_opts& o, Phase& ph, const T* X0,
     // from X' itself so that the residual seen by the solver is that of the
     // stored X' (updated products drift from the stored block in FP32) -- or,
     // in a phase that hands over well above that drift, updated as well
-    block_update<T>(st, s.S[cur], ld, ns, s.YZ, 2 * nb, s.S[nxt], ld, n, T(0), nb, 2 * nb);
+    const T* from[] = {s.S[cur], s.HS[cur], s.MS[cur]};
     if (ph.update_products) {
-      block_update<T>(st, s.HS[cur], ld, ns, s.YZ, 2 * nb, s.HS[nxt], ld, n, T(0), nb, 2 * nb);
-      block_update<T>(st, s.MS[cur], ld, ns, s.YZ, 2 * nb, s.MS[nxt], ld, n, T(0), nb, 2 * nb);
+      T* to[] = {s.S[nxt], s.HS[nxt], s.MS[nxt]};
+      block_updates<T>(st, 3, from, to, ld, ns, s.YZ, 2 * nb, ld, n, T(0), nb, 2 * nb);
     } else {
-      block_update<T>(st, s.HS[cur], ld, ns, s.YZ + nb, nb, s.HS[nxt] + 2 * nb, ld, n, T(0), -1,
-                      0, 2 * nb);
-      block_update<T>(st, s.MS[cur], ld, ns, s.YZ + nb, nb, s.MS[nxt] + 2 * nb, ld, n, T(0), -1,
-                      0, 2 * nb);
+      T* to[] = {s.HS[nxt] + 2 * nb, s.MS[nxt] + 2 * nb};
+      block_update<T>(st, s.S[cur], ld, ns, s.YZ, 2 * nb, s.S[nxt], ld, n, T(0), nb, 2 * nb);
+      block_updates<T>(st, 2, from + 1, to, ld, ns, s.YZ + nb, nb, ld, n, T(0), -1, 0, 2 * nb);
       s.spmm(s.S[nxt], s.HS[nxt], s.MS[nxt], nb);
     }
     cur = nxt;
