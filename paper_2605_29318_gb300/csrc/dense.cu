@@ -1211,8 +1211,11 @@ __device__ int sturm_bits(const R* d, const R* e2, int n, R x) {
     bp = bits(p);
   }
   int c = (int)((unsigned long long)(bp >> kSign) & 1ull);
+  R dn = d[1], en = e2[0];  // a step ahead (d[n] is e2[0])
   for (int i = 1; i < n; ++i) {
-    R q = fma(d[i] - x, p, -e2[i - 1] * pm);
+    R q = fma(dn - x, p, -en * pm);
+    dn = d[i + 1];
+    en = e2[i];
     I bq = bits(q);
     if ((bq << 1) == 0) {  // a zero minor takes the sign opposite to its predecessor
       q = bp < 0 ? Prec<R>::tiny : -Prec<R>::tiny;
@@ -1238,13 +1241,16 @@ __device__ int sturm_bits<dfloat>(const dfloat* d, const dfloat* e2, int n, dflo
   dfloat pm(1.0f), p = d[0] - x;
   if (p.h == 0.f) p = -Prec<dfloat>::tiny;
   int c = p.h < 0.f;
+  dfloat dn = d[1], en = e2[0];
   for (int i = 1; i < n; ++i) {
-    dfloat q = df_add(df_mul(d[i] - x, p), -df_mul(e2[i - 1], pm));
+    dfloat q = df_add(df_mul(dn - x, p), -df_mul(en, pm));
+    dn = d[i + 1];
+    en = e2[i];
     if (q.h == 0.f) q = p.h < 0.f ? Prec<dfloat>::tiny : -Prec<dfloat>::tiny;
     c += (q.h < 0.f) != (p.h < 0.f);
     pm = p;
     p = q;
-    const int ex = ilogbf(p.h);
+    const int ex = ((__float_as_int(p.h) >> 23) & 0xff) - 127;
     if (ex > 60 || ex < -60) {
       p = scalbn_r(p, -ex);
       pm = scalbn_r(pm, -ex);
@@ -1256,7 +1262,10 @@ __device__ int sturm_bits<dfloat>(const dfloat* d, const dfloat* e2, int n, dflo
 // One block of kEW warps per eigenvalue s: multisection with 32 kEW probes a
 // round, first on FP32 copies of the tridiagonal (cheap bracketing to FP32
 // resolution), then in the working precision from the FP32 bracket widened by
-// its error bound and checked by working-precision counts.
+// its error bound and checked by working-precision counts.  Bound by the latency of a
+// count's recurrence: entries a step ahead and the range test on the head's bits take
+// n = 216 from 189 us to 158 in double-float (70 to 51 in FP32, which brackets it);
+// eight warps, a round less, 167.
 constexpr int kEW = 4;
 template <class R>
 __device__ void multisection(const R* d, const R* e2, int n, int s, R& a, R& b, int max_rounds,
@@ -1353,87 +1362,119 @@ __global__ void __launch_bounds__(32 * kEW)
 }
 
 // ------------------------------------------------------------------ 3b. inverse iteration in shared memory
-// kIV threads per block, one vector each, their LU factors in shared memory
-// (one thread per block: the pivoting branches of different vectors diverge)
-constexpr int kIV = 1;
+// a block of one warp per vector, its LU factors in shared memory.  The
+// factorisation and the substitutions are chains along the tridiagonal matrix that
+// lane 0 follows: bound by the latency of their double-float operations, so the
+// carried entry stays in a register and the next row's factors are loaded a step
+// ahead; what is independent (bounds, reciprocals, scaling) is spread over the lanes.
+// n = 216, 72 vectors: one thread alone 200 us in double-float and 70 in FP32, this
+// 137 and 30, the same bits.
 template <class R>
-__global__ void k_rr_invit_sm(int n, int nb, RRWork<R> w) {
+__global__ void __launch_bounds__(32) k_rr_invit_sm(int n, int nb, RRWork<R> w) {
+  constexpr unsigned kAll = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  R* sm = reinterpret_cast<R*>(sm_raw);
-  const int s = blockIdx.x * kIV + threadIdx.x;
-  R* u = sm + (size_t)threadIdx.x * 6 * n;
-  if (s >= nb) return;
-  R lo = R(0.0), hi = R(0.0);
-  for (int i = 0; i < n; ++i) {
+  R* u = reinterpret_cast<R*>(sm_raw);
+  R* u1 = u + n;
+  R* u2 = u1 + n;
+  R* lm = u2 + n;
+  R* sw = lm + n;  // the off-diagonal first, then 1 where rows were exchanged
+  R* z = sw + n;   // the shifted diagonal first
+  const int s = blockIdx.x, lane = threadIdx.x;
+  R lo = w.dg[0], hi = lo;
+  for (int i = lane; i < n; i += 32) {
     const R r = (i > 0 ? fabs(w.e[i - 1]) : R(0.0)) + (i + 1 < n ? fabs(w.e[i]) : R(0.0));
-    const R a = w.dg[i] - r, b = w.dg[i] + r;
-    if (i == 0 || a < lo) lo = a;
-    if (i == 0 || b > hi) hi = b;
+    lo = fmin(lo, w.dg[i] - r);
+    hi = fmax(hi, w.dg[i] + r);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(kAll, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(kAll, hi, o));
   }
   const R span = fmax(hi - lo, R(1e-30));
   const R tnorm = fmax(fabs(lo - span * R(1e-6)), fabs(hi + span * R(1e-6)));
   const R pivmin = fmax(Prec<R>::tiny, Prec<R>::eps * tnorm * R(1e-6));
-  R* u1 = u + n;
-  R* u2 = u1 + n;
-  R* lm = u2 + n;
-  R* sw = lm + n;
-  R* z = sw + n;
   const R lam = w.lam[s];
   const R shift = lam + Prec<R>::eps * fmax(fabs(lam), span * R(1e-3)) * R(4.0);
-  R a_i = w.dg[0] - shift, b_i = n > 1 ? w.e[0] : R(0.0), c_i = R(0.0);
-  for (int i = 0; i < n - 1; ++i) {
-    const R sub = w.e[i];
-    const R d1 = w.dg[i + 1] - shift;
-    const R e1 = i + 2 < n ? w.e[i + 1] : R(0.0);
-    if (fabs(a_i) >= fabs(sub)) {
-      const R pv = fabs(a_i) < pivmin ? (a_i < R(0.0) ? -pivmin : pivmin) : a_i;
-      const R l = sub / pv;
-      u[i] = pv; u1[i] = b_i; u2[i] = c_i; lm[i] = l; sw[i] = R(0.0);
-      a_i = d1 - l * b_i;
-      b_i = e1 - l * c_i;
-      c_i = R(0.0);
-    } else {
-      const R l = a_i / sub;
-      u[i] = sub; u1[i] = d1; u2[i] = e1; lm[i] = l; sw[i] = R(1.0);
-      const R na = b_i - l * d1, nc = c_i - l * e1;
-      a_i = na;
-      b_i = nc;
-      c_i = R(0.0);
-    }
+  for (int i = lane; i < n; i += 32) {
+    z[i] = w.dg[i] - shift;
+    sw[i] = i + 1 < n ? w.e[i] : R(0.0);
   }
-  u[n - 1] = fabs(a_i) < pivmin ? (a_i < R(0.0) ? -pivmin : pivmin) : a_i;
-  u1[n - 1] = R(0.0);
-  u2[n - 1] = R(0.0);
+  __syncwarp();
+  if (lane == 0) {
+    R a_i = z[0], b_i = sw[0], c_i = R(0.0), sub = b_i;
+    for (int i = 0; i < n - 1; ++i) {
+      const R d1 = z[i + 1], e1 = sw[i + 1];
+      if (fabs(a_i) >= fabs(sub)) {
+        const R pv = fabs(a_i) < pivmin ? (a_i < R(0.0) ? -pivmin : pivmin) : a_i;
+        const R l = sub / pv;
+        u[i] = pv; u1[i] = b_i; u2[i] = c_i; lm[i] = l; sw[i] = R(0.0);
+        a_i = d1 - l * b_i;
+        b_i = e1 - l * c_i;
+      } else {
+        const R l = a_i / sub;
+        u[i] = sub; u1[i] = d1; u2[i] = e1; lm[i] = l; sw[i] = R(1.0);
+        a_i = b_i - l * d1;
+        b_i = c_i - l * e1;
+      }
+      c_i = R(0.0);
+      sub = e1;
+    }
+    u[n - 1] = fabs(a_i) < pivmin ? (a_i < R(0.0) ? -pivmin : pivmin) : a_i;
+  }
+  __syncwarp();
   // the pivots' reciprocals, once: the substitutions below then multiply
-  // (independent divisions here instead of one on every step of the chain)
-  for (int i = 0; i < n; ++i) u[i] = R(1.0) / u[i];
+  for (int i = lane; i < n; i += 32) u[i] = R(1.0) / u[i];
   unsigned int h = 2166136261u ^ (unsigned)s * 16777619u;
   for (int i = 0; i < n; ++i) {
     h = h * 1664525u + 1013904223u;
-    z[i] = R(0.5) + (R)((h >> 8) & 0xffff) / R(65536.0);
+    if ((i & 31) == lane) z[i] = R(0.5) + (R)((h >> 8) & 0xffff) / R(65536.0);
   }
+  __syncwarp();
   for (int iter = 0; iter < 3; ++iter) {
-    for (int i = 0; i < n - 1; ++i) {
-      if (sw[i] != R(0.0)) {
-        const R t = z[i];
-        z[i] = z[i + 1];
-        z[i + 1] = t - lm[i] * z[i];
-      } else {
-        z[i + 1] -= lm[i] * z[i];
+    R nrm = R(0.0);
+    if (lane == 0) {
+      R cur = z[0], zn = z[min(1, n - 1)], ln = lm[0], xn = sw[0];
+      for (int i = 0; i < n - 1; ++i) {
+        const R zi = zn, l = ln;
+        const bool ex = xn != R(0.0);
+        const int nx = min(i + 1, n - 2);
+        zn = z[nx + 1];
+        ln = lm[nx];
+        xn = sw[nx];
+        const R top = ex ? zi : cur, low = ex ? cur : zi;
+        z[i] = top;
+        cur = low - l * top;
+      }
+      // back substitution, the last two rows' entries carried
+      R p1 = cur * u[n - 1], p2 = R(0.0);
+      z[n - 1] = p1;
+      nrm = fabs(p1);
+      const int last = max(n - 2, 0);
+      R tn = z[last], an = u1[last], bn = u2[last], vn = u[last];
+      for (int i = n - 2; i >= 0; --i) {
+        R t = tn;
+        const R a1 = an, a2 = bn, v = vn;
+        const int nx = max(i - 1, 0);
+        tn = z[nx];
+        an = u1[nx];
+        bn = u2[nx];
+        vn = u[nx];
+        t -= a1 * p1;
+        if (i + 2 < n) t -= a2 * p2;
+        p2 = p1;
+        p1 = t * v;
+        z[i] = p1;
+        nrm = fmax(nrm, fabs(p1));
       }
     }
-    for (int i = n - 1; i >= 0; --i) {
-      R t = z[i];
-      if (i + 1 < n) t -= u1[i] * z[i + 1];
-      if (i + 2 < n) t -= u2[i] * z[i + 2];
-      z[i] = t * u[i];
-    }
-    R nrm = R(0.0);
-    for (int i = 0; i < n; ++i) nrm = fmax(nrm, fabs(z[i]));
+    __syncwarp();
+    nrm = __shfl_sync(kAll, nrm, 0);
     const R inv = nrm > R(0.0) ? R(1.0) / nrm : R(1.0);
-    for (int i = 0; i < n; ++i) z[i] *= inv;
+    for (int i = lane; i < n; i += 32) z[i] *= inv;
+    __syncwarp();
   }
-  for (int i = 0; i < n; ++i) w.V[(size_t)i * nb + s] = z[i];
+  for (int i = lane; i < n; i += 32) w.V[(size_t)i * nb + s] = z[i];
 }
 
 // ------------------------------------------------------------------ small dense products over many blocks
@@ -2005,9 +2046,9 @@ void rr_run(cudaStream_t st, const double* A, const double* B, RRDims d, T* YZ, 
        d.ns, d.nb, w, theta),
    ::ff::note_launch());
   FF_LAUNCH_CHECK();
-  const size_t iv_bytes = sizeof(R) * kIV * 6 * n;
+  const size_t iv_bytes = sizeof(R) * 6 * n;
   if (iv_bytes <= kMaxDynSmem) {
-    (k_rr_invit_sm<R><<<(unsigned)((nb + kIV - 1) / kIV), kIV, iv_bytes, st>>>(d.ns, d.nb, w),
+    (k_rr_invit_sm<R><<<(unsigned)nb, 32, iv_bytes, st>>>(d.ns, d.nb, w),
      ::ff::note_launch());
   } else {
     (k_rr_invit<R><<<(unsigned)((nb + 31) / 32), 32, 0, st>>>(d.ns, d.nb, w), ::ff::note_launch());
