@@ -1607,9 +1607,26 @@ __global__ void __launch_bounds__(kThreads) k_rr_cholqr(int n, int nb, RRWork<R>
 // k_rr_backtransform applies the groups, last first, to kBW vectors per
 // block: W = V^T Z, W <- T W, Z -= V W, each a product over the block's
 // threads, so a group costs four block barriers instead of kWY dependent
-// warp reductions per vector.
+// warp reductions per vector.  A group's reflectors and T are copied while the
+// group before is applied (all of it fits shared memory at the largest basis, 1,020
+// columns): with their loads and T's at each group's head n = 216 and 72 vectors took 93 us in FP32
+// and 96 in double-float, so 34 and 44.
 constexpr int kWY = 8;
 constexpr int kBW = 8;
+
+// one entry to shared memory, asynchronously; zero where !in
+template <class R>
+__device__ __forceinline__ void copy_entry(R* dst, const R* src, bool in) {
+  static_assert(sizeof(R) == 4 || sizeof(R) == 8, "cp.async sizes");
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  const unsigned bytes = in ? (unsigned)sizeof(R) : 0u;
+  if constexpr (sizeof(R) == 8)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(bytes)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(bytes)
+                 : "memory");
+}
 
 template <class R>
 __global__ void __launch_bounds__(256) k_rr_wy_t(int n, RRWork<R> w, R* __restrict__ T) {
@@ -1651,25 +1668,41 @@ __global__ void __launch_bounds__(256) k_rr_wy_t(int n, RRWork<R> w, R* __restri
 template <class R>
 __global__ void __launch_bounds__(32 * kBW) k_rr_backtransform(int n, int nb, RRWork<R> w,
                                                                const R* __restrict__ T) {
+  static_assert(kWY == kBW, "a warp copies a reflector");
   extern __shared__ __align__(16) unsigned char z_raw[];
-  R* Z = reinterpret_cast<R*>(z_raw);  // n x kBW: the block's vectors, row-major
-  R* V = Z + (size_t)n * kBW;          // kWY x n: the group's reflectors
-  __shared__ R W[kWY * kBW], W2[kWY * kBW];
-  const int tid = threadIdx.x, s0 = blockIdx.x * kBW;
+  R* Z = reinterpret_cast<R*>(z_raw);   // n x kBW: the block's vectors, row-major
+  R* Vs = Z + (size_t)n * kBW;          // two of kWY x n: a group's reflectors, rows past j0
+  __shared__ R W[kWY * kBW], W2[kWY * kBW], Ts[2][kWY * kWY];
+  const int tid = threadIdx.x, s0 = blockIdx.x * kBW, lane = tid & 31, wid = tid >> 5;
   const int ns = min(kBW, nb - s0);
+  const int ng = n > 2 ? (n - 2 + kWY - 1) / kWY : 0;
+  auto tau_of = [&](int g) {
+    const int j = g * kWY + wid;
+    return g >= 0 && j < n - 2 ? w.tau[j] : R(0.0);
+  };
+  R tau = tau_of(ng - 1);
+  auto fetch = [&](int g, int buf) {  // tau: of reflector wid of group g, then of g - 1
+    const int j0 = g * kWY;
+    const bool on = !(tau == R(0.0));
+    R* v = Vs + ((size_t)buf * kWY + wid) * n;
+    const R* src = w.ref + (size_t)(on ? j0 + wid : j0) * n;
+    for (int l = j0 + 1 + lane; l < n; l += 32) copy_entry(v + l, src + l, on && l > j0 + wid);
+    if (tid < kWY * kWY) copy_entry(&Ts[buf][tid], T + (size_t)g * kWY * kWY + tid, true);
+    tau = tau_of(g - 1);
+  };
+  if (ng > 0) fetch(ng - 1, 0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
   for (int t = tid; t < n * kBW; t += blockDim.x) {
     const int i = t / kBW, s = t - i * kBW;
     Z[t] = s < ns ? w.V[(size_t)i * nb + s0 + s] : R(0.0);
   }
-  const int ng = n > 2 ? (n - 2 + kWY - 1) / kWY : 0;
   for (int g = ng - 1; g >= 0; --g) {
     const int j0 = g * kWY, b = min(kWY, n - 2 - j0);
-    for (int t = tid; t < kWY * n; t += blockDim.x) {
-      const int k = t / n, l = t - k * n;
-      V[t] = (k < b && l >= j0 + k + 1 && !(w.tau[j0 + k] == R(0.0)))
-                 ? w.ref[(size_t)(j0 + k) * n + l]
-                 : R(0.0);
-    }
+    const int buf = (ng - 1 - g) & 1;
+    const R* V = Vs + (size_t)buf * kWY * n;
+    if (g > 0) fetch(g - 1, buf ^ 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
     // W = V^T Z: four threads per entry over rows l = p mod 4
     {
@@ -1684,9 +1717,8 @@ __global__ void __launch_bounds__(32 * kBW) k_rr_backtransform(int n, int nb, RR
     __syncthreads();
     if (tid < kWY * kBW) {  // W <- T W
       const int k = tid / kBW, s = tid - k * kBW;
-      const R* tg = T + (size_t)g * kWY * kWY;
       R acc = R(0.0);
-      for (int m = k; m < b; ++m) acc += tg[k * kWY + m] * W[m * kBW + s];
+      for (int m = k; m < b; ++m) acc += Ts[buf][k * kWY + m] * W[m * kBW + s];
       W2[tid] = acc;
     }
     __syncthreads();
@@ -1734,11 +1766,10 @@ __global__ void __launch_bounds__(kThreads)
     if (lsm)
       for (int t = tid; t < nb * nb; t += kThreads) w.G[t] = G[t];
   }
-  if (tid == 0) {
-    int dc = 0;
-    for (int a = 0; a < n; ++a) dc += !w.keep[a];
-    *dropped = dc;
-  }
+  int dc = 0;
+  for (int a0 = 0; a0 < n; a0 += kThreads)
+    dc += __syncthreads_count(a0 + tid < n && !w.keep[a0 + tid]);
+  if (tid == 0) *dropped = dc;
 }
 
 // Xout <- Xin L^-T for `rows` rows (m entries each; L as block_cholesky
@@ -2095,7 +2126,7 @@ void rr_run(cudaStream_t st, const double* A, const double* B, RRDims d, T* YZ, 
     FF_LAUNCH_CHECK();
   }
   (k_rr_backtransform<R><<<(unsigned)((nb + kBW - 1) / kBW), 32 * kBW,
-                           sizeof(R) * n * (kBW + kWY), st>>>(d.ns, d.nb, w, w.scr),
+                           sizeof(R) * n * (kBW + 2 * kWY), st>>>(d.ns, d.nb, w, w.scr),
    ::ff::note_launch());
   FF_LAUNCH_CHECK();
   if (d.want_p) {  // the momentum step's Grams and Z = Zp - V G over many blocks

@@ -37,3 +37,23 @@ def test_eigenvalues_at_every_basis_size(k):
     ev, _, rep, st = ctx.eigenmodes(k, binding.default_opts(tol=1e-7))
     assert st == 0 and rep["max_residual"] <= 1e-7
     assert np.max(np.abs(ev[1:] - lam[1:k]) / lam[1:k]) < 1e-7
+
+
+def test_a_wide_basis():
+    """876 columns (256 modes, the most that a call may ask for, with 36 guard
+    vectors): the modes, put through the operators, have the residual that was
+    asked for, to a hundredth."""
+    import torch
+    from paper_2605_29318_gb300 import binding
+    c = synth.unit_cube(3100, seed=2)
+    a = synth.support_floor(c.X, c.a, factor=1.5)
+    ctx = binding.Context(0, "fp64")
+    ctx.rkpm_build(*(torch.from_numpy(x).cuda() for x in (c.X, c.v, a)))
+    ctx.assemble_hessian(None, None, c.E, c.nu)
+    ev, modes, rep, st = ctx.eigenmodes(256, binding.default_opts(tol=1e-6, guard=36))
+    assert st == 0 and rep["max_residual"] <= 1e-6
+    x = modes.double()
+    HX, MX = ctx.apply_operators(x)
+    t = torch.from_numpy(ev).to(x)
+    r = (HX - MX * t).norm(dim=0) / (t.abs() * MX.norm(dim=0))
+    assert r[1:].max().item() <= 1.01e-6
