@@ -143,11 +143,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int
 //      (distance, then lowest index), and the next one as its bound,
 //   3. one grid barrier,
 //   4. every block chooses centres among the published points alone (two a
-//      thread; 256 threads of four points took 1.3 times as long), folding each into the others, while the
-//      farthest of them comes before every block's bound in that order: no
-//      unpublished point can then come before it, so it is the farthest of all
-//      points.  FP32 decides a choice unless two distances, or one and the
-//      bound, lie within its margin.
+//      thread; 256 threads of four points took 1.3 times as long), folding each
+//      into the others, while the farthest of them comes before every block's
+//      bound in that order: no unpublished point can then come before it, so it
+//      is the farthest of all points.  FP32 decides a choice unless two
+//      distances, or one and the bound, lie within its margin.
 // The first choice of a round always passes, so a round adds one centre at
 // least; holes of the covering are many once some tens of centres stand, and a
 // round adds up to kFpsNew.
