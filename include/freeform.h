@@ -250,10 +250,10 @@ ff_status eigenmodes(ff_ctx* ctx, int k, const ff_eig_opts* opts, const void* X0
  * Many objects in one call: for every item, rkpm_build + assemble_hessian +
  * eigenmodes exactly as the single-object calls do them (same kernels, same
  * arithmetic, so each item's results equal those of the three calls on their
- * own).  `workers` host threads (0: min(count, 4)) each drive their own
- * context on their own non-blocking CUDA stream of `device`, taking the
- * objects largest first from a shared counter, so the latency-bound solves of
- * several objects overlap on the GPU.  The call synchronises the device before
+ * own).  `workers` host threads (0: one an object up to six objects, else four)
+ * each drive their own context on their own non-blocking CUDA stream of
+ * `device`, taking the objects largest first from a shared counter, so the
+ * latency-bound solves of several objects overlap on the GPU.  The call synchronises the device before
  * it starts (the inputs must be ready on any stream) and returns when every
  * item is done.
  *

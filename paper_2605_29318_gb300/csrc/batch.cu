@@ -42,11 +42,14 @@ ff_status eigenmodes_batched(int device, int precision, ff_batch_item* items, in
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(),
                    [&](int a, int b) { return items[a].n > items[b].n; });
-  // Four by default: past that the host threads wait for one another in the
-  // driver's launch path (~2,500 launches an object).  2, 4, 6 and 8 workers: 206,
-  // 171, 189 and 203 ms for 8 objects of 2,000-20,000 particles; 531, 409, 434 and
-  // 457 ms for 24; 1463, 1350, 1356 and 1386 ms for 16 of 2,000-200,000.
-  const int nw = std::min(count, workers > 0 ? workers : 4);
+  // By default one thread an object up to six objects, else four: past four the host
+  // threads wait for one another in the driver's launch path (~2,000 launches an
+  // object), but with five or six objects that costs less than a second turn.  Of
+  // 2,000-20,000 particles, 3, 4, 5, 6 and 8 threads: 5 objects 119, 126 and 111 ms;
+  // 6 objects 130, 134, 138 and 127; 7 objects 158, 143, 148 and 162; 8 objects 181,
+  // 194, 179, 190 and 199 (168, 166, 167, 170 and 191 another seed); 12 objects 240,
+  // 237, 238, 236 and 259.
+  const int nw = std::min(count, workers > 0 ? workers : count <= 6 ? 6 : 4);
   std::atomic<int> next{0};
   auto work = [&]() {
     if (cudaSetDevice(device) != cudaSuccess) {
