@@ -253,9 +253,9 @@ ff_status eigenmodes(ff_ctx* ctx, int k, const ff_eig_opts* opts, const void* X0
  * own).  `workers` host threads (0: one an object up to six objects, else four)
  * each drive their own context on their own non-blocking CUDA stream of
  * `device`, taking the objects largest first from a shared counter, so the
- * latency-bound solves of several objects overlap on the GPU.  The call synchronises the device before
- * it starts (the inputs must be ready on any stream) and returns when every
- * item is done.
+ * latency-bound solves of several objects overlap on the GPU.  The call
+ * synchronises the device before it starts (the inputs must be ready on any
+ * stream) and returns when every item is done.
  *
  *   device, precision  as for ff_create
  *   items     host array of count items; inputs as for rkpm_build and
