@@ -166,7 +166,8 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_wait2() { asm volatile("cp.async.wait_group 2;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+// every copy of the thread, those it has committed to no group among them
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, unsigned b0, unsigned b1) {
   asm volatile(
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(32 * WB, WB == 4 && NT <= 5 ? 8 : 1)
   cp_commit();
   if (s + kWB < ns) stage_step(1, u1);
   cp_commit();
-  {  // in the group of the third step
+  {  // in the group of the third step (in none where the warp has no k-step)
     const long long o = (long long)k0 * m;
     for (int q = threadIdx.x; q < nrow * (m / 4); q += 32 * kWB) {
       cp_async16(own_r + 4 * q, res + o + 4 * q);
@@ -311,8 +312,8 @@ __global__ void __launch_bounds__(32 * WB, WB == 4 && NT <= 5 ? 8 : 1)
     if (s >= ns) break;
     phase(2);
   }
-  cp_wait0();
-  __syncthreads();  // every warp is done with its staging buffers
+  cp_wait_all();
+  __syncthreads();  // every warp's copies are there, and it is done with its staging buffers
   float* red = reinterpret_cast<float*>(work);  // [kWB][16][P]
   const int g = lane >> 2, t = lane & 3;
 #pragma unroll
