@@ -261,13 +261,20 @@ struct TileDims {
 struct TileMax {
   int over, pts, cols, pairs, row;
 };
-constexpr TileDims kTileCap{512, 1536, 20480, 1536, 1024, 4096};
+// of a tile whose tables hold entries of tbytes: 1,200 columns are the most that eight
+// warps' double-float rows leave room for (1,536 would take 280,592 bytes)
+__host__ __device__ constexpr TileDims tile_cap(int tbytes) {
+  return tbytes == 8 ? TileDims{512, 1200, 20480, 1200, 1024, 4096}
+                     : TileDims{512, 1536, 20480, 1536, 1024, 4096};
+}
 
 // shared memory of a tile: what lasts (points, list entries, sorted columns),
 // then the column table, later the warps' rows
 struct TileSmem {
   int ptab, plist, poff, scols, pid, lr, ctab, cid, cols, warp, per_warp, loc, total;
-  __host__ __device__ TileSmem(const TileDims& d, int mode, int tbytes) {
+  __host__ __device__ constexpr TileSmem(const TileDims& d, int mode, int tbytes)
+      : ptab(0), plist(0), poff(0), scols(0), pid(0), lr(0), ctab(0), cid(0), cols(0), warp(0),
+        per_warp(0), loc(0), total(0) {
     int at = 0;
     auto take = [&](int bytes) {
       const int o = at;
@@ -297,6 +304,10 @@ struct TileSmem {
     if (total < tables) total = tables;
   }
 };
+// whatever the caps let through fits a block (227 KB, beside the kernel's own words)
+static_assert(TileSmem(tile_cap(4), 1, 4).total <= 227 * 1024 - 64 &&
+                  TileSmem(tile_cap(8), 1, 8).total <= 227 * 1024 - 64,
+              "a tile within the caps does not fit a block");
 
 template <int MODE, class T, class TO>
 __global__ void __launch_bounds__(kTileT, 2)
@@ -670,16 +681,17 @@ void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, doubl
   const long long* tpos = c->nbrT_pos.as<long long>();
   const float* vol = c->vol.as<float>();
   ProfScope ps_pattern(kProfPattern);
-  // nodal clouds in tiles of rows; a tile beyond kTileCap (wide supports, clouds
+  // nodal clouds in tiles of rows; a tile beyond tile_cap (wide supports, clouds
   // of very uneven density) sends the whole cloud to the row-owner passes below
   TileMax tmax{1, 0, 0, 0, 0};
   if (!c->twoset) {
     TileMax* dmax = reinterpret_cast<TileMax*>(c->scratch[6].ensure(sizeof(TileMax)));
     FF_CUDA(cudaMemsetAsync(dmax, 0, sizeof(TileMax), st));
-    const int smem = TileSmem(kTileCap, 0, 4).total;
+    const TileDims cap = tile_cap(tdf ? 8 : 4);
+    const int smem = TileSmem(cap, 0, 4).total;
     set_max_dyn_smem((const void*)k_tile_rows<0, float, float>, smem);
     (k_tile_rows<0, float, float><<<ceil_div(n, kTileRows), kTileT, smem, st>>>(
-         ptr, idx, tptr, tidx, tpos, nullptr, nullptr, n1, vol, nullptr, n, kTileCap, cnt, dmax,
+         ptr, idx, tptr, tidx, tpos, nullptr, nullptr, n1, vol, nullptr, n, cap, cnt, dmax,
          nullptr, nullptr, nullptr, nullptr, nullptr),
      ::ff::note_launch());
     FF_LAUNCH_CHECK();
