@@ -1045,11 +1045,11 @@ ff_status run_eigenmodes(ff_ctx* c, int k, const ff_eig_opts& o, const void* X0,
 
 template <class T>
 void spmm_hm(ff_ctx* c, const T* X, T* YH, T* YM, int ld, int m) {
-  // FP64 blocks of whole fours keep the summed form of their kernel, others the
-  // difference form they had in the general kernel; wide blocks go in the widest
-  // pieces the vector kernels take
-  const bool diff = sizeof(T) == 8 && m % 4 != 0;
-  const int piece = sizeof(T) == 4 || !diff ? 128 : 64;
+  // FP64 blocks of whole fours up to 128 columns take the summed form of their
+  // kernel, others the difference form, under which a constant column gives zero
+  // exactly; wide blocks go in the widest pieces the vector kernels take
+  const bool diff = sizeof(T) == 8 && (m % 4 != 0 || m > 128);
+  const int piece = diff ? 64 : 128;
   const int cols = ld > m ? ld : m;
   for (int c0 = 0; c0 < cols; c0 += piece)
     spmm_hm_raw<T>(c->stream, c->a_ptr.as<long long>(), c->a_col.as<int>(), c->a_val.as<T>(), c->n,
