@@ -122,9 +122,7 @@ __device__ __forceinline__ dfloat df_sqrt(dfloat a) {
 // n = nearest integer to x / ln 2, f = x - n ln 2 with ln 2 carried as a
 // double-float (|f| <= ln 2 / 2 up to rounding), then the Taylor polynomial of
 // e^f to degree 13 by Horner's rule (truncation below (ln2/2)^14 / 14! < 2e-17),
-// scaled by 2^n exactly.  The terms from f^8 / 8! (5.6e-9) on are summed in FP32,
-// whose rounding of them is 2^-51 of the result; the rest in double-float.
-// About 2^-45 relative: the error of n ln 2 dominates.
+// scaled by 2^n exactly.  About 2^-45 relative: the error of n ln 2 dominates.
 __device__ __forceinline__ dfloat df_exp(dfloat x) {
   const float n = rintf(__fmul_rn(x.h, 1.44269504f));
   const dfloat ln2(0.6931471805599453);
@@ -144,12 +142,9 @@ __device__ __forceinline__ dfloat df_exp(dfloat x) {
                                    1.0 / 39916800,
                                    1.0 / 479001600,
                                    1.0 / 6227020800.0};
-  float t = (float)kInvFact[13];
+  dfloat p(kInvFact[13]);
 #pragma unroll
-  for (int k = 12; k >= 8; --k) t = __fmaf_rn(t, f.h, (float)kInvFact[k]);
-  dfloat p(t);
-#pragma unroll
-  for (int k = 7; k >= 0; --k) p = df_add(df_mul(p, f), dfloat(kInvFact[k]));
+  for (int k = 12; k >= 0; --k) p = df_add(df_mul(p, f), dfloat(kInvFact[k]));
   const int e = (int)n;
   return dfloat(ldexpf(p.h, e), ldexpf(p.l, e));
 }
