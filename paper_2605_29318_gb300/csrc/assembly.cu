@@ -84,16 +84,22 @@ __global__ void k_material(const int* __restrict__ perm, long long n, const floa
   wh[j] = (T)((double)vol[j] * (lam + 4.0 * mu));
 }
 
+// rows to a tile (k_tile_rows below); wide (if given) holds a byte a tile, and the
+// row-owner passes take the rows of the tiles marked in it
+constexpr int kTileRows = 16;
+
 // pass 1: unique 2-hop columns per row
 __global__ void k_pattern_count(const long long* __restrict__ ptr, const int* __restrict__ idx,
                                 const long long* __restrict__ tptr, const int* __restrict__ tidx,
                                 long long n, int tsize, int* __restrict__ cnt,
+                                const unsigned char* __restrict__ wide,
                                 DevFlags* __restrict__ flags) {
   extern __shared__ int sm_tab[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   int* tab = sm_tab + wib * tsize;
   const long long rows_per_grid = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long k = (long long)blockIdx.x * (blockDim.x >> 5) + wib; k < n; k += rows_per_grid) {
+    if (wide && !wide[k / kTileRows]) continue;
     for (int q = lane; q < tsize; q += 32) tab[q] = kEmpty;
     __syncwarp();
     int fresh_cnt = 0;
@@ -131,7 +137,7 @@ __global__ void k_assemble(const long long* __restrict__ ptr, const int* __restr
                            const T* __restrict__ wh, long long n, int tsize, int maxrow,
                            const long long* __restrict__ aptr, int* __restrict__ acol,
                            TO* __restrict__ aval, float* __restrict__ hf32,
-                           float* __restrict__ hdiag) {
+                           float* __restrict__ hdiag, const unsigned char* __restrict__ wide) {
   extern __shared__ unsigned char sm_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   // per-warp layout: tab[tsize], rnk[tsize], keys[maxrow], skeys[maxrow] (int),
@@ -149,6 +155,7 @@ __global__ void k_assemble(const long long* __restrict__ ptr, const int* __restr
   T* vm = vh + maxrow;
   const long long rows_per_grid = (long long)gridDim.x * wpb;
   for (long long k = (long long)blockIdx.x * wpb + wib; k < n; k += rows_per_grid) {
+    if (wide && !wide[k / kTileRows]) continue;
     for (int q = lane; q < tsize; q += 32) tab[q] = kEmpty;
     __syncwarp();
     for (long long a = tptr[k]; a < tptr[k + 1]; ++a) {
@@ -249,9 +256,13 @@ size_t assemble_smem_per_warp(int tsize, int maxrow, size_t tbytes) {
 // accumulators in shared memory, at two blocks an SM.  The row-owner pass took 1.81 +
 // 14.4 ms (count, values) for 200k particles in FP32, this 1.11 + 3.39 ms; in
 // double-float (50k) 0.48 + 4.07 ms, this 0.29 + 1.09 ms.
-// MODE 0 counts the rows' columns and reports the largest tile; MODE 1 writes
-// columns and values, its tables sized by that.
-constexpr int kTileRows = 16, kTileT = 256, kTileWarps = kTileT / 32;
+// MODE 0 counts the rows' columns, reports the largest tile and marks in `wide`
+// those beyond the capacities (a wide support, a dense spot), whose rows are left to
+// the row-owner passes; MODE 1 writes the other tiles' columns and values, its
+// tables sized by the report.  100,000 particles in FP32 with supports of 2.2, 2.4, 2.6
+// and 3.0 spacings, the whole call: 12.0, 17.7, 36.2 and 102.4 ms by the row-owner passes
+// alone, 3.6, 6.9, 29.0 and 102.1 so (at 3.0 all tiles are wide).
+constexpr int kTileT = 256, kTileWarps = kTileT / 32;
 
 struct TileDims {
   int pts, cols, pairs, row;  // capacities: points, columns and list entries of a
@@ -259,7 +270,8 @@ struct TileDims {
   int ptab, ctab;             // hash slots
 };
 struct TileMax {
-  int over, pts, cols, pairs, row;
+  int wide;                    // tiles beyond the capacities
+  int pts, cols, pairs, row;   // the most of the others
 };
 // of a tile whose tables hold entries of tbytes: 1,200 columns are the most that eight
 // warps' double-float rows leave room for (1,536 would take 280,592 bytes)
@@ -318,9 +330,10 @@ __global__ void __launch_bounds__(kTileT, 2)
                 const T* __restrict__ wh, long long n, TileDims dims, int* __restrict__ cnt,
                 TileMax* __restrict__ tmax, const long long* __restrict__ aptr,
                 int* __restrict__ acol, TO* __restrict__ aval, float* __restrict__ hf32,
-                float* __restrict__ hdiag) {
+                float* __restrict__ hdiag, unsigned char* __restrict__ wide) {
   constexpr unsigned kAll = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char sm_raw[];
+  if (MODE && wide[blockIdx.x]) return;
   __shared__ int s_np, s_nc, s_tot, s_over;
   const TileSmem L(dims, MODE, (int)sizeof(T));
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -421,10 +434,14 @@ __global__ void __launch_bounds__(kTileT, 2)
   const int nc = s_nc, tot = s_tot;
   over = over || s_over || nc > dims.cols;
   if (MODE == 0 && tid == 0) {
-    if (over) tmax->over = 1;
-    atomicMax(&tmax->pts, np);
-    atomicMax(&tmax->cols, nc);
-    atomicMax(&tmax->pairs, tot);
+    wide[blockIdx.x] = over;
+    if (over) {
+      atomicAdd(&tmax->wide, 1);
+    } else {
+      atomicMax(&tmax->pts, np);
+      atomicMax(&tmax->cols, nc);
+      atomicMax(&tmax->pairs, tot);
+    }
   }
   if (over) return;
   if (MODE) {  // the columns in order (bitonic): a number becomes a rank
@@ -681,36 +698,39 @@ void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, doubl
   const long long* tpos = c->nbrT_pos.as<long long>();
   const float* vol = c->vol.as<float>();
   ProfScope ps_pattern(kProfPattern);
-  // nodal clouds in tiles of rows; a tile beyond tile_cap (wide supports, clouds
-  // of very uneven density) sends the whole cloud to the row-owner passes below
-  TileMax tmax{1, 0, 0, 0, 0};
-  if (!c->twoset) {
-    TileMax* dmax = reinterpret_cast<TileMax*>(c->scratch[6].ensure(sizeof(TileMax)));
+  // nodal clouds in tiles of rows; the rows of tiles beyond tile_cap (wide supports,
+  // clouds of very uneven density) take the row-owner passes below
+  const int ntiles = c->twoset ? 0 : (int)ceil_div(n, kTileRows);
+  TileMax tmax{};
+  unsigned char* wide = nullptr;  // null: every row is the row-owner passes'
+  if (ntiles > 0) {
+    TileMax* dmax = reinterpret_cast<TileMax*>(c->scratch[6].ensure(sizeof(TileMax) + ntiles));
+    wide = reinterpret_cast<unsigned char*>(dmax + 1);
     FF_CUDA(cudaMemsetAsync(dmax, 0, sizeof(TileMax), st));
     const TileDims cap = tile_cap(tdf ? 8 : 4);
     const int smem = TileSmem(cap, 0, 4).total;
     set_max_dyn_smem((const void*)k_tile_rows<0, float, float>, smem);
-    (k_tile_rows<0, float, float><<<ceil_div(n, kTileRows), kTileT, smem, st>>>(
+    (k_tile_rows<0, float, float><<<ntiles, kTileT, smem, st>>>(
          ptr, idx, tptr, tidx, tpos, nullptr, nullptr, n1, vol, nullptr, n, cap, cnt, dmax,
-         nullptr, nullptr, nullptr, nullptr, nullptr),
+         nullptr, nullptr, nullptr, nullptr, nullptr, wide),
      ::ff::note_launch());
     FF_LAUNCH_CHECK();
     FF_CUDA(cudaMemcpyAsync(&tmax, dmax, sizeof(TileMax), cudaMemcpyDeviceToHost, st));
     f = read_flags(c);
     check_material(f);
   }
-  const bool tiles = !tmax.over;
+  const bool tiles = tmax.wide < ntiles, owners = tmax.wide > 0 || !wide;
   // row-owner pass 1: unique columns per row, in a table of 2048 slots per warp
   // (4 warps per block); clouds of uneven density (wide supports reaching into
   // dense regions) retry with 16384 slots per warp (2 warps per block)
-  for (int attempt = 0; !tiles && attempt < 2; ++attempt) {
+  for (int attempt = 0; owners && attempt < 2; ++attempt) {
     const int tsize1 = attempt == 0 ? 2048 : 16384;
     const int wpb1 = attempt == 0 ? 4 : 2;
     const size_t smem1 = sizeof(int) * tsize1 * wpb1;
     if (smem1 > 48 * 1024) set_max_dyn_smem((const void*)k_pattern_count, (int)smem1);
     if (attempt > 0) reset_flags(c);
     int grid1 = (int)std::min<long long>(ceil_div(n, wpb1), (long long)sm_count() * 16);
-    (k_pattern_count<<<grid1, 32 * wpb1, smem1, st>>>(ptr, idx, tptr, tidx, n, tsize1, cnt,
+    (k_pattern_count<<<grid1, 32 * wpb1, smem1, st>>>(ptr, idx, tptr, tidx, n, tsize1, cnt, wide,
                                                      c->flags.as<DevFlags>()),
      ::ff::note_launch());
     FF_LAUNCH_CHECK();
@@ -751,12 +771,13 @@ void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, doubl
                        slots(tmax.pts), slots(tmax.cols)};
       const int smem = TileSmem(d, 1, (int)sizeof(TT)).total;
       set_max_dyn_smem((const void*)k_tile_rows<1, TT, TO>, smem);
-      (k_tile_rows<1, TT, TO><<<ceil_div(n, kTileRows), kTileT, smem, st>>>(
+      (k_tile_rows<1, TT, TO><<<ntiles, kTileT, smem, st>>>(
            ptr, idx, tptr, tidx, tpos, phi, dphi, n1, vol, wh, n, d, nullptr, nullptr, aptr, acol,
-           aval, hf32, hdiag),
+           aval, hf32, hdiag, wide),
        ::ff::note_launch());
-      return;
+      FF_LAUNCH_CHECK();
     }
+    if (!owners) return;
     const int maxrow = std::max(f.max_row, 1);
     int tsize2 = 64;
     while (tsize2 < 2 * maxrow) tsize2 <<= 1;
@@ -767,7 +788,7 @@ void build_matrices(ff_ctx* c, const float* E, const float* nu, double E0, doubl
     set_max_dyn_smem((const void*)k_assemble<TT, TO>, (int)std::max<size_t>(smem, 48 * 1024));
     (k_assemble<TT, TO><<<grid2, 32 * wpb2, smem, st>>>(ptr, idx, tptr, tidx, tpos, phi, dphi, n1,
                                                        vol, wh, n, tsize2, maxrow, aptr, acol,
-                                                       aval, hf32, hdiag),
+                                                       aval, hf32, hdiag, wide),
      ::ff::note_launch());
   };
   if (f64 && !tdf)  // FP32 tables and sums, FP64 storage
