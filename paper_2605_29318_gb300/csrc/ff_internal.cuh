@@ -274,6 +274,18 @@ long long twoset_cover(ff_ctx* c, const float* Q, long long nq, Buf& ptrb, Buf& 
 void twoset_shape(ff_ctx* c, const float* Q, long long nq, const long long* ptr, const int* idx,
                   long long n1, void* phi, void* dphi, bool f32);
 
+// What one pass found, kept for the next in scratch: more than kKeptScratch goes back
+// to the device once that has run, so that a call on many points does not hold it for
+// the life of the context.  Giving back and taking anew costs such a call 0.4 ms: 1.2
+// million points in FP32 14.7 and 15.1 ms so on 2,000 particles (16.9 searching twice),
+// 3.03 and 3.50 ms on 3,000 centres.
+constexpr size_t kKeptScratch = 256ull << 20;
+inline void give_back(ff_ctx* c, Buf& b, size_t room) {
+  if (room <= kKeptScratch) return;
+  FF_CUDA(cudaStreamSynchronize(c->stream));
+  b.release();
+}
+
 // skinning weight fields and linear blend skinning at query points (skinning.cu)
 void skinning_weights(ff_ctx* c, const float* Q, long long nq, const void* C, int m, void* W);
 void lbs_deform(ff_ctx* c, const float* Q, long long nq, const void* W, int m, const void* Z,

@@ -438,8 +438,8 @@ void weights_t(ff_ctx* c, const float* Q, long long nq, const T* C, int m, T* W)
                      g.bdims[0], g.bdims[1], g.bdims[2]};
     int* cnt = reinterpret_cast<int*>(c->sk_cnt.ensure(sizeof(int) * (nq + 1)));
     long long* ptr = reinterpret_cast<long long*>(c->sk_ptr.ensure(sizeof(long long) * (nq + 1)));
-    // the hits kept between the passes while they are small; without them the
-    // second pass searches again
+    // the hits kept between the passes while they are small (2.8 million points; more
+    // than kKeptScratch is given back); without them the second pass searches again
     unsigned* masks = nullptr;
     const size_t room = sizeof(unsigned) * 32 * kMaskRounds * (size_t)nq;
     if (room <= (1ull << 30)) {
@@ -460,6 +460,7 @@ void weights_t(ff_ctx* c, const float* Q, long long nq, const T* C, int m, T* W)
          Q, nq, c->pos.as<float4>(), gd, c->cell_start.as<int>(), nullptr, masks, ptr, idx),
      ::ff::note_launch());
     FF_LAUNCH_CHECK();
+    if (masks) give_back(c, c->scratch[6], room);
     qptr = ptr;
     qidx = idx;
     phi = reinterpret_cast<S*>(c->sk_phi.ensure(sizeof(S) * std::max(nq1, 1LL)));

@@ -906,7 +906,7 @@ long long twoset_cover(ff_ctx* c, const float* Q, long long nq, Buf& ptrb, Buf& 
   int* cnt = reinterpret_cast<int*>(cntb.ensure(sizeof(int) * (nq + 1)));
   // as bits between the two passes while they take less room than the lists
   // (K / 8 bytes a point against 4 a pair, ~100 pairs) and 1 GB at most; else, or
-  // without that room, the tests run twice
+  // without that room, the tests run twice.  More than kKeptScratch is given back
   const int words = (K + 31) / 32;
   const size_t room = sizeof(unsigned) * (size_t)words * nq;
   unsigned* bits = nullptr;
@@ -941,6 +941,7 @@ long long twoset_cover(ff_ctx* c, const float* Q, long long nq, Buf& ptrb, Buf& 
          idx),
      ::ff::note_launch());
   FF_LAUNCH_CHECK();
+  if (bits) give_back(c, c->scratch[6], room);
   return n1;
 }
 
