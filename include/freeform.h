@@ -248,10 +248,11 @@ ff_status eigenmodes(ff_ctx* ctx, int k, const ff_eig_opts* opts, const void* X0
 
 /* ---------------------------------------------------------- eigenmodes_batched
  * Many objects in one call: for every item, rkpm_build + assemble_hessian +
- * eigenmodes exactly as the single-object calls do them (same kernels, same
- * arithmetic, so each item's results equal those of the three calls on their
- * own).  `workers` host threads (0: one an object up to six objects, else four)
- * each drive their own context on their own non-blocking CUDA stream of
+ * eigenmodes as the single-object calls do them (the same arithmetic in the same
+ * order, so each item's results equal those of the three calls on their own;
+ * where an object alone may take the preconditioner's steps in one launch, a
+ * batch takes them one by one).  `workers` host threads (0: four, or five for
+ * five objects) each drive their own context on their own non-blocking CUDA stream of
  * `device`, taking the objects largest first from a shared counter, so the
  * latency-bound solves of several objects overlap on the GPU.  The call
  * synchronises the device before it starts (the inputs must be ready on any

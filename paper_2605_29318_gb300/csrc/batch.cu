@@ -3,8 +3,10 @@
 // largest first from a shared counter and runs the single-object calls on
 // them.  One object's solve is a chain of small latency-bound launches with a
 // host read-back per iteration, so a single object leaves most SMs idle;
-// several objects in flight on separate streams fill them.  Each item runs the
-// same kernels as alone, so its results do not depend on the batch.
+// several objects in flight on separate streams fill them.  Each item takes the
+// same sums in the same order as alone, so its results do not depend on the batch
+// (the preconditioner's polynomial goes step by step where an object alone may take
+// it in one launch, cheb_poly_tc).
 #include <algorithm>
 #include <atomic>
 #include <cstring>
@@ -42,14 +44,18 @@ ff_status eigenmodes_batched(int device, int precision, ff_batch_item* items, in
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(),
                    [&](int a, int b) { return items[a].n > items[b].n; });
-  // By default one thread an object up to six objects, else four: past four the host
+  // By default four threads, or one an object where there are five: past four the host
   // threads wait for one another in the driver's launch path (~2,000 launches an
-  // object), but with five or six objects that costs less than a second turn.  Of
-  // 2,000-20,000 particles, 3, 4, 5, 6 and 8 threads: 5 objects 119, 126 and 111 ms;
-  // 6 objects 130, 134, 138 and 127; 7 objects 158, 143, 148 and 162; 8 objects 181,
-  // 194, 179, 190 and 199 (168, 166, 167, 170 and 191 another seed); 12 objects 240,
-  // 237, 238, 236 and 259.
-  const int nw = std::min(count, workers > 0 ? workers : count <= 6 ? 6 : 4);
+  // object), which with five objects costs less than a second turn.  Medians, the mean of
+  // three draws of objects of 2,000-20,000 particles, with 3, 4, 5, 6 and 8 threads:
+  //    4 objects  108   93 ms               8 objects  173  179  175  185  200 ms
+  //    5 objects  114  122  108            10 objects  216  211  204  217  232
+  //    6 objects  141  141  146  144       12 objects  240  236  241  238  261
+  //    7 objects  165  153  162  168       16 objects  325  303  309  313  323
+  // (draws differ by 10 %; 8 objects are a tie of three to five).  One draw of 48 and of 96:
+  // 695, 654, 660, 701, 718 and 1339, 1218, 1196, 1215, 1301; of 48 up to 200,000 particles
+  // 2986, 2928, 2956, 2979, 3025.
+  const int nw = std::min(count, workers > 0 ? workers : count == 5 ? 5 : 4);
   std::atomic<int> next{0};
   auto work = [&]() {
     if (cudaSetDevice(device) != cudaSuccess) {
