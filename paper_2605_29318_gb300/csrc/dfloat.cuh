@@ -61,6 +61,18 @@ __device__ __forceinline__ dfloat df_add(dfloat a, dfloat b) {
   return r;
 }
 
+// the same with the tails' sum exact too (Shewchuk 1997): no digits lost where the
+// heads cancel
+__device__ __forceinline__ dfloat df_add2(dfloat a, dfloat b) {
+  float s, e, t, f, h, l;
+  two_sum(a.h, b.h, s, e);
+  two_sum(a.l, b.l, t, f);
+  fast_two_sum(s, __fadd_rn(e, t), h, l);
+  dfloat r;
+  fast_two_sum(h, __fadd_rn(l, f), r.h, r.l);
+  return r;
+}
+
 __device__ __forceinline__ dfloat df_mul(dfloat a, dfloat b) {
   const float p = __fmul_rn(a.h, b.h);
   float e = __fmaf_rn(a.h, b.h, -p);
@@ -105,6 +117,20 @@ __device__ __forceinline__ dfloat df_div(dfloat a, dfloat b) {
   dfloat q;
   fast_two_sum(q1, q2, q.h, q.l);
   return df_add(q, dfloat(q3));
+}
+
+// a / b as df_div, its quotients products with r = 1 / b.h: for several divisions by
+// one b (each quotient's rounding is corrected by the next remainder all the same)
+__device__ __forceinline__ dfloat df_div_by(dfloat a, dfloat b, float r) {
+  const float q1 = __fmul_rn(a.h, r);
+  const dfloat b1 = df_mul(b, dfloat(q1));
+  dfloat e = df_add(a, dfloat(-b1.h, -b1.l));
+  const float q2 = __fmul_rn(e.h, r);
+  const dfloat b2 = df_mul(b, dfloat(q2));
+  e = df_add(e, dfloat(-b2.h, -b2.l));
+  dfloat q;
+  fast_two_sum(q1, q2, q.h, q.l);
+  return df_add(q, dfloat(__fmul_rn(e.h, r)));
 }
 
 // sqrt(a), a >= 0: the FP32 root y of the head, then y + (a - y^2) / (2 y)

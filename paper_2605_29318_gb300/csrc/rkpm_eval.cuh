@@ -12,19 +12,38 @@
 namespace ff {
 namespace rkpm {
 
+// w(q) and w'(q) / q of the cubic B-spline, from q^2: its root has half the square's
+// relative error, and the inner piece takes the square itself
 template <class C>
-__device__ __forceinline__ void bspline(C q, C& w, C& dwq) {
+__device__ __forceinline__ void bspline(C q2, C& w, C& dwq) {
+  const C q = sqrt(q2);
   if (q <= C(0.5)) {
-    w = C(2.0 / 3.0) - C(4) * q * q + C(4) * q * q * q;
+    w = C(2.0 / 3.0) - C(4) * (q2 * (C(1) - q));
     dwq = C(-8) + C(12) * q;
   } else if (q <= C(1)) {
-    C t = C(1) - q;
-    w = C(4.0 / 3.0) * t * t * t;
-    dwq = C(-4) * t * t / q;
+    const C t = C(1) - q, t2 = t * t;
+    w = C(4.0 / 3.0) * t * t2;
+    dwq = C(-4) * t2 / q;
   } else {
     w = C(0);
     dwq = C(0);
   }
+}
+
+// a + b where the terms may cancel
+template <class C>
+__device__ __forceinline__ C sum2(C a, C b) {
+  if constexpr (std::is_same_v<C, dfloat>)
+    return df_add2(a, b);
+  else
+    return a + b;
+}
+
+// normalises an accumulator of mac between two terms: the tail of a dozen unnormalised
+// terms grows, and with it the rounding of its own sum
+template <class C>
+__device__ __forceinline__ void settle(C& a) {
+  if constexpr (std::is_same_v<C, dfloat>) fast_two_sum(a.h, a.l, a.h, a.l);
 }
 
 // Raw kernels varphi_k as functors: from the squared distance d2 = |X - p_k|^2
@@ -34,10 +53,10 @@ struct BSpline {
   static constexpr bool kStash = false;
   template <class C>
   __device__ __forceinline__ void eval(int, float4 p, C d2, C& w, C& gs) const {
-    const C ak = (C)p.w;
+    const C ak = (C)p.w, ak2 = ak * ak;
     C dwq;
-    bspline<C>(sqrt(d2) / ak, w, dwq);
-    gs = -dwq / (ak * ak);
+    bspline<C>(d2 / ak2, w, dwq);
+    gs = -dwq / ak2;
   }
 };
 
@@ -94,12 +113,38 @@ __device__ __forceinline__ constexpr int sidx(int r, int c) {
   return lo * 4 - lo * (lo - 1) / 2 + (hi - lo);
 }
 
-// Cholesky factor of a 4x4 SPD matrix: the strict lower triangle and the
-// diagonal's reciprocals, so that a solve has no divisions.
+// A divisor d with its reciprocal r, rounded once: t / d as t r corrected by the
+// remainder, as good as a division.  (t r by itself is a rounding more, which M's
+// condition number amplifies: 7 to 12 % on a row's largest error, in FP32 and in
+// double-float.)
+template <class C>
+struct Divisor {
+  C d, r;
+  __device__ __forceinline__ void set(C x) {
+    d = x;
+    r = C(1) / x;
+  }
+  __device__ __forceinline__ C into(C t) const {
+    const C q = t * r;
+    return fma(fma(-q, d, t), r, q);
+  }
+};
+template <>
+struct Divisor<dfloat> {
+  dfloat d;
+  float r;
+  __device__ __forceinline__ void set(dfloat x) {
+    d = x;
+    r = __fdiv_rn(1.f, x.h);
+  }
+  __device__ __forceinline__ dfloat into(dfloat t) const { return df_div_by(t, d, r); }
+};
+
+// Cholesky factor of a 4x4 SPD matrix: the strict lower triangle and the diagonal
 template <class C>
 struct Chol4 {
   C l[4][4];
-  C r[4];
+  Divisor<C> piv[4];
   // false if a pivot is not positive relative to the trace
   __device__ __forceinline__ bool factor(const C* m, C rel_tol) {
     const C tr = m[0] + m[4] + m[7] + m[9];
@@ -110,13 +155,13 @@ struct Chol4 {
 #pragma unroll
       for (int p = 0; p < j; ++p) s -= l[j][p] * l[j][p];
       ok = ok && s > rel_tol * tr;
-      r[j] = C(1) / sqrt(s);
+      piv[j].set(sqrt(s));
 #pragma unroll
       for (int i = j + 1; i < 4; ++i) {
         C t = m[sidx(i, j)];
 #pragma unroll
         for (int p = 0; p < j; ++p) t -= l[i][p] * l[j][p];
-        l[i][j] = t * r[j];
+        l[i][j] = piv[j].into(t);
       }
     }
     return ok;
@@ -128,14 +173,14 @@ struct Chol4 {
       C t = b[i];
 #pragma unroll
       for (int p = 0; p < i; ++p) t -= l[i][p] * y[p];
-      y[i] = t * r[i];
+      y[i] = piv[i].into(t);
     }
 #pragma unroll
     for (int i = 3; i >= 0; --i) {
       C t = y[i];
 #pragma unroll
       for (int p = i + 1; p < 4; ++p) t -= l[p][i] * x[p];
-      x[i] = t * r[i];
+      x[i] = piv[i].into(t);
     }
   }
 };
@@ -144,7 +189,7 @@ struct Chol4 {
 // outputs of precision T (phi; with GRAD dphi too).  Every lane of the warp
 // takes part (a group without a row passes s == e).  Returns 0 ok, 1 singular,
 // 2 ill-conditioned (only when check_cond), the same in every lane of a group;
-// nothing is written then.
+// no values are written then (where kernels are stashed, phi holds those).
 //
 // The row's pairs cost ~110 (values alone: ~50) instructions an entry of a
 // lane, the moment solve ~900 a warp whatever the rows it holds; so a warp
@@ -184,9 +229,13 @@ __device__ __forceinline__ int shape_rows(const float4* __restrict__ pos, long l
 #pragma unroll
       for (int b = a; b < 4; ++b, ++o) {
         const C pp = P[a] * P[b];
-        mac(m[o], w, pp);  // fused (unnormalised in double-float), finished below
+        mac(m[o], w, pp);  // fused, finished below
+        settle(m[o]);
 #pragma unroll
-        for (int d = 0; d < ND; ++d) mac(dm[d][o], g[d], pp);
+        for (int d = 0; d < ND; ++d) {
+          mac(dm[d][o], g[d], pp);
+          settle(dm[d][o]);
+        }
       }
   }
 #pragma unroll
@@ -233,10 +282,10 @@ __device__ __forceinline__ int shape_rows(const float4* __restrict__ pos, long l
     for (int r = 0; r < 4; ++r) {
       C t = C(0);
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) t += dm[d][sidx(r, cc)] * Cv[cc];
+      for (int cc = 0; cc < 4; ++cc) t = sum2(t, dm[d][sidx(r, cc)] * Cv[cc]);
       rhs[r] = -t;
     }
-    rhs[1 + d] += isi;
+    rhs[1 + d] = sum2(rhs[1 + d], isi);
     ch.solve(rhs, dC[d]);
   }
   for (long long t = s + lane; t < e; t += L) {
@@ -263,7 +312,7 @@ __device__ __forceinline__ int shape_rows(const float4* __restrict__ pos, long l
 #pragma unroll
       for (int a = 1; a < 4; ++a) mac(PdC, P[a], dC[d][a]);
       PdC = finish(PdC);
-      dphi[d * n1 + t] = (T)(g[d] * PC + w * PdC);
+      dphi[d * n1 + t] = (T)sum2(g[d] * PC, w * PdC);
     }
   }
   return 0;

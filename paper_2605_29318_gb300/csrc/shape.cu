@@ -27,8 +27,9 @@ using rkpm::shape_rows;
 
 // lanes a row: a nodal row has ~30-45 nodes, so eight lanes take four to six
 // of them each and a warp's moment solve serves four rows (FP32, 200k
-// particles: 1.41 ms with a warp a row, 0.15 ms and 0.16 ms of FP64 redo now;
-// double-float, 50k particles: 1.34 ms, 0.37 ms now)
+// particles: 1.41 ms with a warp a row, 0.37 ms now with the FP64 redo; double-float,
+// 50k particles: 1.33 ms, 0.51 ms now, of which 0.15 for sums and quotients as exact
+// as a warp a row has them)
 constexpr int kLanes = 8;
 
 template <class T>

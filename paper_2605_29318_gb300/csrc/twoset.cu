@@ -849,8 +849,9 @@ __global__ void k_centre_inv(const double* __restrict__ rad, int K, float4* __re
 // lanes a row: a point has ~100 covering centres, so eight lanes take a dozen
 // each and a warp's moment solve serves four points.  FP32, 1M points of 98
 // centres: 3.17 ms with a warp a point, 1.61 ms in its
-// order of operations (0.95 ms in a free one; values alone 0.51 ms);
-// double-float, 228k points: 5.73 ms, 2.09 ms now.
+// order of operations (0.95 ms in a free one; values alone 0.6 ms); double-float,
+// 228k points: 5.79 ms, 2.91 ms now, of which 0.73 for sums and quotients as exact
+// as a warp a point has them.
 constexpr int kShapeLanes = 8;
 
 template <class T, bool GRAD>
