@@ -190,10 +190,10 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, unsigned
 // own rows of res, x and d therefore come with the third step's group and are
 // finished as the contiguous run they are, 64 registers let eight blocks share an
 // SM, and a step's kernel starts while the one before drains, reading its tables
-// before it waits for that one's vectors.  50,000 rows, 40 columns: 31.7 us a step
-// without these, 27.2 so, and 3 us less between steps.  Gathers that keep lines in
-// L1 (29.5 us), and two (30.8) or four (33.1) row blocks in a block to share them,
-// were slower.
+// before it waits for that one's vectors.  50,000 rows, 40 columns, launch lists (cold,
+// serialised): 28.2 us a step without these, 23.3 so, and about 3 us less between steps.
+// Slower, in a timing where this form took 27.2 us and the one before 31.7: gathers that
+// keep lines in L1 (29.5), two (30.8) or four (33.1) row blocks in a block to share them.
 __host__ __device__ constexpr size_t tc_rows_bytes(int NT) { return (size_t)kTcRows * (8 * NT * 10 + 8); }
 __host__ __device__ constexpr int tc_red_ld(int NT) { return 8 * NT + (NT % 2 ? 0 : 8); }  // conflict-free for 8 rows
 
