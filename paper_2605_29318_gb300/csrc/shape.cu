@@ -16,6 +16,8 @@
 // matrix has a 1-norm condition number above `cond_limit` is recomputed entirely
 // in FP64 by a second kernel.  FP64 mode computes
 // and stores double-float pairs (FP32 head and tail, ~2^-47 relative).
+#include <type_traits>
+
 #include "dfloat.cuh"
 #include "ff_internal.cuh"
 #include "rkpm_eval.cuh"
@@ -29,32 +31,42 @@ using rkpm::shape_rows;
 // of them each and a warp's moment solve serves four rows (FP32, 200k
 // particles: 1.41 ms with a warp a row, 0.37 ms now with the FP64 redo; double-float,
 // 50k particles: 1.33 ms, 0.51 ms now, of which 0.15 for sums and quotients as exact
-// as a warp a row has them)
+// as a warp a row has them).  Few rows take a warp each, and an ill-conditioned FP32 row
+// its FP64 redo at once: their time is one row's chain of operations, which is shorter so.
+// With eight lanes and with a warp: FP32 300 particles 75 and 41 us, 8,000 75 and 58, 12,000
+// 83 and 76 (no second launch); double-float 1,000 44 and 32 us, 2,432 (the warps that are
+// resident) 48 both, 2,600 47 and 65.
 constexpr int kLanes = 8;
 
-template <class T>
+template <class T, int L>
 __global__ void __launch_bounds__(256, 2)
     k_shape(const float4* __restrict__ pos, const long long* __restrict__ ptr,
             const int* __restrict__ idx, long long n, long long n1, T* __restrict__ phi,
             T* __restrict__ dphi, double cond_limit, int* __restrict__ redo,
             DevFlags* __restrict__ flags) {
-  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
-  const bool live = i < n, first = threadIdx.x % kLanes == 0;
+  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / L;
+  const bool live = i < n, first = threadIdx.x % L == 0;
   const long long s = live ? ptr[i] : 0, e = live ? ptr[i + 1] : 0;
   const float4 Xi = live ? pos[i] : make_float4(0.f, 0.f, 0.f, 1.f);
+  int st;
   if constexpr (sizeof(T) == 4) {
-    const int st =
-        shape_rows<float, T, kLanes, true>(pos, s, e, idx, Xi, phi, dphi, n1, cond_limit, true);
-    if (live && st != 0 && first) rkpm::redo_later(redo, i);
+    st = shape_rows<float, T, L, true>(pos, s, e, idx, Xi, phi, dphi, n1, cond_limit, true);
+    if constexpr (L == 32) {
+      if (live && st != 0) {
+        st = shape_rows<double, T, L, true>(pos, s, e, idx, Xi, phi, dphi, n1, 0.0, false);
+        if (st == 0 && first) atomicAdd(&flags->fallback, 1);
+      }
+    } else {
+      if (live && st != 0 && first) rkpm::redo_later(redo, i);
+      return;
+    }
   } else {
     // FP64 outputs computed in double-float (~2^-47 relative; GB300's FP64
     // rate made this kernel FP64-bound)
-    const int st = shape_rows<dfloat, T, kLanes, true>(pos, s, e, idx, Xi, phi, dphi, n1, 0.0,
-                                                       false);
-    if (live && st != 0 && first &&
-        atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0)
-      flags->index = (int)i;
+    st = shape_rows<dfloat, T, L, true>(pos, s, e, idx, Xi, phi, dphi, n1, 0.0, false);
   }
+  if (live && st != 0 && first && atomicCAS(&flags->code, 0, (int)FF_ERR_SINGULAR_MOMENT) == 0)
+    flags->index = (int)i;
 }
 
 }  // namespace
@@ -72,16 +84,26 @@ void build_shape(ff_ctx* c) {
   const long long* ptr = c->nbr_ptr.as<long long>();
   const int* idx = c->nbr_idx.as<int>();
   DevFlags* flags = c->flags.as<DevFlags>();
-  const unsigned grid = ceil_div(n * kLanes, T);
-  if (c->prec == FF_PREC_FP64) {  // stored as double-float pairs for the assembly
-    (k_shape<dfloat><<<grid, T, 0, c->stream>>>(pos, ptr, idx, n, n1, c->phi.as<dfloat>(),
-                                                c->dphi.as<dfloat>(), cond_limit, nullptr, flags),
+  const bool few = n <= (c->prec == FF_PREC_FP64 ? 16 : 64) * (long long)sm_count();
+  const unsigned grid = ceil_div(n * (few ? 32 : kLanes), T);
+  auto run = [&](auto tag, auto lanes, int* redo) {
+    using S = decltype(tag);
+    (k_shape<S, decltype(lanes)::value><<<grid, T, 0, c->stream>>>(
+         pos, ptr, idx, n, n1, c->phi.as<S>(), c->dphi.as<S>(), cond_limit, redo, flags),
      ::ff::note_launch());
+  };
+  using Warp = std::integral_constant<int, 32>;
+  using Part = std::integral_constant<int, kLanes>;
+  if (c->prec == FF_PREC_FP64) {  // stored as double-float pairs for the assembly
+    if (few)
+      run(dfloat{}, Warp{}, nullptr);
+    else
+      run(dfloat{}, Part{}, nullptr);
+  } else if (few) {
+    run(float{}, Warp{}, nullptr);
   } else {
     int* redo = rkpm::redo_list(c, n);
-    (k_shape<float><<<grid, T, 0, c->stream>>>(pos, ptr, idx, n, n1, c->phi.as<float>(),
-                                               c->dphi.as<float>(), cond_limit, redo, flags),
-     ::ff::note_launch());
+    run(float{}, Part{}, redo);
     FF_LAUNCH_CHECK();
     (rkpm::k_shape_redo<float, true, rkpm::BSpline><<<rkpm::redo_grid(n), 256, 0, c->stream>>>(
          pos, pos, nullptr, 0.f, ptr, idx, n1, c->phi.as<float>(), c->dphi.as<float>(), redo,
