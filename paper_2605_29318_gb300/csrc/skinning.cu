@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(TB, 1024 / (TB * PTS))
                 fma(z[4 * d + 1], X[p][1], fma(z[4 * d], X[p][0], z[4 * d + 3]))));
     };
     int j = 0;
-    if constexpr (READ == kCopy || READ == kLoad)
+    if constexpr (READ == kCopy || READ == kLoad) {
       for (; j + E <= jn; j += E) {
         T wv[PTS][E];
 #pragma unroll
@@ -337,6 +337,11 @@ __global__ void __launch_bounds__(TB, 1024 / (TB * PTS))
 #pragma unroll
           for (int p = 0; p < PTS; ++p) add(p, wv[p][u], sz[j + u]);
       }
+    }
+    // (unrolled, the few modes of kDirect all run in the remainder: two modes in FP64 took
+    // 95 us for 1M points, 71 so)
+    constexpr int kModes = READ == kDirect ? 1 : 4;
+#pragma unroll kModes
     for (; j < jn; ++j)
 #pragma unroll
       for (int p = 0; p < PTS; ++p) {
