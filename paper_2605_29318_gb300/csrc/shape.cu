@@ -14,7 +14,7 @@
 // lane of the group the sums; each then solves the 4x4 system (Cholesky) and
 // writes phi / grad phi for its own neighbours.  In FP32 mode a row whose moment
 // matrix has a 1-norm condition number above `cond_limit` is recomputed entirely
-// in FP64 by a second kernel.  FP64 mode computes
+// in FP64 (by a second kernel, or in place where rows are few).  FP64 mode computes
 // and stores double-float pairs (FP32 head and tail, ~2^-47 relative).
 #include <type_traits>
 
